@@ -492,6 +492,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
     panel_off += int64_t(sn[s].ld) * S.sn_k[s];
     sn[s].uoff = S.sn_uoff[s];
     sn[s].frontoff = S.sn_frontoff[s];
+    sn[s].eoff = 0;
     F.maxk = std::max(F.maxk, S.sn_k[s]);
     F.maxm = std::max(F.maxm, S.sn_m[s]);
   }
@@ -530,11 +531,28 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
     }
     F.solve_panel_elems = off;
     F.snlev = ST.nlev;
+    if (precision == 0) {                            // digits of the solve panels: one exponent per row
+      int64_t rows = 0;
+      for (hz::SnDev& d : ssn) {
+        d.eoff = rows;
+        rows += d.m;
+      }
+      TRY(dalloc(c, &F.rexp, std::max<int64_t>(rows, 1)));
+    }
     TRY(upload(c, &F.ssn, ssn));
   }
   TRY(upload(c, &F.rowlist, S.rowlist));
-  TRY(upload(c, &F.cptr, S.cptr));
-  TRY(upload(c, &F.cidx, S.cidx));
+  {
+    // update vectors are stored in the order in which the parents' rows read them (a parent row's
+    // child contributions are adjacent): u index of row slot r, child rank q = cptr[r] + q, and
+    // wpos gives the index that each update row writes
+    if (S.cptr.back() >= int64_t(1) << 32 || S.u_elems >= int64_t(1) << 32)
+      return fail(c, HZ_ERR_OOM, "more update rows than a device holds");
+    std::vector<uint32_t> p32(S.cptr.begin(), S.cptr.end()), w(size_t(S.u_elems), 0u);
+    for (size_t q = 0; q < S.cidx.size(); q++) w[size_t(S.cidx[q])] = uint32_t(q);
+    TRY(upload(c, &F.cptr, p32));
+    TRY(upload(c, &F.wpos, w));
+  }
   TRY(upload(c, &F.rel, S.rel));
   TRY(upload(c, &F.reloff, S.sn_reloff));
   TRY(upload(c, &F.gidx, S.gidx));
@@ -723,25 +741,43 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
   F.t_lev_sn = ST.lev_sn;
   F.t_sn_k = ST.k;
   F.t_sn_m = ST.m;
+  F.h_lev_k.assign(size_t(ST.nlev), 16);
+  F.h_lev_m.assign(size_t(ST.nlev), 0);
+  for (int l = 0; l < ST.nlev; l++)
+    for (int32_t q = ST.lev_ptr[size_t(l)]; q < ST.lev_ptr[size_t(l) + 1]; q++) {
+      const size_t ci = size_t(ST.lev_sn[size_t(q)]);
+      F.h_lev_k[size_t(l)] = std::max(F.h_lev_k[size_t(l)], (ST.k[ci] + 15) / 16 * 16);
+      F.h_lev_m[size_t(l)] = std::max(F.h_lev_m[size_t(l)], ST.m[ci]);
+    }
   TRY(build_sweep_tasks(c, F, sp));
   F.sweep_chunk = bwd_rows;
   F.sweep_scale = 1.0;
   // batched sweeps for nrhs_block right-hand sides (pseudo-block FGMRES)
   if (nrhs_block > 1) {
     F.mS = nrhs_block;
-    F.mbwd_rows = 128;
     std::vector<int2> mf;
     std::vector<int4> mb, mfin;
-    std::vector<int64_t> mf_ptr(nlev + 1), mb_ptr(nlev + 1);
+    std::vector<int64_t> mf_ptr(ST.nlev + 1), mb_ptr(ST.nlev + 1);
+    F.h_mfwd_rt.assign(size_t(ST.nlev), 64);
     int64_t max_mb = 0;
-    for (int l = 0; l < nlev; l++) {
+    for (int l = 0; l < ST.nlev; l++) {
       mf_ptr[l] = int64_t(mf.size());
       mb_ptr[l] = int64_t(mb.size());
-      for (int32_t q = S.lev_ptr[l]; q < S.lev_ptr[l + 1]; q++) {
-        const int s = S.lev_sn[q];
-        const int k = S.sn_k[s], m = S.sn_m[s];
-        for (int rb = 0; rb * 64 < m; rb++) mf.push_back(make_int2(s, rb));
-        const int nch = (m + F.mbwd_rows - 1) / F.mbwd_rows;
+      if (precision == 0) {
+        // digit sweeps: 64-row tasks (32 with 16 right-hand sides: eight warps' worth of
+        // tiles); 16-row tasks on levels with fewer than two tasks per SM, as in plan_sweeps
+        const int wide = nrhs_block == 16 ? 32 : 64;
+        int64_t nf = 0;
+        for (int32_t q = ST.lev_ptr[size_t(l)]; q < ST.lev_ptr[size_t(l) + 1]; q++)
+          nf += (ST.m[size_t(ST.lev_sn[size_t(q)])] + wide - 1) / wide;
+        F.h_mfwd_rt[size_t(l)] = nf < 2 * 152 ? 16 : wide;
+      }
+      const int rt = F.h_mfwd_rt[size_t(l)];
+      for (int32_t q = ST.lev_ptr[size_t(l)]; q < ST.lev_ptr[size_t(l) + 1]; q++) {
+        const int s = ST.lev_sn[size_t(q)];
+        const int k = ST.k[size_t(s)], m = ST.m[size_t(s)];
+        for (int rb = 0; rb * rt < m; rb++) mf.push_back(make_int2(s, rb));
+        const int nch = (m + hz::kMultiBwdRows - 1) / hz::kMultiBwdRows;
         for (int cb = 0; cb * 32 < k; cb++) {
           const int fin = int(mfin.size());
           mfin.push_back(make_int4(s, cb, int(int64_t(mb.size()) - mb_ptr[l]), nch));
@@ -750,14 +786,14 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
       }
       max_mb = std::max(max_mb, int64_t(mb.size()) - mb_ptr[l]);
     }
-    mf_ptr[nlev] = int64_t(mf.size());
-    mb_ptr[nlev] = int64_t(mb.size());
+    mf_ptr[ST.nlev] = int64_t(mf.size());
+    mb_ptr[ST.nlev] = int64_t(mb.size());
     TRY(upload(c, &F.mfwd_tasks, mf));
     TRY(upload(c, &F.mbwd_tasks, mb));
     TRY(upload(c, &F.mbfin_tasks, mfin));
     TRY(upload(c, &F.mbwd_counters, std::vector<unsigned int>(std::max<size_t>(mfin.size(), 1), 0u)));
-    F.h_mfwd_ptr = new int64_t[nlev + 1];
-    F.h_mbwd_ptr = new int64_t[nlev + 1];
+    F.h_mfwd_ptr = new int64_t[mf_ptr.size()];
+    F.h_mbwd_ptr = new int64_t[mb_ptr.size()];
     std::copy(mf_ptr.begin(), mf_ptr.end(), F.h_mfwd_ptr);
     std::copy(mb_ptr.begin(), mb_ptr.end(), F.h_mbwd_ptr);
     const int64_t vsz = int64_t(vs) * nrhs_block;
@@ -844,6 +880,7 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
   for (int g = 0; g < F.ngrp; g++)                 // groups one after the other in one workspace
     for (int l = 0; l < F.nlev; l++) hz::launch_factor_level(F, l, g, w, fronts, scratch, c->status, tiny, c->st);
   hz::launch_merge_panels(F, c->st);              // merged solve supernodes of the sweeps
+  if (F.precision == 0) hz::launch_to_digits(F, c->st);
   if (verbose) {
     cudaStreamSynchronize(c->st);
     std::fprintf(stderr, "[hz] factor: %d levels in %.3f s\n", F.nlev,

@@ -7,18 +7,21 @@
 
 namespace hz {
 
-// One supernode of a batched multifrontal factorisation (56 bytes).
 // widest merged solve supernode of the complex128 sweeps (see FactorDev::ssn)
 constexpr int kMaxSolveK = 448;
 constexpr int kMaxSolveK64 = 512;   // the same for the complex64 sweeps
+constexpr int kMultiBwdRows = 128;  // rows per backward task of the batched sweeps
+
+// One supernode of a batched multifrontal factorisation (64 bytes).
 
 struct SnDev {
   int32_t k, m, first, parent;   // pivots, front order, first vector index, parent (-1 root)
   int32_t ld, pad_;              // panel leading dimension (m, or m rounded up to 4 for complex64)
   int64_t rowoff;                // into rowlist / cptr slots
   int64_t paneloff;              // panel (m x k, column-major, ld m) in the factor store
-  int64_t uoff;                  // update vector (m - k) in the solve workspace
+  int64_t uoff;                  // update rows (m - k): index into wpos
   int64_t frontoff;              // front (m x m, column-major) in the frontal workspace
+  int64_t eoff;                  // complex128 solve tree: row exponents of the panel's digits (m of them)
 };
 
 // Device view of a batched symbolic factorisation plus its numeric factor.
@@ -46,9 +49,10 @@ struct FactorDev {
   std::vector<MergeStep> merges;
   int64_t merge_tmp_elems = 0;
   void* merge_tmp = nullptr;
+  int16_t* rexp = nullptr;            // complex128: exponent of each solve panel row's digits (sweeps64.cu)
   int32_t* rowlist = nullptr;
-  int64_t* cptr = nullptr;
-  int64_t* cidx = nullptr;
+  uint32_t* cptr = nullptr;      // per row slot: its children's updates are u[cptr[r] .. cptr[r + 1])
+  uint32_t* wpos = nullptr;      // per update row (uoff + i): where in u it goes
   int32_t* rel = nullptr;
   int64_t* reloff = nullptr;
   int32_t* gidx = nullptr;       // ntot: global index of each local vector entry
@@ -91,6 +95,9 @@ struct FactorDev {
   cudaEvent_t* level_events = nullptr;  // optional (diagnostics): 2 * nlev + 1 events around sweep levels
   int* h_fwd_rt = nullptr;            // nlev: complex128 forward task rows (16 or 64)
   int* h_bwd_rows = nullptr;          // nlev: complex128 backward chunk rows
+  // per solve level: widest supernode (rounded up to 16 columns), tallest one, and the rows
+  // of the batched forward tasks
+  std::vector<int> h_lev_k, h_lev_m, h_mfwd_rt;
   int32_t max_slot = 0;
   // kernel variants of the schedule (host-side counts, reported through hz_stats)
   int32_t v_fwd_wide = 0, v_fwd_narrow = 0, v_bwd_wide = 0, v_bwd_narrow = 0;
@@ -118,7 +125,6 @@ struct FactorDev {
   unsigned int* mbwd_counters = nullptr;
   int64_t* h_mfwd_ptr = nullptr;
   int64_t* h_mbwd_ptr = nullptr;
-  int32_t mbwd_rows = 128;
   void* mt_loc = nullptr;
   void* mz_loc = nullptr;
   void* mx_loc = nullptr;
@@ -189,6 +195,11 @@ void launch_gather(const FactorDev& F, const double2* src, cudaStream_t st);
 void launch_solve(const FactorDev& F, cudaStream_t st);
 // Builds the merged solve panels from the factor panels (after the last factor level).
 void launch_merge_panels(const FactorDev& F, cudaStream_t st);
+// complex128 (sweeps64.cu): rewrites the solve panels as digits, and the sweeps on them for one
+// and for S interleaved right-hand sides.
+void launch_to_digits(const FactorDev& F, cudaStream_t st);
+void launch_solve_dig(const FactorDev& F, cudaStream_t st);
+void launch_solve_dig_multi(const FactorDev& F, int S, cudaStream_t st);
 void launch_prolong(const FactorDev& F, const double2* y, double2* z, cudaStream_t st);
 
 void launch_local_multi(const FactorDev& F, int S, const double2* src, const double2* y, double2* dst,

@@ -18,6 +18,7 @@
 #include <atomic>
 
 #include "dev.h"
+#include "dmath.cuh"
 
 namespace hz {
 
@@ -25,75 +26,7 @@ namespace hz {
 static std::atomic<long long> g_launches{0};
 long long launch_count() { return g_launches.load(); }
 void add_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
-#define HZ_COUNT() g_launches.fetch_add(1, std::memory_order_relaxed)
-
-// ---------------------------------------------------------------------------
-// complex helpers
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float xfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double xfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-template <typename V> struct RealOf;
-template <> struct RealOf<float2> { using T = float; };
-template <> struct RealOf<double2> { using T = double; };
-
-template <typename V>
-__device__ __forceinline__ V mk(typename RealOf<V>::T x, typename RealOf<V>::T y) {
-  V v;
-  v.x = x;
-  v.y = y;
-  return v;
-}
-template <typename V> __device__ __forceinline__ V czero() { return mk<V>(0, 0); }
-template <typename V> __device__ __forceinline__ V cadd(V a, V b) { return mk<V>(a.x + b.x, a.y + b.y); }
-template <typename V> __device__ __forceinline__ V csub(V a, V b) { return mk<V>(a.x - b.x, a.y - b.y); }
-template <typename V> __device__ __forceinline__ V cneg(V a) { return mk<V>(-a.x, -a.y); }
-template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
-  return mk<V>(xfma(a.x, b.x, -a.y * b.y), xfma(a.x, b.y, a.y * b.x));
-}
-// c + a b
-template <typename V> __device__ __forceinline__ V cmad(V a, V b, V c) {
-  c.x = xfma(a.x, b.x, c.x);
-  c.x = xfma(-a.y, b.y, c.x);
-  c.y = xfma(a.x, b.y, c.y);
-  c.y = xfma(a.y, b.x, c.y);
-  return c;
-}
-// c - a b
-template <typename V> __device__ __forceinline__ V cmsub(V a, V b, V c) {
-  c.x = xfma(-a.x, b.x, c.x);
-  c.x = xfma(a.y, b.y, c.x);
-  c.y = xfma(-a.x, b.y, c.y);
-  c.y = xfma(-a.y, b.x, c.y);
-  return c;
-}
-// c + conj(a) b
-template <typename V> __device__ __forceinline__ V cmadc(V a, V b, V c) {
-  c.x = xfma(a.x, b.x, c.x);
-  c.x = xfma(a.y, b.y, c.x);
-  c.y = xfma(a.x, b.y, c.y);
-  c.y = xfma(-a.y, b.x, c.y);
-  return c;
-}
-template <typename V> __device__ __forceinline__ V cinv(V a) {
-  const typename RealOf<V>::T d = a.x * a.x + a.y * a.y;
-  return mk<V>(a.x / d, -a.y / d);
-}
-template <typename V> __device__ __forceinline__ V from2(double2 a);
-template <> __device__ __forceinline__ double2 from2<double2>(double2 a) { return a; }
-template <> __device__ __forceinline__ float2 from2<float2>(double2 a) { return make_float2(float(a.x), float(a.y)); }
-__device__ __forceinline__ double2 to2(double2 a) { return a; }
-__device__ __forceinline__ double2 to2(float2 a) { return make_double2(a.x, a.y); }
-
-template <typename V> __device__ __forceinline__ V shfl_xor(V v, int m, int w = 32) {
-  v.x = __shfl_xor_sync(0xffffffffu, v.x, m, w);
-  v.y = __shfl_xor_sync(0xffffffffu, v.y, m, w);
-  return v;
-}
-template <typename V> __device__ __forceinline__ V warp_sum(V v) {
-  for (int o = 16; o > 0; o >>= 1) v = cadd(v, shfl_xor(v, o));
-  return v;
-}
+#define HZ_COUNT() add_launches(1)
 
 // widest supernode (pivot columns) any kernel handles
 constexpr int kMaxK = 128;
@@ -337,23 +270,6 @@ __global__ void __launch_bounds__(256) k_cb(const int4* tasks, const SnDev* sn, 
 // forever.  Either bit makes hz_factor return HZ_ERR_TIMEOUT and leaves the context
 // unfactored.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
-// Programmatic dependent launch (the triangular sweeps, one launch per tree level): a level's
-// kernel lets the next level's grid start as soon as all of its CTAs are running
-// (launch_dependents), and the next level reads nothing of the previous levels' results
-// before griddepcontrol.wait, which returns once the previous grid has completed and its
-// writes are visible.  Loads issued before the wait touch only the factor panels and the
-// task descriptors, which no sweep writes.  Without the launch attribute both are no-ops.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-// 16-byte asynchronous copy global -> shared (L2 only), and the wait for all of a thread's copies
-__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(sdst)), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
 __device__ __forceinline__ float tf32_rna(float x) {
   uint32_t y;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(x));
@@ -666,114 +582,10 @@ void launch_factor_level(const FactorDev& F, int lev, int grp, double w, void* f
 // ---------------------------------------------------------------------------
 // batched supernodal solves  (A_i^{-1}: forward with D^{-1}, then backward)
 // ---------------------------------------------------------------------------
-// Loads of solve vectors (t, u, z, x) bypass L1 (ld.global.cg): each value is read
-// once per sweep, so caching it in L1 only evicts panel lines.
-template <typename V> __device__ __forceinline__ V ldv(const V* p);
-template <> __device__ __forceinline__ float2 ldv<float2>(const float2* p) { return __ldcg(p); }
-template <> __device__ __forceinline__ double2 ldv<double2>(const double2* p) { return __ldcg(p); }
-
 template <typename V>
 __global__ void k_gather(int64_t ntot, const int32_t* gidx, const double2* src, V* dst) {
   for (int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; q < ntot; q += int64_t(gridDim.x) * blockDim.x)
     dst[q] = from2<V>(src[gidx[q]]);
-}
-
-// Forward, 64 rows of one supernode per task:
-//   b1 = t[pivots] + children's updates;  rows < k:  z = D^{-1} (T b1);
-//   rows >= k:  u = (children's updates) - G b1.
-// Forward, RT rows of one supernode per task; 256 threads = RT rows x (256 / RT)
-// column groups.  64-row tasks where a tree level has many supernodes; 16-row tasks
-// where it has few (the top of a single tree), so that such a level still spreads
-// over every SM (its FP64 arithmetic, not its bytes, is the bound there).
-template <typename V, int RT>
-__device__ __forceinline__ void fwd_item(const int2 t, const SnDev* sn, const int64_t* cptr, const int64_t* cidx,
-                                         const V* panels, const V* tin, V* zout, V* u) {
-  constexpr int CG = 256 / RT;
-  __shared__ V b1[kMaxSolveK];
-  __shared__ V part[CG][RT];
-  const SnDev S = sn[t.x];
-  const int k = S.k, m = S.m, tid = threadIdx.x;
-  const int64_t* cp = cptr + S.rowoff;
-  const int rr = tid % RT, cg = tid / RT;
-  const int r = t.y * RT + rr;
-  const V* P = panels + S.paneloff;
-  V acc = czero<V>(), acc2 = czero<V>();
-  if constexpr (RT == 16) {
-    // sparse levels: the panel values (at most kMaxK / 16 per thread) are loaded before
-    // the right-hand side is gathered; the sums keep the loop's order (even q: acc)
-    constexpr int MQ = kMaxK / CG;
-    V pv[MQ];
-    const int jmax = min(r, k);
-#pragma unroll
-    for (int q = 0; q < MQ; q++) {
-      const int j = cg + CG * q;
-      pv[q] = (r < m && j < jmax) ? P[r + int64_t(j) * S.ld] : czero<V>();
-    }
-    pdl_wait();
-    for (int j = tid; j < k; j += blockDim.x) {
-      V a = ldv(tin + S.first + j);
-      for (int64_t c = cp[j]; c < cp[j + 1]; c++) a = cadd(a, ldv(u + cidx[c]));
-      b1[j] = a;
-    }
-    __syncthreads();
-    if (r < m) {
-#pragma unroll
-      for (int q = 0; q < MQ; q++) {
-        const int j = cg + CG * q;
-        if (j < jmax) {
-          if (q % 2 == 0) acc = cmad(pv[q], b1[j], acc);
-          else acc2 = cmad(pv[q], b1[j], acc2);
-        }
-      }
-      // merged solve supernodes wider than kMaxK: the remaining columns, same chains
-      int j = cg + CG * MQ;
-      for (; j + CG < jmax; j += 2 * CG) {
-        acc = cmad(P[r + int64_t(j) * S.ld], b1[j], acc);
-        acc2 = cmad(P[r + int64_t(j + CG) * S.ld], b1[j + CG], acc2);
-      }
-      if (j < jmax) acc = cmad(P[r + int64_t(j) * S.ld], b1[j], acc);
-    }
-  } else {
-    pdl_wait();
-    for (int j = tid; j < k; j += blockDim.x) {
-      V a = ldv(tin + S.first + j);
-      for (int64_t c = cp[j]; c < cp[j + 1]; c++) a = cadd(a, ldv(u + cidx[c]));
-      b1[j] = a;
-    }
-    __syncthreads();
-    if (r < m) {
-      const int jmax = min(r, k);
-      int j = cg;
-      for (; j + CG < jmax; j += 2 * CG) {
-        acc = cmad(P[r + int64_t(j) * S.ld], b1[j], acc);
-        acc2 = cmad(P[r + int64_t(j + CG) * S.ld], b1[j + CG], acc2);
-      }
-      if (j < jmax) acc = cmad(P[r + int64_t(j) * S.ld], b1[j], acc);
-    }
-  }
-  part[cg][rr] = cadd(acc, acc2);
-  __syncthreads();
-  if (cg == 0 && r < m) {
-    V tot = part[0][rr];
-#pragma unroll
-    for (int q = 1; q < CG; q++) tot = cadd(tot, part[q][rr]);
-    if (r < k) {
-      zout[S.first + r] = cmul(P[r + int64_t(r) * S.ld], cadd(b1[r], tot));
-    } else {
-      V b2 = czero<V>();
-      for (int64_t c = cp[r]; c < cp[r + 1]; c++) b2 = cadd(b2, ldv(u + cidx[c]));
-      u[S.uoff + (r - k)] = csub(b2, tot);
-    }
-  }
-  __syncthreads();                                   // b1 / part are reused by the next item
-}
-
-template <typename V, int RT>
-__global__ void __launch_bounds__(256) k_fwd(const int2* tasks, const SnDev* sn, const int64_t* cptr,
-                                             const int64_t* cidx, const V* panels, const V* tin, V* zout,
-                                             V* u) {
-  pdl_trigger();
-  fwd_item<V, RT>(tasks[blockIdx.x], sn, cptr, cidx, panels, tin, zout, u);
 }
 
 // Backward, split over row chunks so that tall supernodes use many CTAs:
@@ -781,115 +593,6 @@ __global__ void __launch_bounds__(256) k_fwd(const int2* tasks, const SnDev* sn,
 //   vec = (z, -x[ancestor rows]) for 32 pivot columns j of one supernode;
 // then x[j] = z[j] + sum of the partials in chunk order (deterministic).
 constexpr int kBwdRows = 512;
-// Fused second stage of the backward sweep ("last block done"), for a (supernode,
-// column block) split over several row chunks: every partial-sum CTA of the pair
-// publishes its 32 sums, fences, and bumps the pair's counter; the CTA that brings it
-// to `chunks` adds the partials in chunk order (deterministic), writes x, and resets
-// the counter for the next sweep.  No CTA ever waits on another.  (The single-chunk
-// case finishes inside its own CTA and never touches the counter.)
-template <typename V>
-__device__ __forceinline__ void bwd_finish(const int4 fin, const SnDev& S, const V* zin, const V* partial_level,
-                                           V* x, unsigned int* counter) {
-  __shared__ unsigned int ticket;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) ticket = atomicAdd(counter, 1u);
-  __syncthreads();
-  if (ticket != unsigned(fin.w) - 1) return;
-  __threadfence();
-  const int c = threadIdx.x;
-  if (c < 32) {
-    const int j = fin.y * 32 + c;
-    if (j < S.k) {
-      V acc = czero<V>();
-      for (int ch = 0; ch < fin.w; ch++) {
-        const V* pp = partial_level + int64_t(fin.z + ch) * 32 + c;
-        V v;
-        if constexpr (sizeof(V) == 8) {
-          const float2 t = __ldcg(reinterpret_cast<const float2*>(pp));
-          v.x = t.x; v.y = t.y;
-        } else {
-          const double2 t = __ldcg(reinterpret_cast<const double2*>(pp));
-          v.x = t.x; v.y = t.y;
-        }
-        acc = cadd(acc, v);
-      }
-      x[S.first + j] = cadd(zin[S.first + j], acc);
-    }
-    if (c == 0) *counter = 0u;
-  }
-}
-
-// complex128 backward partial sums, transposed mapping for FP64 throughput: thread
-// (c, s) sums column j = 32 * block + c over slice s (of 8) of the chunk's rows,
-// reading its column sequentially (L1 reuse of each 128-byte line); the 8 slice
-// sums are then added in a fixed order.  No shuffle reductions on the FP64 pipe.
-// PF (narrow chunks of at most 64 rows, sparse levels): each thread's <= 8 panel values are
-// loaded before the chunk's right-hand side is gathered; the sums keep the loop's order.
-// A supernode that fits in one chunk is finished by its own CTA, with the same sums, without
-// the partial-sum round trip and ticket of bwd_finish.
-template <bool PF>
-__global__ void __launch_bounds__(256) k_bwd_partial_c128(const int4* tasks, const SnDev* sn,
-                                                          const int32_t* rowlist, const double2* panels,
-                                                          const double2* zin, double2* x, double2* partial,
-                                                          int rows, const int4* fins, unsigned int* counters) {
-  pdl_trigger();
-  __shared__ double2 vec[kBwdRows];
-  __shared__ double2 red[8][33];
-  const int4 t = tasks[blockIdx.x];
-  const SnDev S = sn[t.x];
-  const int k = S.k, m = S.m, tid = threadIdx.x, c = tid & 31, s = tid >> 5;
-  const int r0 = t.z * rows, r1 = min(m, r0 + rows);
-  const int32_t* rl = rowlist + S.rowoff;
-  const int j = t.y * 32 + c;
-  const int slice = (rows + 7) / 8;
-  const int ra = max(r0 + s * slice, j + 1), rb = min(r1, r0 + (s + 1) * slice);
-  const double2* col = panels + S.paneloff + int64_t(j < k ? j : 0) * S.ld;
-  double2 pre[8];
-  if constexpr (PF) {
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-      const int r = ra + q;
-      pre[q] = (j < k && r < rb) ? col[r] : make_double2(0.0, 0.0);
-    }
-  }
-  pdl_wait();
-  for (int r = r0 + tid; r < r1; r += blockDim.x) vec[r - r0] = (r < k) ? zin[S.first + r] : cneg(x[rl[r]]);
-  __syncthreads();
-  double2 a0 = make_double2(0.0, 0.0), a1 = a0;
-  if (j < k) {
-    if constexpr (PF) {
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int r = ra + q;
-        if (r < rb) {
-          if (q % 2 == 0) a0 = cmad(pre[q], vec[r - r0], a0);     // the loop's pairs (r, r + 1)
-          else a1 = cmad(pre[q], vec[r - r0], a1);
-        }
-      }
-    } else {
-      int r = ra;
-      for (; r + 1 < rb; r += 2) {
-        a0 = cmad(col[r], vec[r - r0], a0);
-        a1 = cmad(col[r + 1], vec[r + 1 - r0], a1);
-      }
-      if (r < rb) a0 = cmad(col[r], vec[r - r0], a0);
-    }
-  }
-  red[s][c] = cadd(a0, a1);
-  __syncthreads();
-  const bool single = m <= rows;                     // the only chunk: finish here, no ticket
-  if (s == 0) {
-    double2 tot = red[0][c];
-    for (int q = 1; q < 8; q++) tot = cadd(tot, red[q][c]);
-    if (!single)
-      partial[int64_t(blockIdx.x) * 32 + c] = tot;
-    else if (j < k)
-      x[S.first + j] = cadd(zin[S.first + j], cadd(make_double2(0.0, 0.0), tot));
-  }
-  if (!single) bwd_finish<double2>(fins[t.w], S, zin, partial, x, counters + t.w);
-}
-
 // complex64 forward, 512 / CG rows of one supernode per task: thread t owns the row
 // pair (2p, 2p+1), p = t % (256 / CG), for the pivot columns j = t / (256 / CG) mod CG,
 // with 16-byte loads; the right-hand side b1 is gathered once per task.  CG = 2 (256
@@ -902,8 +605,8 @@ __global__ void __launch_bounds__(256) k_bwd_partial_c128(const int4* tasks, con
 // (even q on one chain, odd q on the other).
 constexpr int kFwdAsync = 8, kFwdNarrowAsync = 8;
 template <int CG>
-__device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, const int64_t* cptr,
-                                             const int64_t* cidx, const float2* panels, const float2* tin,
+__device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, const uint32_t* cptr,
+                                             const uint32_t* wpos, const float2* panels, const float2* tin,
                                              float2* zout, float2* u) {
   constexpr int NP = 256 / CG;                       // row pairs per task
   constexpr int ROWS = 2 * NP;
@@ -912,9 +615,14 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
   const SnDev S = sn[t.x];
   const int k = S.k, m = S.m, tid = threadIdx.x;
   const int pr = tid % NP, cg = tid / NP;
-  const int64_t* cp = cptr + S.rowoff;
+  const uint32_t* cp = cptr + S.rowoff;
   const int r = t.y * ROWS + 2 * pr;                 // rows r, r + 1 (r even, ld % 4 == 0)
   const int rr = t.y * ROWS + tid;                   // update row finished by this thread
+  // where this thread's child contributions lie and where its update goes: loaded before the
+  // wait for the previous level, so that only the contributions themselves come after it
+  const bool upd = tid < ROWS && rr >= k && rr < m;
+  const uint32_t g0 = tid < k ? cp[tid] : 0u, g1 = tid < k ? cp[tid + 1] : 0u;
+  const uint32_t h0 = upd ? cp[rr] : 0u, h1 = upd ? cp[rr + 1] : 0u, uw = upd ? wpos[S.uoff + (rr - k)] : 0u;
   float2 a0 = make_float2(0.f, 0.f), a1 = a0, c0 = a0, c1 = a0, b2 = a0;
   if constexpr (CG == 8) {
     constexpr int MQ = kMaxK / CG, PF = 8;              // PF of the MQ columns are prefetched,
@@ -935,13 +643,13 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
       if (r < m && j < j1) cp_async16(&apf[(q - PF) * 256 + tid], P4 + int64_t(j) * ld4);
     }
     pdl_wait();
-    for (int jj = tid; jj < k; jj += blockDim.x) {
+    for (int jj = tid; jj < k; jj += 256) {
+      const uint32_t c0 = jj == tid ? g0 : cp[jj], c1 = jj == tid ? g1 : cp[jj + 1];
       float2 acc = ldv(tin + S.first + jj);
-      for (int64_t c = cp[jj]; c < cp[jj + 1]; c++) acc = cadd(acc, ldv(u + cidx[c]));
+      for (uint32_t c = c0; c < c1; c++) acc = cadd(acc, ldv(u + c));
       b1[jj] = acc;
     }
-    if (tid < ROWS && rr >= k && rr < m)
-      for (int64_t c = cp[rr]; c < cp[rr + 1]; c++) b2 = cadd(b2, ldv(u + cidx[c]));
+    for (uint32_t c = h0; c < h1; c++) b2 = cadd(b2, ldv(u + c));
     if constexpr (NA > 0) cp_async_wait_all();        // each thread reads back only its own copies
     __syncthreads();
     if (r < m) {
@@ -998,13 +706,13 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
       if (r < m && j < j1) cp_async16(&apf[q * 256 + tid], P4 + int64_t(j) * ld4);
     }
     pdl_wait();
-    for (int jj = tid; jj < k; jj += blockDim.x) {
+    for (int jj = tid; jj < k; jj += 256) {
+      const uint32_t c0 = jj == tid ? g0 : cp[jj], c1 = jj == tid ? g1 : cp[jj + 1];
       float2 acc = ldv(tin + S.first + jj);
-      for (int64_t c = cp[jj]; c < cp[jj + 1]; c++) acc = cadd(acc, ldv(u + cidx[c]));
+      for (uint32_t c = c0; c < c1; c++) acc = cadd(acc, ldv(u + c));
       b1[jj] = acc;
     }
-    if (tid < ROWS && rr >= k && rr < m)
-      for (int64_t c = cp[rr]; c < cp[rr + 1]; c++) b2 = cadd(b2, ldv(u + cidx[c]));
+    for (uint32_t c = h0; c < h1; c++) b2 = cadd(b2, ldv(u + c));
     if constexpr (NA > 0) cp_async_wait_all();        // each thread reads back only its own copies
     __syncthreads();
     if (r < m) {
@@ -1066,17 +774,16 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
     if (rr < k)
       zout[S.first + rr] = cmul(P[rr + int64_t(rr) * S.ld], cadd(b1[rr], tot));
     else
-      u[S.uoff + (rr - k)] = csub(b2, tot);
+      u[uw] = csub(b2, tot);
   }
-  __syncthreads();                                   // b1 / part are reused by the next item
 }
 
 template <int CG>
-__global__ void __launch_bounds__(256, 4) k_fwd_c64(const int2* tasks, const SnDev* sn, const int64_t* cptr,
-                                                 const int64_t* cidx, const float2* panels, const float2* tin,
+__global__ void __launch_bounds__(256, 4) k_fwd_c64(const int2* tasks, const SnDev* sn, const uint32_t* cptr,
+                                                 const uint32_t* wpos, const float2* panels, const float2* tin,
                                                  float2* zout, float2* u) {
   pdl_trigger();
-  fwd_c64_item<CG>(tasks[blockIdx.x], sn, cptr, cidx, panels, tin, zout, u);
+  fwd_c64_item<CG>(tasks[blockIdx.x], sn, cptr, wpos, panels, tin, zout, u);
 }
 
 // complex64 backward partial sums with 16-byte loads (two rows per lane), two forms:
@@ -1207,56 +914,21 @@ __global__ void k_prolong(int64_t n, const int64_t* pptr, const int32_t* pidx, c
   }
 }
 
-// One tree level of a sweep.  The complex64 sweeps launch with programmatic stream
-// serialisation (unless HZ_NO_PDL is set), so that a level's CTAs start their panel loads
-// while the previous level's grid drains; the kernels wait (pdl_wait) before they read any
-// result of that level.  The complex128 sweeps (FP64-bound) launch plainly: on the coarse
-// factor the early start measured slower (5.8 -> 6.2 ms per coarse solve on the 5 Hz
-// workload).
-static bool pdl_enabled(bool fp64) {
-  static const bool on = std::getenv("HZ_NO_PDL") == nullptr;
-  return on && !fp64;
-}
-template <typename... KArgs, typename... Args>
-static void launch_level(void (*kern)(KArgs...), int64_t grid, cudaStream_t st, bool pdl, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(grid));
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = pdl ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
-template <typename V>
-static void solve_t(const FactorDev& F, cudaStream_t st) {
-  const V* P = (const V*)F.panels;
-  V* t = (V*)F.t_loc;
-  V* z = (V*)F.z_loc;
-  V* x = (V*)F.x_loc;
-  V* u = (V*)F.u_ws;
-  V* part = (V*)F.bwd_partial;
-  const SnDev* SN = F.ssn ? F.ssn : F.sn;
-  const bool pdl = pdl_enabled(sizeof(V) == 16);
+static void solve_c64(const FactorDev& F, cudaStream_t st) {
+  const float2* P = (const float2*)F.panels;
+  float2 *t = (float2*)F.t_loc, *z = (float2*)F.z_loc, *x = (float2*)F.x_loc, *u = (float2*)F.u_ws;
+  float2* part = (float2*)F.bwd_partial;
+  const bool pdl = pdl_enabled();
   if (F.level_events) cudaEventRecord(F.level_events[0], st);
   for (int l = 0; l < F.snlev; l++) {
     const int64_t b = F.h_fwd_ptr[l], e = F.h_fwd_ptr[l + 1];
     if (e > b) {
       HZ_COUNT();
       const int2* tk = F.fwd_tasks + b;
-      if constexpr (sizeof(V) == 8) {
-        if (F.h_fwd_rt && F.h_fwd_rt[l] == 64)
-          launch_level(k_fwd_c64<8>, e - b, st, pdl, tk, SN, F.cptr, F.cidx, P, t, z, u);
-        else
-          launch_level(k_fwd_c64<2>, e - b, st, pdl, tk, SN, F.cptr, F.cidx, P, t, z, u);
-      } else if (F.h_fwd_rt && F.h_fwd_rt[l] == 16)
-        launch_level(k_fwd<V, 16>, e - b, st, pdl, tk, SN, F.cptr, F.cidx, P, t, z, u);
+      if (F.h_fwd_rt[l] == 64)
+        launch_level(k_fwd_c64<8>, e - b, 256, 0, st, pdl, tk, F.ssn, F.cptr, F.wpos, P, t, z, u);
       else
-        launch_level(k_fwd<V, 64>, e - b, st, pdl, tk, SN, F.cptr, F.cidx, P, t, z, u);
+        launch_level(k_fwd_c64<2>, e - b, 256, 0, st, pdl, tk, F.ssn, F.cptr, F.wpos, P, t, z, u);
     }
     if (F.level_events) cudaEventRecord(F.level_events[1 + l], st);
   }
@@ -1265,22 +937,13 @@ static void solve_t(const FactorDev& F, cudaStream_t st) {
     if (e > b) {
       HZ_COUNT();
       const int4* tk = F.bwd_tasks + b;
-      const int rows = F.h_bwd_rows ? F.h_bwd_rows[l] : F.bwd_rows;
-      if constexpr (sizeof(V) == 8) {
-        if (rows <= 128)
-          launch_level(k_bwd_partial_c64<kBwdPrefetch>, e - b, st, pdl, tk, SN, F.rowlist, P, z, x, part, rows,
-                       F.bfin_tasks, F.bwd_counters);
-        else
-          launch_level(k_bwd_partial_c64<kBwdAsync>, e - b, st, pdl, tk, SN, F.rowlist, P, z, x, part, rows,
-                       F.bfin_tasks, F.bwd_counters);
-      } else {
-        if (rows <= 64)
-          launch_level(k_bwd_partial_c128<true>, e - b, st, pdl, tk, SN, F.rowlist, P, z, x, part, rows,
-                       F.bfin_tasks, F.bwd_counters);
-        else
-          launch_level(k_bwd_partial_c128<false>, e - b, st, pdl, tk, SN, F.rowlist, P, z, x, part, rows,
-                       F.bfin_tasks, F.bwd_counters);
-      }
+      const int rows = F.h_bwd_rows[l];
+      if (rows <= 128)
+        launch_level(k_bwd_partial_c64<kBwdPrefetch>, e - b, 256, 0, st, pdl, tk, F.ssn, F.rowlist, P, z, x, part, rows,
+                     F.bfin_tasks, F.bwd_counters);
+      else
+        launch_level(k_bwd_partial_c64<kBwdAsync>, e - b, 256, 0, st, pdl, tk, F.ssn, F.rowlist, P, z, x, part, rows,
+                     F.bfin_tasks, F.bwd_counters);
     }
     if (F.level_events) cudaEventRecord(F.level_events[1 + F.snlev + (F.snlev - 1 - l)], st);
   }
@@ -1298,8 +961,8 @@ void launch_gather(const FactorDev& F, const double2* src, cudaStream_t st) {
 }
 
 void launch_solve(const FactorDev& F, cudaStream_t st) {
-  if (F.precision == 0) solve_t<double2>(F, st);
-  else solve_t<float2>(F, st);
+  if (F.precision == 0) launch_solve_dig(F, st);
+  else solve_c64(F, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1464,20 +1127,20 @@ __global__ void k_prolong_multi(int64_t n, const int64_t* pptr, const int32_t* p
 
 // Forward, 64 rows x S right-hand sides per task; 128 threads = 64 rows x 2 column parities.
 template <typename V, int S>
-__global__ void __launch_bounds__(128) k_fwd_multi(const int2* tasks, const SnDev* sn, const int64_t* cptr,
-                                                   const int64_t* cidx, const V* panels, const V* tin, V* zout,
-                                                   V* u) {
+__global__ void __launch_bounds__(128) k_fwd_multi(const int2* tasks, const SnDev* sn, const uint32_t* cptr,
+                                                   const uint32_t* wpos, const V* panels, const V* tin, V* zout,
+                                                   V* u, int kpad) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* b1 = reinterpret_cast<V*>(smem_raw);               // kMaxK x S
-  V* part = b1 + kMaxK * S;                               // 2 x 64 x S
+  V* b1 = reinterpret_cast<V*>(smem_raw);               // kpad x S
+  V* part = b1 + kpad * S;                                // 2 x 64 x S
   const int2 t = tasks[blockIdx.x];
   const SnDev Sn = sn[t.x];
   const int k = Sn.k, m = Sn.m, tid = threadIdx.x;
-  const int64_t* cp = cptr + Sn.rowoff;
+  const uint32_t* cp = cptr + Sn.rowoff;
   for (int e = tid; e < k * S; e += blockDim.x) {
     const int j = e / S, i = e % S;
     V acc = tin[int64_t(Sn.first + j) * S + i];
-    for (int64_t c = cp[j]; c < cp[j + 1]; c++) acc = cadd(acc, u[cidx[c] * S + i]);
+    for (uint32_t c = cp[j]; c < cp[j + 1]; c++) acc = cadd(acc, u[int64_t(c) * S + i]);
     b1[e] = acc;
   }
   __syncthreads();
@@ -1508,8 +1171,8 @@ __global__ void __launch_bounds__(128) k_fwd_multi(const int2* tasks, const SnDe
       zout[int64_t(Sn.first + rw) * S + i] = cmul(panels[Sn.paneloff + rw + int64_t(rw) * Sn.ld], cadd(b1[rw * S + i], tot));
     } else {
       V b2 = czero<V>();
-      for (int64_t c = cp[rw]; c < cp[rw + 1]; c++) b2 = cadd(b2, u[cidx[c] * S + i]);
-      u[(Sn.uoff + (rw - k)) * S + i] = csub(b2, tot);
+      for (uint32_t c = cp[rw]; c < cp[rw + 1]; c++) b2 = cadd(b2, u[int64_t(c) * S + i]);
+      u[int64_t(wpos[Sn.uoff + (rw - k)]) * S + i] = csub(b2, tot);
     }
   }
 }
@@ -1589,31 +1252,34 @@ __global__ void __launch_bounds__(128) k_bwd_multi(const int4* tasks, const SnDe
   if (tid == 0) counters[t.w] = 0u;
 }
 
-template <typename V, int S>
-static void solve_multi_t(const FactorDev& F, const V* t_in, V* z, V* x, V* u, V* part, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    // at most 64 KB are used (S = 16, complex128); leave room for the static shared variables
+template <int S>
+static void solve_multi_c64(const FactorDev& F, cudaStream_t st) {
+  using V = float2;
+  static const bool attr = [] {
     cudaFuncSetAttribute(k_fwd_multi<V, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_bwd_multi<V, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
+    return true;
+  }();
+  (void)attr;
   const V* P = (const V*)F.panels;
-  const size_t fsm = size_t(kMaxK * S + 2 * 64 * S) * sizeof(V);
-  for (int l = 0; l < F.nlev; l++) {
+  V *t = (V*)F.mt_loc, *z = (V*)F.mz_loc, *x = (V*)F.mx_loc, *u = (V*)F.mu_ws;
+  for (int l = 0; l < F.snlev; l++) {
     const int64_t b = F.h_mfwd_ptr[l], e = F.h_mfwd_ptr[l + 1];
     if (e > b) {
       HZ_COUNT();
-      k_fwd_multi<V, S><<<unsigned(e - b), 128, fsm, st>>>(F.mfwd_tasks + b, F.sn, F.cptr, F.cidx, P, t_in, z, u);
+      const int kpad = F.h_lev_k[l];
+      const size_t fsm = size_t(kpad * S + 2 * 64 * S) * sizeof(V);
+      k_fwd_multi<V, S><<<unsigned(e - b), 128, fsm, st>>>(F.mfwd_tasks + b, F.ssn, F.cptr, F.wpos, P, t, z, u, kpad);
     }
   }
-  const size_t bsm = size_t(F.mbwd_rows * S + 4 * 32 * S) * sizeof(V);
-  for (int l = F.nlev - 1; l >= 0; l--) {
+  const size_t bsm = size_t(kMultiBwdRows * S + 4 * 32 * S) * sizeof(V);
+  for (int l = F.snlev - 1; l >= 0; l--) {
     const int64_t b = F.h_mbwd_ptr[l], e = F.h_mbwd_ptr[l + 1];
     if (e > b) {
       HZ_COUNT();
-      k_bwd_multi<V, S><<<unsigned(e - b), 128, bsm, st>>>(F.mbwd_tasks + b, F.sn, F.rowlist, P, z, x, part,
-                                                           F.mbwd_rows, F.mbfin_tasks, F.mbwd_counters);
+      k_bwd_multi<V, S><<<unsigned(e - b), 128, bsm, st>>>(F.mbwd_tasks + b, F.ssn, F.rowlist, P, z, x,
+                                                           (V*)F.mbwd_partial, kMultiBwdRows, F.mbfin_tasks,
+                                                           F.mbwd_counters);
     }
   }
 }
@@ -1623,7 +1289,8 @@ static void prec_multi_t(const FactorDev& F, const double2* src, const double2* 
   V* t = (V*)F.mt_loc;
   HZ_COUNT();
   k_gather_multi<V, S><<<grid_for(F.ntot * S, 256), 256, 0, st>>>(F.ntot, F.gidx, src, t);
-  solve_multi_t<V, S>(F, t, (V*)F.mz_loc, (V*)F.mx_loc, (V*)F.mu_ws, (V*)F.mbwd_partial, st);
+  if constexpr (sizeof(V) == 8) solve_multi_c64<S>(F, st);
+  else launch_solve_dig_multi(F, S, st);
   HZ_COUNT();
   k_prolong_multi<V, S><<<grid_for(F.nglob * S, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw,
                                                                    (const V*)F.mx_loc, y, dst);

@@ -1,0 +1,930 @@
+// Triangular sweeps of the complex128 factors on the tensor cores (sm_103a).
+//
+// GB300 issues two FP64 FMAs per SM and clock, so a complex128 sweep on the FP64 units takes
+// two SM-clocks per panel entry and right-hand side, three times what reading the entry
+// costs.  Here the products run as exact integer products instead:
+//   * after the factorisation every panel entry x (rows below the pivot) is rewritten in
+//     place as two 64-bit integers D = x 2^(1084 - E), E the largest exponent field of the
+//     entry's panel row, |D| < 2^62; each as eight balanced base-256 digits in [-128, 127],
+//     stored with 128 added (so a byte is a digit).  The row's E - 1084 is kept beside the
+//     panel.  Same bytes as the doubles; the diagonal keeps D^{-1} in FP64;
+//   * the right-hand side of a task is written in digits too, with one exponent per task
+//     and right-hand side;
+//   * a digit product sum runs on mma.sync m16n8k16 (f16 in, f32 accumulators): a digit and
+//     a product of digits are exact, and at most 8 digit pairs x 64 columns x 2 products of
+//     at most 2^14 meet in one accumulator, at most 2^24, so every sum is exact too.
+//     Digit pairs (i, j) with i + j <= 7 are kept; what is dropped is below 2^-59 (rms) of
+//     the largest product for 64 columns.
+// The digits of one operand hold 62 bits below the row's largest entry, against the 53 of a
+// double below each entry, and the column sum is exact where the FP64 loop rounded at every
+// step.  A right-hand side with an infinity or NaN gives NaN in every row of its tasks.
+//
+// Bound: reading the panels (16 bytes per entry: 0.69 SM-clocks at 6.8 TB/s), beside about
+// 0.3 for unpacking digits (20 integer and half2 operations per entry) and 0.25 for the
+// products of one right-hand side (32 MMAs of 2 clocks per 256 entries).
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "dev.h"
+#include "dmath.cuh"
+
+namespace hz {
+
+namespace {
+
+constexpr int kBias = 1084;               // D = x 2^(kBias - E)
+constexpr int16_t kRowNonFinite = 0x7fff;
+constexpr uint64_t kDigitBias = 0x8080808080808080ull;
+constexpr uint32_t kZeroWord = 0x80808080u;
+constexpr int kPairStride = 24;           // words per column pair of a digit vector (15 used; 24 t mod 32 differ)
+
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// digits (with 128 added to each) of x, with x < 2^(E - 1022) for the largest exponent field E
+// of its group; sh = 1 + E - max(exponent field of x, 1)
+__device__ __forceinline__ uint64_t to_digits(double x, int sh) {
+  const int hi = __double2hiint(x);
+  const uint32_t top = (uint32_t(hi) & 0xfffffu) | (((hi >> 20) & 0x7ff) ? 0x100000u : 0u);
+  const uint64_t m = ((uint64_t(top) << 32) | uint32_t(__double2loint(x))) << 10;
+  const uint64_t d = m >> min(sh, 63);
+  return (hi < 0 ? ~d + 1 : d) + kDigitBias;
+}
+
+// 2^e s for a result s of a digit product sum
+__device__ __forceinline__ double scale2(double s, int e) {
+  if (e >= -1000 && e <= 1000) return s * __hiloint2double((e + 1023) << 20, 0);
+  return scalbn(s, e);
+}
+
+__device__ __forceinline__ uint32_t h2sub(uint32_t a) {      // half2 (1024 + b) -> b - 128
+  const __half2 c = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));
+  __half2 v = *reinterpret_cast<__half2*>(&a);
+  v = __hsub2(v, c);
+  return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// the four digits of two 32-bit digit words as half2 (x's digit, y's digit), most significant first
+__device__ __forceinline__ void word_digits(uint32_t x, uint32_t y, uint32_t* out) {
+  const uint32_t p = __byte_perm(x, y, 0x5140), q = __byte_perm(x, y, 0x7362);
+  out[0] = h2sub(__byte_perm(q, 0x64646464u, 0x4342));
+  out[1] = h2sub(__byte_perm(q, 0x64646464u, 0x4140));
+  out[2] = h2sub(__byte_perm(p, 0x64646464u, 0x4342));
+  out[3] = h2sub(__byte_perm(p, 0x64646464u, 0x4140));
+}
+
+__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+               "{%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ uint4 ld_panel(const uint4* p) { return __ldg(p); }
+__device__ __forceinline__ uint4 zero_entry() { return make_uint4(kZeroWord, kZeroWord, kZeroWord, kZeroWord); }
+
+// Position of column pair p of a 16-column step in a digit vector: fragment register b0 reads
+// pairs at positions 0-3, b1 at 4-7.  forward: pairs (2t, 2t + 1) and (2t + 8, 2t + 9) as they
+// come; backward: lane t holds four consecutive rows, pairs 2t and 2t + 1.
+__device__ __forceinline__ int pair_pos_bwd(int p) { return (p >> 1) + 4 * (p & 1); }
+
+// One 16 x 16 step of the panel for one right-hand side: raw[q], q = 0..7, are the entries
+// (row half q & 1, k index order 2t, 2t+1, 2t+8, 2t+9 = q >> 1).  c: Re x re, Im x im,
+// Re x im and Im x re, whose eight columns are the digit weights (four chains of eight MMAs).
+__device__ __forceinline__ void step_single(const uint4* raw, const uint32_t* bre, const uint32_t* bim, int off,
+                                            float (*c)[4]) {
+#pragma unroll
+  for (int w = 0; w < 2; w++) {                      // high words: digits 0-3; low words: 4-7
+    uint32_t ar[4][4], ai[4][4];                     // [digit][fragment register]
+#pragma unroll
+    for (int h = 0; h < 2; h++)                      // row half
+#pragma unroll
+      for (int kp = 0; kp < 2; kp++) {               // k pair
+        const uint4 x = raw[(2 * kp) * 2 + h], y = raw[(2 * kp + 1) * 2 + h];
+        uint32_t o[4];
+        word_digits(w == 0 ? x.y : x.x, w == 0 ? y.y : y.x, o);
+#pragma unroll
+        for (int d = 0; d < 4; d++) ar[d][2 * kp + h] = o[d];
+        word_digits(w == 0 ? x.w : x.z, w == 0 ? y.w : y.z, o);
+#pragma unroll
+        for (int d = 0; d < 4; d++) ai[d][2 * kp + h] = o[d];
+      }
+#pragma unroll
+    for (int d = 0; d < 4; d++) {
+      const int o = off - (4 * w + d);
+      const uint32_t r0 = bre[o], r1 = bre[o + 4 * kPairStride], i0 = bim[o], i1 = bim[o + 4 * kPairStride];
+      mma16816(c[0], ar[d], r0, r1);
+      mma16816(c[1], ai[d], i0, i1);
+      mma16816(c[2], ar[d], i0, i1);
+      mma16816(c[3], ai[d], r0, r1);
+    }
+  }
+}
+
+// adds the accumulators to the sums of the real part (tot[0]) and the imaginary part (tot[1])
+__device__ __forceinline__ void flush_single(float (*c)[4], int (*tot)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    tot[0][q] += __float2int_rn(c[0][q]) - __float2int_rn(c[1][q]);
+    tot[1][q] += __float2int_rn(c[2][q]) + __float2int_rn(c[3][q]);
+    c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
+  }
+}
+
+// The eight weighted digit sums of a row lie two per lane in a quad: lane t = 0 returns the upper
+// four and t = 2 the lower four as one integer (digit weights 256^3 .. 1).
+__device__ __forceinline__ int64_t quad_half(int hi, int lo) {
+  const int64_t v = int64_t(hi) * 256 + lo;
+  return v * 65536 + __shfl_xor_sync(0xffffffffu, v, 1);
+}
+// value of the two halves: result 2^88 2^(exponents)
+__device__ __forceinline__ double halves_value(int64_t hi, int64_t lo) {
+  return fma(double(lo), 0x1p-32, double(hi));
+}
+
+// a + the pt-th parts of u[c0 .. c1), in order; the first two loads are issued together
+__device__ __forceinline__ double add_updates_part(double a, const double* ud, uint32_t c0, uint32_t c1, int pt) {
+  double v0 = 0.0, v1 = 0.0;
+  if (c0 < c1) v0 = __ldcg(ud + 2 * int64_t(c0) + pt);
+  if (c0 + 1 < c1) v1 = __ldcg(ud + 2 * int64_t(c0) + 2 + pt);
+  a = (a + v0) + v1;
+  for (uint32_t c = c0 + 2; c < c1; c++) a += __ldcg(ud + 2 * int64_t(c) + pt);
+  return a;
+}
+
+// Writes the digits of the value pair (x, y) (already in units of the group's exponent) as the
+// shifted-digit rows of a digit vector: word 7 + i is digit i, words 0-6 are zero.
+__device__ __forceinline__ void put_pair(uint32_t* dst, uint64_t dx, uint64_t dy) {
+#pragma unroll
+  for (int i = 0; i < 7; i++) dst[i] = 0u;
+  uint32_t o[4];
+  word_digits(uint32_t(dx >> 32), uint32_t(dy >> 32), o);
+#pragma unroll
+  for (int i = 0; i < 4; i++) dst[7 + i] = o[i];
+  word_digits(uint32_t(dx), uint32_t(dy), o);
+#pragma unroll
+  for (int i = 0; i < 4; i++) dst[11 + i] = o[i];
+}
+
+// largest value over the block (128 threads); syncs
+__device__ __forceinline__ int block_max(int v, int* red) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return max(max(red[0], red[1]), max(red[2], red[3]));
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// panels -> digits, in place; one task = RT rows of one solve supernode
+// ---------------------------------------------------------------------------
+template <int RT>
+__global__ void __launch_bounds__(256) k_to_digits(const int2* tasks, const SnDev* sn, double2* panels,
+                                                   int16_t* rexp) {
+  constexpr int CG = 256 / RT;
+  __shared__ int red[CG][RT];
+  const int2 t = tasks[blockIdx.x];
+  const SnDev S = sn[t.x];
+  const int rr = threadIdx.x % RT, cg = threadIdx.x / RT, r = t.y * RT + rr;
+  const int jmax = r < S.m ? min(r, S.k) : 0;
+  double2* P = panels + S.paneloff + r;
+  int e = 1;
+  for (int j = cg; j < jmax; j += CG) {
+    const double2 v = P[int64_t(j) * S.ld];
+    e = max(e, max(exp_field(v.x), exp_field(v.y)));
+  }
+  red[cg][rr] = e;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < CG; q++) e = max(e, red[q][rr]);
+  for (int j = cg; j < jmax; j += CG) {
+    const double2 v = P[int64_t(j) * S.ld];
+    const uint64_t a = to_digits(v.x, 1 + e - max(exp_field(v.x), 1));
+    const uint64_t b = to_digits(v.y, 1 + e - max(exp_field(v.y), 1));
+    P[int64_t(j) * S.ld] = make_double2(__longlong_as_double(int64_t(a)), __longlong_as_double(int64_t(b)));
+  }
+  if (cg == 0 && r < S.m) rexp[S.eoff + r] = e == 0x7ff ? kRowNonFinite : int16_t(e - kBias);
+}
+
+// ---------------------------------------------------------------------------
+// one right-hand side
+// ---------------------------------------------------------------------------
+// Panel steps of a warp are copied into its own ring of kRing slots (4 KB each) by cp.async, the
+// first ones before the right-hand side is gathered; each lane reads back only what it copied,
+// so the ring needs no barrier.  Measured on the subdomain sweeps of the 349,461-dof survey
+// model (9.8 GB, 16 subdomains): 5.82 ms on the FP64 units; with digits 4.7 ms with the panels
+// in registers (one step ahead, two blocks of 256 threads per SM), 3.81 ms with this ring (four
+// blocks of 128; five blocks 3.93, three slots 4.41).  About a third of a task's time is its
+// 16-column steps; the rest is the chain task -> supernode -> right-hand side -> digits, which
+// the other blocks of the SM cover only in part.
+constexpr int kRing = 2;
+
+// Forward, 16 MT rows of one supernode per task (rows < k: z = D^{-1} (T b1); rows >= k:
+// u = children's updates - G b1); 4 warps = MT row tiles x 4 / MT groups of 16-column steps.
+// What the last step needs (children's updates of the update rows, D^{-1}, row exponents) is
+// loaded with the right-hand side.
+template <int MT>
+__global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnDev* sn, const uint32_t* cptr,
+                                                    const uint32_t* wpos, const double2* panels,
+                                                    const int16_t* rexp, const double2* tin, double2* zout,
+                                                    double2* u, int kpad) {
+  pdl_trigger();
+  constexpr int CG = 4 / MT, RT = 16 * MT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint4* ring = reinterpret_cast<uint4*>(smem_raw);                      // 4 warps x kRing x 8 x 32
+  double* b1 = reinterpret_cast<double*>(ring + 4 * kRing * 256);        // kpad x 2
+  uint32_t* bre = reinterpret_cast<uint32_t*>(b1 + 2 * kpad);            // kpad / 2 pairs x kPairStride
+  uint32_t* bim = bre + (kpad / 2) * kPairStride;
+  __shared__ int64_t sums[CG][RT][2][2];                                 // [group][row][part][half]
+  __shared__ int red[4];
+  const int2 tk = tasks[blockIdx.x];
+  const SnDev S = sn[tk.x];
+  const int k = S.k, m = S.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int g = lane >> 2, t = lane & 3, mt = wid % MT, cg = wid / MT;
+  const uint32_t* cp = cptr + S.rowoff;
+  const int row0 = tk.y * RT + mt * 16;
+  const int ra = row0 + g, rb = ra + 8;
+  const int ja = ra < m ? min(ra, k) : 0, jb = rb < m ? min(rb, k) : 0;
+  const int nst = row0 < m ? (min(row0 + 15, k) + 15) / 16 : 0;          // 16-column steps of this tile
+  const int nfull = row0 + 15 < m ? min(row0, k) / 16 : 0;               // steps without a masked entry
+  const uint4* P = reinterpret_cast<const uint4*>(panels + S.paneloff);
+  uint4* myring = ring + wid * (kRing * 256) + lane;
+  auto issue = [&](int s, int slot) {
+    if (s < nst) {
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int j = 16 * s + 2 * t + (q & 1) + 8 * (q >> 1);
+        const uint4* col = P + int64_t(j) * S.ld;
+        if (j < ja) cp_async16(myring + slot * 256 + (2 * q) * 32, col + ra);
+        if (j < jb) cp_async16(myring + slot * 256 + (2 * q + 1) * 32, col + rb);
+      }
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int q = 0; q < kRing; q++) issue(cg + q * CG, q);
+  // this thread's result: row tid / 2 of the task, part tid & 1
+  const int r = tk.y * RT + (tid >> 1), pt = tid & 1;
+  const bool mine = tid < 2 * RT && r < m;
+  double2 dinv = make_double2(0.0, 0.0);
+  int re = 0;
+  const bool upd = mine && r >= k;
+  if (mine) {
+    re = rexp[S.eoff + r];
+    if (r < k) dinv = panels[S.paneloff + r + int64_t(r) * S.ld];
+  }
+  // where this thread's child contributions lie and where its update goes
+  const uint32_t h0 = upd ? cp[r] : 0u, h1 = upd ? cp[r + 1] : 0u, uw = upd ? wpos[S.uoff + (r - k)] : 0u;
+  const uint32_t g0 = tid < 2 * k ? cp[tid >> 1] : 0u, g1 = tid < 2 * k ? cp[(tid >> 1) + 1] : 0u;
+  pdl_wait();
+  const double *tind = reinterpret_cast<const double*>(tin + S.first), *ud = reinterpret_cast<const double*>(u);
+  int e = 1;
+  for (int q = tid; q < 2 * k; q += 128) {
+    const int j = q >> 1;
+    const uint32_t c0 = q == tid ? g0 : cp[j], c1 = q == tid ? g1 : cp[j + 1];
+    const double a = add_updates_part(__ldcg(tind + q), ud, c0, c1, q & 1);
+    b1[q] = a;
+    e = max(e, exp_field(a));
+  }
+  const double b2 = add_updates_part(0.0, ud, h0, h1, pt);
+  const int E = block_max(e, red);                                       // publishes b1 too
+  const int kp = (k + 15) / 16 * 16;
+  for (int q = tid; q < kp; q += 128) {                                  // pair q / 2, part q & 1
+    const int p = q >> 1, j = 2 * p;
+    const double x = j < k ? b1[2 * j + (q & 1)] : 0.0, y = j + 1 < k ? b1[2 * j + 2 + (q & 1)] : 0.0;
+    put_pair(((q & 1) ? bim : bre) + p * kPairStride, to_digits(x, 1 + E - max(exp_field(x), 1)),
+             to_digits(y, 1 + E - max(exp_field(y), 1)));
+  }
+  __syncthreads();
+  float c[4][4];
+  int tot[2][4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
+    tot[0][q] = tot[1][q] = 0;
+  }
+  int it = 0;
+  for (int s = cg; s < nst; s += CG, it++) {
+    cp_async_wait<kRing - 1>();
+    const int slot = it % kRing;
+    uint4 raw[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) raw[q] = myring[slot * 256 + q * 32];
+    if (s >= nfull) {
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int j = 16 * s + 2 * t + (q & 1) + 8 * (q >> 1);
+        if (j >= ja) raw[2 * q] = zero_entry();
+        if (j >= jb) raw[2 * q + 1] = zero_entry();
+      }
+    }
+    step_single(raw, bre, bim, (8 * s + t) * kPairStride + g + 7, c);
+    issue(s + kRing * CG, slot);                                         // the slot's entries are in use above
+    if ((it & 3) == 3) flush_single(c, tot);                             // at most 64 columns per accumulator
+  }
+  flush_single(c, tot);
+  const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
+  const int64_t v2 = quad_half(tot[0][2], tot[0][3]), v3 = quad_half(tot[1][2], tot[1][3]);
+  if ((t & 1) == 0) {
+    sums[cg][mt * 16 + g][0][t >> 1] = v0;
+    sums[cg][mt * 16 + g][1][t >> 1] = v1;
+    sums[cg][mt * 16 + g + 8][0][t >> 1] = v2;
+    sums[cg][mt * 16 + g + 8][1][t >> 1] = v3;
+  }
+  __syncthreads();
+  if (tid < 2 * RT) {                                                    // whole warps
+    int64_t hi = 0, lo = 0;
+#pragma unroll
+    for (int q = 0; q < CG; q++) {
+      hi += sums[q][tid >> 1][pt][0];
+      lo += sums[q][tid >> 1][pt][1];
+    }
+    double s = scale2(halves_value(hi, lo), 88 + re + E - kBias);
+    if (E == 0x7ff || re == kRowNonFinite) s = nan("");
+    const double a = s + (mine && r < k ? b1[2 * r + pt] : 0.0);
+    const double o = __shfl_xor_sync(0xffffffffu, a, 1);                 // the other part
+    if (mine) {
+      // D^{-1} (a, o): real part dx a - dy o, imaginary part dx a + dy o (a, o swapped)
+      if (r < k)
+        reinterpret_cast<double*>(zout + S.first + r)[pt] = fma(dinv.x, a, pt ? dinv.y * o : -dinv.y * o);
+      else
+        reinterpret_cast<double*>(u + uw)[pt] = b2 - s;
+    }
+  }
+}
+
+// Backward, 32 pivot columns x one row chunk per task: sums over the chunk's rows r > j of
+// P[r][j] vec[r], vec = (z, -x[ancestor rows]), with each panel row's exponent folded into
+// vec's.  4 warps = 2 column tiles x 2 groups of 16-row steps.  A supernode of one chunk is
+// finished here, else by the last CTA of the column block (bwd_finish).
+__global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnDev* sn, const int32_t* rowlist,
+                                                    const double2* panels, const int16_t* rexp,
+                                                    const double2* zin, double2* x, double2* partial, int rows,
+                                                    int rpad, const int4* fins, unsigned int* counters) {
+  pdl_trigger();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint4* ring = reinterpret_cast<uint4*>(smem_raw);                      // 4 warps x kRing x 8 x 32
+  double* vec = reinterpret_cast<double*>(ring + 4 * kRing * 256);       // rpad x 2
+  uint32_t* vre = reinterpret_cast<uint32_t*>(vec + 2 * rpad);
+  uint32_t* vim = vre + (rpad / 2) * kPairStride;
+  int* vex = reinterpret_cast<int*>(vim + (rpad / 2) * kPairStride);     // rpad
+  __shared__ int64_t sums[2][32][2][2];                                  // [group][column][part][half]
+  __shared__ int red[4];
+  const int4 tk = tasks[blockIdx.x];
+  const SnDev S = sn[tk.x];
+  const int k = S.k, m = S.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int g = lane >> 2, t = lane & 3, ct = wid & 1, sl = wid >> 1;
+  const int r0 = tk.z * rows, r1 = min(m, r0 + rows);
+  const int j0 = tk.y * 32 + ct * 16;
+  const int ja = j0 + g, jb = ja + 8;
+  const uint4* P = reinterpret_cast<const uint4*>(panels + S.paneloff);
+  const uint4* Pa = P + int64_t(ja < k ? ja : 0) * S.ld;
+  const uint4* Pb = P + int64_t(jb < k ? jb : 0) * S.ld;
+  const int nst = (r1 - r0 + 15) / 16;
+  // steps whose rows all lie at or above the tile's first column hold nothing
+  const int sfirst = j0 < k ? max(0, (j0 + 1 - r0) / 16) : nst;
+  const bool fullcols = j0 + 15 < k;
+  uint4* myring = ring + wid * (kRing * 256) + lane;
+  auto issue = [&](int s, int slot) {
+    if (s < nst) {
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int r = r0 + 16 * s + 4 * t + q;
+        if (ja < k && r < r1 && r > ja) cp_async16(myring + slot * 256 + (2 * q) * 32, Pa + r);
+        if (jb < k && r < r1 && r > jb) cp_async16(myring + slot * 256 + (2 * q + 1) * 32, Pb + r);
+      }
+    }
+    cp_async_commit();
+  };
+  const int s0 = sfirst + ((sl - sfirst) & 1);
+#pragma unroll
+  for (int q = 0; q < kRing; q++) issue(s0 + 2 * q, q);
+  const int32_t* rl = rowlist + S.rowoff;
+  int e = -4000, bad = 0;
+  pdl_wait();
+  for (int q = tid; q < 2 * (r1 - r0); q += 128) {
+    const int r = r0 + (q >> 1), pt = q & 1;
+    const double v = r < k ? __ldcg(reinterpret_cast<const double*>(zin + S.first + r) + pt)
+                           : -__ldcg(reinterpret_cast<const double*>(x + rl[r]) + pt);
+    const int re = rexp[S.eoff + r];
+    vec[q] = v;
+    if (pt == 0) vex[q >> 1] = re;
+    const int ev = exp_field(v);
+    bad |= (ev == 0x7ff) | (re == kRowNonFinite);
+    e = max(e, max(ev, 1) + re);
+  }
+  const bool nonfinite = __syncthreads_or(bad) != 0;
+  const int E = block_max(e, red);
+  for (int q = tid; q < 16 * nst; q += 128) {
+    const int p = q >> 1, r = 2 * p, pt = q & 1;
+    double x0 = 0.0, x1 = 0.0;
+    int e0 = 0, e1 = 0;
+    if (r < r1 - r0) {
+      x0 = vec[2 * r + pt];
+      e0 = vex[r];
+    }
+    if (r + 1 < r1 - r0) {
+      x1 = vec[2 * r + 2 + pt];
+      e1 = vex[r + 1];
+    }
+    uint32_t* dst = (pt ? vim : vre) + ((p & ~7) + pair_pos_bwd(p & 7)) * kPairStride;
+    put_pair(dst, to_digits(x0, 1 + E - max(exp_field(x0), 1) - e0), to_digits(x1, 1 + E - max(exp_field(x1), 1) - e1));
+  }
+  __syncthreads();
+  float c[4][4];
+  int tot[2][4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
+    tot[0][q] = tot[1][q] = 0;
+  }
+  int it = 0;
+  for (int s = s0; s < nst; s += 2, it++) {
+    cp_async_wait<kRing - 1>();
+    const int slot = it % kRing;
+    uint4 raw[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) raw[q] = myring[slot * 256 + q * 32];
+    const int rs = r0 + 16 * s;
+    if (!fullcols || rs + 16 > r1 || rs <= j0 + 15) {
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int r = rs + 4 * t + q;
+        if (ja >= k || r >= r1 || r <= ja) raw[2 * q] = zero_entry();
+        if (jb >= k || r >= r1 || r <= jb) raw[2 * q + 1] = zero_entry();
+      }
+    }
+    step_single(raw, vre, vim, (8 * s + t) * kPairStride + g + 7, c);
+    issue(s + 2 * kRing, slot);
+    if ((it & 3) == 3) flush_single(c, tot);
+  }
+  flush_single(c, tot);
+  const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
+  const int64_t v2 = quad_half(tot[0][2], tot[0][3]), v3 = quad_half(tot[1][2], tot[1][3]);
+  if ((t & 1) == 0) {
+    sums[sl][ct * 16 + g][0][t >> 1] = v0;
+    sums[sl][ct * 16 + g][1][t >> 1] = v1;
+    sums[sl][ct * 16 + g + 8][0][t >> 1] = v2;
+    sums[sl][ct * 16 + g + 8][1][t >> 1] = v3;
+  }
+  __syncthreads();
+  const bool single = m <= rows;
+  if (tid < 64) {
+    const int j = tk.y * 32 + (tid >> 1), pt = tid & 1;
+    double s = scale2(halves_value(sums[0][tid >> 1][pt][0] + sums[1][tid >> 1][pt][0],
+                                   sums[0][tid >> 1][pt][1] + sums[1][tid >> 1][pt][1]), 88 + E - kBias);
+    if (nonfinite) s = nan("");
+    if (!single)
+      reinterpret_cast<double*>(partial)[int64_t(blockIdx.x) * 64 + tid] = s;
+    else if (j < k)
+      reinterpret_cast<double*>(x + S.first + j)[pt] = __ldcg(reinterpret_cast<const double*>(zin + S.first + j) + pt) + s;
+  }
+  if (!single) bwd_finish<double2>(fins[tk.w], S, zin, partial, x, counters + tk.w);
+}
+
+// ---------------------------------------------------------------------------
+// S right-hand sides (interleaved per row): an MMA's eight columns are the real and
+// imaginary parts of four right-hand sides, and the digit pairs (i, j) with i + j = d add up
+// in accumulator d, so 72 MMAs serve 256 entries x 4 right-hand sides (0.14 SM-clocks per
+// complex product, against 2 on the FP64 units).  Panel digits are unpacked once per warp.
+// ---------------------------------------------------------------------------
+namespace {
+
+__device__ __forceinline__ void step_multi(const uint4* raw, const uint32_t* bd, int S2, int pstride, float (*cr)[4],
+                                           float (*ci)[4]) {
+  uint32_t b[8][2];
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    b[j][0] = bd[j * S2];
+    b[j][1] = bd[4 * pstride + j * S2];
+  }
+#pragma unroll
+  for (int w = 0; w < 2; w++) {
+#pragma unroll
+    for (int part = 0; part < 2; part++) {
+      uint32_t a[4][4];
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int kp = 0; kp < 2; kp++) {
+          const uint4 x = raw[(2 * kp) * 2 + h], y = raw[(2 * kp + 1) * 2 + h];
+          uint32_t o[4];
+          if (part == 0) word_digits(w == 0 ? x.y : x.x, w == 0 ? y.y : y.x, o);
+          else word_digits(w == 0 ? x.w : x.z, w == 0 ? y.w : y.z, o);
+#pragma unroll
+          for (int d = 0; d < 4; d++) a[d][2 * kp + h] = o[d];
+        }
+#pragma unroll
+      for (int d = 0; d < 4; d++)
+#pragma unroll
+        for (int j = 0; j < 8 - (4 * w + d); j++) mma16816(part ? ci[4 * w + d + j] : cr[4 * w + d + j], a[d], b[j][0], b[j][1]);
+    }
+  }
+}
+
+// value of the weighted digit sums t[0..7] = result 2^88 2^(exponents)
+__device__ __forceinline__ double digit_value(const int* t) {
+  const int64_t hi = ((int64_t(t[0]) * 256 + t[1]) * 256 + t[2]) * 256 + t[3];
+  const int64_t lo = ((int64_t(t[4]) * 256 + t[5]) * 256 + t[6]) * 256 + t[7];
+  return fma(double(lo), 0x1p-32, double(hi));
+}
+
+// adds the accumulators of one flush to the FP64 sums: acc[h] (row half h) += this lane's
+// right-hand side; exps: right-hand side exponent + row exponents
+__device__ __forceinline__ void flush_multi(float (*cr)[4], float (*ci)[4], double2* acc, int ea, int eb) {
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    int tr[8], ti[8];
+#pragma unroll
+    for (int d = 0; d < 8; d++) {
+      tr[d] = __float2int_rn(cr[d][2 * h]) - __float2int_rn(ci[d][2 * h + 1]);
+      ti[d] = __float2int_rn(cr[d][2 * h + 1]) + __float2int_rn(ci[d][2 * h]);
+    }
+    const int sc = 88 + (h ? eb : ea);
+    acc[h].x += scale2(digit_value(tr), sc);
+    acc[h].y += scale2(digit_value(ti), sc);
+  }
+#pragma unroll
+  for (int d = 0; d < 8; d++)
+#pragma unroll
+    for (int q = 0; q < 4; q++) cr[d][q] = ci[d][q] = 0.f;
+}
+
+// Digits of a block of kb values x S right-hand sides (src: row-major kb x S, rows >= cnt are
+// zero) into bd[pair][digit][right-hand side][part]; the exponents of each right-hand side are
+// already in ex.  rowe: row exponents folded in (backward), or null.
+template <int S, bool BWD>
+__device__ __forceinline__ void put_digits_multi(uint32_t* bd, int pstride, const double2* src, int cnt, int kb,
+                                                 const int* ex, const int* rowe) {
+  for (int q = threadIdx.x; q < (kb / 2) * S * 2; q += 256) {
+    const int part = q & 1, i = (q >> 1) % S, p = (q >> 1) / S;
+    const int r = 2 * p, E = ex[i];
+    double x = 0.0, y = 0.0;
+    int e0 = 0, e1 = 0;
+    if (r < cnt) {
+      const double2 v = src[r * S + i];
+      x = part ? v.y : v.x;
+      if (BWD) e0 = rowe[r];
+    }
+    if (r + 1 < cnt) {
+      const double2 v = src[(r + 1) * S + i];
+      y = part ? v.y : v.x;
+      if (BWD) e1 = rowe[r + 1];
+    }
+    const uint64_t dx = to_digits(x, 1 + E - max(exp_field(x), 1) - e0);
+    const uint64_t dy = to_digits(y, 1 + E - max(exp_field(y), 1) - e1);
+    uint32_t* dst = bd + ((p & ~7) + (BWD ? pair_pos_bwd(p & 7) : (p & 7))) * pstride + 2 * i + part;
+    uint32_t o[4];
+    word_digits(uint32_t(dx >> 32), uint32_t(dy >> 32), o);
+#pragma unroll
+    for (int d = 0; d < 4; d++) dst[d * 2 * S] = o[d];
+    word_digits(uint32_t(dx), uint32_t(dy), o);
+#pragma unroll
+    for (int d = 0; d < 4; d++) dst[(4 + d) * 2 * S] = o[d];
+  }
+}
+
+// per right-hand side: largest exponent field (plus row exponent) of a block of values; 256
+// threads = 256 / S rows at a time, right-hand side fastest
+template <int S, bool BWD>
+__device__ __forceinline__ void block_exponents(const double2* src, int cnt, int* ex, int* nonfin, const int* rowe) {
+  const int i = threadIdx.x % S;
+  int e = BWD ? -4000 : 1, bad = 0;
+  for (int r = threadIdx.x / S; r < cnt; r += 256 / S) {
+    const double2 v = src[r * S + i];
+    const int ev = max(exp_field(v.x), exp_field(v.y));
+    bad |= ev == 0x7ff;
+    if (BWD) {
+      bad |= rowe[r] == kRowNonFinite;
+      e = max(e, max(ev, 1) + rowe[r]);
+    } else {
+      e = max(e, ev);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o >= S; o >>= 1) {
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+  }
+  if ((threadIdx.x & 31) < S) {
+    atomicMax(&ex[i], e);
+    if (bad) atomicOr(&nonfin[i], 1);
+  }
+}
+
+}  // namespace
+
+// columns (forward) or rows (backward) whose digits are in shared memory at once: 64 per
+// group of steps, so that no accumulator takes more
+template <int KG> constexpr int kMultiKb = 16 * (KG > 4 ? KG : 4);
+template <int S> constexpr int kMultiPairStride = 16 * S + 8;     // words; 8 t mod 32 differ
+
+// Forward: 16 MT rows x S right-hand sides per task; 8 warps = S / 4 groups of four
+// right-hand sides x MT row tiles x KG groups of 16-column steps.
+template <int S, int MT>
+__global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const SnDev* sn, const uint32_t* cptr,
+                                                       const uint32_t* wpos, const double2* panels,
+                                                       const int16_t* rexp, const double2* tin, double2* zout,
+                                                       double2* u, int kpad) {
+  constexpr int NT = S / 4, KG = 8 / (NT * MT), KB = kMultiKb<KG>, PS = kMultiPairStride<S>, RT = 16 * MT;
+  static_assert(NT * MT * KG == 8, "eight warps");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* b1 = reinterpret_cast<double2*>(smem_raw);                    // kpad x S
+  double2* part = b1 + kpad * S;                                          // KG x RT x S
+  uint32_t* bd = reinterpret_cast<uint32_t*>(part + KG * RT * S);        // KB / 2 x PS
+  __shared__ int ex[2][S], nonfin[S];
+  const int2 tk = tasks[blockIdx.x];
+  const SnDev Sn = sn[tk.x];
+  const int k = Sn.k, m = Sn.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int g = lane >> 2, t = lane & 3, nt = wid % NT, mt = (wid / NT) % MT, kg = wid / (NT * MT);
+  const uint32_t* cp = cptr + Sn.rowoff;
+  const int row0 = tk.y * RT + mt * 16, ra = row0 + g, rb = ra + 8;
+  const int ja = ra < m ? min(ra, k) : 0, jb = rb < m ? min(rb, k) : 0;
+  const int jend = min(min(tk.y * RT + RT - 1, m - 1), k);               // columns any row of the task needs
+  const uint4* P = reinterpret_cast<const uint4*>(panels + Sn.paneloff);
+  uint4 raw[8];
+  auto load = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int j = 16 * s + 2 * t + (q & 1) + 8 * (q >> 1);
+      const uint4* col = P + int64_t(j) * Sn.ld;
+      raw[2 * q] = j < ja ? ld_panel(col + ra) : zero_entry();
+      raw[2 * q + 1] = j < jb ? ld_panel(col + rb) : zero_entry();
+    }
+  };
+  if (tid < S) {
+    ex[0][tid] = 1;
+    nonfin[tid] = 0;
+  }
+  if (16 * kg < jend) load(kg);
+  for (int e = tid; e < k * S; e += 256) {
+    const int j = e / S, i = e % S;
+    double2 a = ldv(tin + int64_t(Sn.first + j) * S + i);
+    for (uint32_t c = cp[j]; c < cp[j + 1]; c++) a = cadd(a, ldv(u + int64_t(c) * S + i));
+    b1[e] = a;
+  }
+  float cr[8][4], ci[8][4];
+#pragma unroll
+  for (int d = 0; d < 8; d++)
+#pragma unroll
+    for (int q = 0; q < 4; q++) cr[d][q] = ci[d][q] = 0.f;
+  double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+  const int ea = ra < m ? rexp[Sn.eoff + ra] : 0, eb = rb < m ? rexp[Sn.eoff + rb] : 0;
+  const int rhs = 4 * nt + t;                                             // this lane's right-hand side
+  __syncthreads();
+  for (int j0 = 0, blk = 0; j0 < jend; j0 += KB, blk++) {
+    int* exb = ex[blk & 1];
+    block_exponents<S, false>(b1 + j0 * S, min(KB, k - j0), exb, nonfin, nullptr);
+    __syncthreads();
+    put_digits_multi<S, false>(bd, PS, b1 + j0 * S, min(KB, k - j0), KB, exb, nullptr);
+    if (tid < S) ex[(blk + 1) & 1][tid] = 1;
+    __syncthreads();
+    for (int s = j0 / 16 + kg; s < (j0 + KB) / 16 && 16 * s < jend; s += KG) {
+      step_multi(raw, bd + (8 * (s - j0 / 16) + t) * PS + 8 * nt + g, 2 * S, PS, cr, ci);
+      if (16 * (s + KG) < jend) load(s + KG);
+    }
+    flush_multi(cr, ci, acc, ea + exb[rhs] - kBias, eb + exb[rhs] - kBias);
+    __syncthreads();                                                      // bd and ex are reused
+  }
+  part[(kg * RT + mt * 16 + g) * S + rhs] = acc[0];
+  part[(kg * RT + mt * 16 + g + 8) * S + rhs] = acc[1];
+  __syncthreads();
+  for (int e = tid; e < RT * S; e += 256) {
+    const int i = e % S, r = tk.y * RT + e / S;
+    if (r >= m) continue;
+    double2 s = part[e];
+#pragma unroll
+    for (int q = 1; q < KG; q++) s = cadd(s, part[q * RT * S + e]);
+    if (nonfin[i] || rexp[Sn.eoff + r] == kRowNonFinite) s = make_double2(nan(""), nan(""));
+    if (r < k) {
+      zout[int64_t(Sn.first + r) * S + i] = cmul(panels[Sn.paneloff + r + int64_t(r) * Sn.ld], cadd(b1[r * S + i], s));
+    } else {
+      double2 b2 = make_double2(0.0, 0.0);
+      for (uint32_t c = cp[r]; c < cp[r + 1]; c++) b2 = cadd(b2, ldv(u + int64_t(c) * S + i));
+      u[int64_t(wpos[Sn.uoff + (r - k)]) * S + i] = csub(b2, s);
+    }
+  }
+}
+
+// Backward: 32 pivot columns x S right-hand sides x one chunk of kMultiBwdRows rows per task.
+template <int S>
+__global__ void __launch_bounds__(256) k_bwd_dig_multi(const int4* tasks, const SnDev* sn, const int32_t* rowlist,
+                                                       const double2* panels, const int16_t* rexp,
+                                                       const double2* zin, double2* x, double2* partial,
+                                                       const int4* fins, unsigned int* counters) {
+  constexpr int NT = S / 4, KG = 4 / NT, KB = 64, PS = kMultiPairStride<S>, ROWS = kMultiBwdRows;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* vec = reinterpret_cast<double2*>(smem_raw);                   // ROWS x S; then KG x 32 x S partial sums
+  uint32_t* bd = reinterpret_cast<uint32_t*>(vec + ROWS * S);            // KB / 2 x PS
+  __shared__ int ex[2][S], nonfin[S], vex[ROWS];
+  __shared__ unsigned int ticket;
+  const int4 tk = tasks[blockIdx.x];
+  const SnDev Sn = sn[tk.x];
+  const int k = Sn.k, m = Sn.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int g = lane >> 2, t = lane & 3, nt = wid % NT, ct = (wid / NT) & 1, kg = wid / (2 * NT);
+  const int r0 = tk.z * ROWS, r1 = min(m, r0 + ROWS), cnt = r1 - r0;
+  const int j0 = tk.y * 32 + ct * 16, ja = j0 + g, jb = ja + 8;
+  const uint4* P = reinterpret_cast<const uint4*>(panels + Sn.paneloff);
+  const uint4* Pa = P + int64_t(ja < k ? ja : 0) * Sn.ld;
+  const uint4* Pb = P + int64_t(jb < k ? jb : 0) * Sn.ld;
+  const int nst = (cnt + 15) / 16;
+  uint4 raw[8];
+  auto load = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int r = r0 + 16 * s + 4 * t + q;
+      raw[2 * q] = (ja < k && r < r1 && r > ja) ? ld_panel(Pa + r) : zero_entry();
+      raw[2 * q + 1] = (jb < k && r < r1 && r > jb) ? ld_panel(Pb + r) : zero_entry();
+    }
+  };
+  if (tid < S) {
+    ex[0][tid] = -4000;
+    nonfin[tid] = 0;
+  }
+  if (kg < nst) load(kg);
+  const int32_t* rl = rowlist + Sn.rowoff;
+  for (int r = tid; r < cnt; r += 256) vex[r] = rexp[Sn.eoff + r0 + r];
+  for (int e = tid; e < cnt * S; e += 256) {
+    const int r = r0 + e / S, i = e % S;
+    vec[e] = r < k ? ldv(zin + int64_t(Sn.first + r) * S + i) : cneg(ldv(x + int64_t(rl[r]) * S + i));
+  }
+  float cr[8][4], ci[8][4];
+#pragma unroll
+  for (int d = 0; d < 8; d++)
+#pragma unroll
+    for (int q = 0; q < 4; q++) cr[d][q] = ci[d][q] = 0.f;
+  double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+  const int rhs = 4 * nt + t;
+  __syncthreads();
+  for (int q0 = 0, blk = 0; q0 < cnt; q0 += KB, blk++) {
+    int* exb = ex[blk & 1];
+    const int nr = min(KB, cnt - q0);
+    block_exponents<S, true>(vec + q0 * S, nr, exb, nonfin, vex + q0);
+    __syncthreads();
+    put_digits_multi<S, true>(bd, PS, vec + q0 * S, nr, KB, exb, vex + q0);
+    if (tid < S) ex[(blk + 1) & 1][tid] = -4000;
+    __syncthreads();
+    for (int s = q0 / 16 + kg; s < (q0 + KB) / 16 && s < nst; s += KG) {
+      step_multi(raw, bd + (8 * (s - q0 / 16) + t) * PS + 8 * nt + g, 2 * S, PS, cr, ci);
+      if (s + KG < nst) load(s + KG);
+    }
+    flush_multi(cr, ci, acc, exb[rhs] - kBias, exb[rhs] - kBias);
+    __syncthreads();
+  }
+  vec[(kg * 32 + ct * 16 + g) * S + rhs] = acc[0];
+  vec[(kg * 32 + ct * 16 + g + 8) * S + rhs] = acc[1];
+  __syncthreads();
+  const bool single = m <= ROWS;
+  double2* out = partial + int64_t(blockIdx.x) * 32 * S;
+  for (int e = tid; e < 32 * S; e += 256) {
+    double2 s = vec[e];
+#pragma unroll
+    for (int q = 1; q < KG; q++) s = cadd(s, vec[q * 32 * S + e]);
+    if (nonfin[e % S]) s = make_double2(nan(""), nan(""));
+    const int j = tk.y * 32 + e / S;
+    if (!single)
+      out[e] = s;
+    else if (j < k)
+      x[int64_t(Sn.first + j) * S + e % S] = cadd(ldv(zin + int64_t(Sn.first + j) * S + e % S), s);
+  }
+  if (single) return;
+  // last CTA of the column block: partials in chunk order (no CTA waits on another)
+  const int4 fin = fins[tk.w];
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) ticket = atomicAdd(counters + tk.w, 1u);
+  __syncthreads();
+  if (ticket != unsigned(fin.w) - 1) return;
+  __threadfence();
+  for (int e = tid; e < 32 * S; e += 256) {
+    const int j = fin.y * 32 + e / S;
+    if (j >= k) continue;
+    double2 a = make_double2(0.0, 0.0);
+    for (int ch = 0; ch < fin.w; ch++) a = cadd(a, ldv(partial + int64_t(fin.z + ch) * 32 * S + e));
+    x[int64_t(Sn.first + j) * S + e % S] = cadd(ldv(zin + int64_t(Sn.first + j) * S + e % S), a);
+  }
+  if (tid == 0) counters[tk.w] = 0u;
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr size_t kRingBytes = size_t(4) * kRing * 256 * 16;
+size_t fwd_smem(int kpad) { return kRingBytes + size_t(kpad) * 16 + size_t(kpad) * kPairStride * 4; }
+size_t bwd_smem(int rpad) { return kRingBytes + size_t(rpad) * 20 + size_t(rpad) * kPairStride * 4; }
+template <int S, int MT> size_t fwd_multi_smem(int kpad) {
+  constexpr int KG = 8 / (S / 4 * MT);
+  return size_t(kpad) * S * 16 + size_t(KG) * 16 * MT * S * 16 + size_t(kMultiKb<KG> / 2) * kMultiPairStride<S> * 4;
+}
+template <int S> size_t bwd_multi_smem() {
+  return size_t(kMultiBwdRows) * S * 16 + size_t(32) * kMultiPairStride<S> * 4;
+}
+template <typename K> void allow_smem(K kern) {
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+}
+void set_attrs_dig() {
+  static const bool done = [] {
+    allow_smem(k_fwd_dig<1>);
+    allow_smem(k_fwd_dig<4>);
+    allow_smem(k_bwd_dig);
+    allow_smem(k_fwd_dig_multi<4, 1>);
+    allow_smem(k_fwd_dig_multi<4, 4>);
+    allow_smem(k_fwd_dig_multi<8, 1>);
+    allow_smem(k_fwd_dig_multi<8, 4>);
+    allow_smem(k_fwd_dig_multi<16, 1>);
+    allow_smem(k_fwd_dig_multi<16, 2>);
+    allow_smem(k_bwd_dig_multi<4>);
+    allow_smem(k_bwd_dig_multi<8>);
+    allow_smem(k_bwd_dig_multi<16>);
+    return true;
+  }();
+  (void)done;
+}
+
+}  // namespace
+
+void launch_to_digits(const FactorDev& F, cudaStream_t st) {
+  for (int l = 0; l < F.snlev; l++) {
+    const int64_t b = F.h_fwd_ptr[l], e = F.h_fwd_ptr[l + 1];
+    if (e == b) continue;
+    add_launches(1);
+    if (F.h_fwd_rt[l] == 16)
+      k_to_digits<16><<<unsigned(e - b), 256, 0, st>>>(F.fwd_tasks + b, F.ssn, (double2*)F.panels, F.rexp);
+    else
+      k_to_digits<64><<<unsigned(e - b), 256, 0, st>>>(F.fwd_tasks + b, F.ssn, (double2*)F.panels, F.rexp);
+  }
+}
+
+void launch_solve_dig(const FactorDev& F, cudaStream_t st) {
+  set_attrs_dig();
+  const double2* P = (const double2*)F.panels;
+  double2 *t = (double2*)F.t_loc, *z = (double2*)F.z_loc, *x = (double2*)F.x_loc, *u = (double2*)F.u_ws;
+  const bool pdl = pdl_enabled();
+  if (F.level_events) cudaEventRecord(F.level_events[0], st);
+  for (int l = 0; l < F.snlev; l++) {
+    const int64_t b = F.h_fwd_ptr[l], e = F.h_fwd_ptr[l + 1];
+    if (e > b) {
+      add_launches(1);
+      const int kpad = F.h_lev_k[l];
+      if (F.h_fwd_rt[l] == 16)
+        launch_level(k_fwd_dig<1>, e - b, 128, fwd_smem(kpad), st, pdl, F.fwd_tasks + b, F.ssn, F.cptr, F.wpos, P,
+                     F.rexp, t, z, u, kpad);
+      else
+        launch_level(k_fwd_dig<4>, e - b, 128, fwd_smem(kpad), st, pdl, F.fwd_tasks + b, F.ssn, F.cptr, F.wpos, P,
+                     F.rexp, t, z, u, kpad);
+    }
+    if (F.level_events) cudaEventRecord(F.level_events[1 + l], st);
+  }
+  for (int l = F.snlev - 1; l >= 0; l--) {
+    const int64_t b = F.h_bwd_ptr[l], e = F.h_bwd_ptr[l + 1];
+    if (e > b) {
+      add_launches(1);
+      const int rows = F.h_bwd_rows[l], rpad = (std::min(rows, F.h_lev_m[l]) + 15) / 16 * 16;
+      launch_level(k_bwd_dig, e - b, 128, bwd_smem(rpad), st, pdl, F.bwd_tasks + b, F.ssn, F.rowlist, P, F.rexp, z, x,
+                   (double2*)F.bwd_partial, rows, rpad, F.bfin_tasks, F.bwd_counters);
+    }
+    if (F.level_events) cudaEventRecord(F.level_events[1 + F.snlev + (F.snlev - 1 - l)], st);
+  }
+}
+
+template <int S, int MT>
+static void fwd_multi_level(const FactorDev& F, int l, int64_t b, int64_t e, cudaStream_t st) {
+  const int kpad = F.h_lev_k[l];
+  k_fwd_dig_multi<S, MT><<<unsigned(e - b), 256, fwd_multi_smem<S, MT>(kpad), st>>>(
+      F.mfwd_tasks + b, F.ssn, F.cptr, F.wpos, (const double2*)F.panels, F.rexp, (const double2*)F.mt_loc,
+      (double2*)F.mz_loc, (double2*)F.mu_ws, kpad);
+}
+
+template <int S>
+static void solve_dig_multi_t(const FactorDev& F, cudaStream_t st) {
+  constexpr int MTW = S == 16 ? 2 : 4;
+  for (int l = 0; l < F.snlev; l++) {
+    const int64_t b = F.h_mfwd_ptr[l], e = F.h_mfwd_ptr[l + 1];
+    if (e == b) continue;
+    add_launches(1);
+    if (F.h_mfwd_rt[l] == 16) fwd_multi_level<S, 1>(F, l, b, e, st);
+    else fwd_multi_level<S, MTW>(F, l, b, e, st);
+  }
+  for (int l = F.snlev - 1; l >= 0; l--) {
+    const int64_t b = F.h_mbwd_ptr[l], e = F.h_mbwd_ptr[l + 1];
+    if (e == b) continue;
+    add_launches(1);
+    k_bwd_dig_multi<S><<<unsigned(e - b), 256, bwd_multi_smem<S>(), st>>>(
+        F.mbwd_tasks + b, F.ssn, F.rowlist, (const double2*)F.panels, F.rexp, (const double2*)F.mz_loc,
+        (double2*)F.mx_loc, (double2*)F.mbwd_partial, F.mbfin_tasks, F.mbwd_counters);
+  }
+}
+
+void launch_solve_dig_multi(const FactorDev& F, int S, cudaStream_t st) {
+  set_attrs_dig();
+  if (S == 4) solve_dig_multi_t<4>(F, st);
+  else if (S == 8) solve_dig_multi_t<8>(F, st);
+  else solve_dig_multi_t<16>(F, st);
+}
+
+}  // namespace hz
