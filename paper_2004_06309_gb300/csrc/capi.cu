@@ -645,6 +645,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
   F.v_tc_multi = spf.tc_multi;
   F.v_tc_kstages = spf.tc_kstages;
   F.v_max_k = spf.max_k;
+  F.h_flev_k.assign(size_t(nlev), 1);
   for (int l = 0; l < nlev; l++) {
     lev_ptr[l] = S.lev_ptr[l];
     wg_ptr[l] = int64_t(wg.size());
@@ -657,6 +658,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
     for (int32_t q = S.lev_ptr[l]; q < S.lev_ptr[l + 1]; q++) {
       const int s = S.lev_sn[q];
       const int k = S.sn_k[s], m = S.sn_m[s], r = m - k;
+      F.h_flev_k[size_t(l)] = std::max(F.h_flev_k[size_t(l)], k);
       const int gs = grp_of(s);
       if (gs != cur_g) {                           // a group's W blocks start the scratch again
         cur_g = gs;

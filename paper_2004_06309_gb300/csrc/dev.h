@@ -98,6 +98,7 @@ struct FactorDev {
   // per solve level: widest supernode (rounded up to 16 columns), tallest one, and the rows
   // of the batched forward tasks
   std::vector<int> h_lev_k, h_lev_m, h_mfwd_rt;
+  std::vector<int> h_flev_k;          // per factor level: widest supernode
   int32_t max_slot = 0;
   // kernel variants of the schedule (host-side counts, reported through hz_stats)
   int32_t v_fwd_wide = 0, v_fwd_narrow = 0, v_bwd_wide = 0, v_bwd_narrow = 0;
@@ -190,6 +191,10 @@ void launch_fill_values(int64_t nnz, const double* K, const double2* M, const do
 // children, factor, and copy the panels to the factor store.
 void launch_factor_level(const FactorDev& F, int lev, int grp, double w, void* fronts, void* scratch,
                          DevStatus* status, double tiny, cudaStream_t st);
+
+// Pivot blocks of one level (diag.cu): F11 = L D L^T, T = L^{-1} in place, D^{-1} on the diagonal.
+void launch_diag(int precision, int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, void* fronts,
+                 DevStatus* status, double tiny, cudaStream_t st);
 
 void launch_gather(const FactorDev& F, const double2* src, cudaStream_t st);
 void launch_solve(const FactorDev& F, cudaStream_t st);

@@ -92,63 +92,6 @@ __global__ void __launch_bounds__(256) k_extend_add(const int2* tasks, const SnD
   }
 }
 
-__device__ __forceinline__ void record_pivot(DevStatus* st, double mag, double tiny) {
-  unsigned long long bits = __double_as_longlong(mag);
-  atomicMin(reinterpret_cast<unsigned long long*>(&st->min_pivot), bits);
-  if (!(mag >= tiny)) atomicOr(&st->zero_pivot, 1u);
-}
-
-// Pivot block: F11 = L D L^T in shared memory, then T = L^{-1} (unit lower) in
-// place; the front keeps T below the diagonal and D^{-1} on it.
-template <typename V>
-__global__ void __launch_bounds__(256) k_diag(const int32_t* lev_sn, const SnDev* sn, V* fronts,
-                                              DevStatus* status, double tiny) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* A = reinterpret_cast<V*>(smem_raw);
-  const SnDev S = sn[lev_sn[blockIdx.x]];
-  const int k = S.k, m = S.m, ld = k + 1;
-  V* dinv = A + ld * k;
-  V* row = dinv + k;
-  V* F = fronts + S.frontoff;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  for (int e = tid; e < k * k; e += blockDim.x) {
-    const int i = e % k, j = e / k;
-    A[i + j * ld] = (i >= j) ? F[i + int64_t(j) * m] : czero<V>();
-  }
-  __syncthreads();
-  for (int j = 0; j < k; j++) {
-    const V d = A[j + j * ld];
-    const V di = cinv(d);
-    if (tid == 0) {
-      dinv[j] = di;
-      record_pivot(status, sqrt(double(d.x) * double(d.x) + double(d.y) * double(d.y)), tiny);
-    }
-    for (int c = j + 1 + wid; c < k; c += 8) {
-      const V lc = cmul(A[c + j * ld], di);
-      for (int i = c + lane; i < k; i += 32) A[i + c * ld] = cmsub(A[i + j * ld], lc, A[i + c * ld]);
-    }
-    __syncthreads();
-    for (int i = j + 1 + tid; i < k; i += blockDim.x) A[i + j * ld] = cmul(A[i + j * ld], di);
-    __syncthreads();
-  }
-  // T = L^{-1}, row by row: T[i][j] = -(L[i][j] + sum_{j<l<i} L[i][l] T[l][j])
-  for (int i = 1; i < k; i++) {
-    for (int l = tid; l < i; l += blockDim.x) row[l] = A[i + l * ld];
-    __syncthreads();
-    for (int j = tid; j < i; j += blockDim.x) {
-      V acc = row[j];
-      for (int l = j + 1; l < i; l++) acc = cmad(row[l], A[l + j * ld], acc);
-      A[i + j * ld] = cneg(acc);
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < k * k; e += blockDim.x) {
-    const int i = e % k, j = e / k;
-    if (i > j) F[i + int64_t(j) * m] = A[i + j * ld];
-    else if (i == j) F[i + int64_t(j) * m] = dinv[j];
-  }
-}
-
 // Off-diagonal block, 32 rows per task:
 //   W = F21 T^T  (= L21 D), saved to the level scratch for the Schur update,
 //   G = W D^{-1} T  (= F21 F11^{-1} = L21 L11^{-1}), written over F21.
@@ -466,27 +409,38 @@ __global__ void __launch_bounds__(256) k_cb_tc(const int4* tasks, const SnDev* s
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(256));
 }
 
+// Zeroes the lower triangles of a level's fronts (nothing reads above them).  grid.y CTAs
+// share a front's columns, one column per warp at a time: bound by writing the fronts, and a
+// single CTA per front left the top levels' few tall fronts to a few SMs (28 -> 2 ms per
+// factorisation of the 349,461-dof survey model, both precisions' factors).
 template <typename V>
-__global__ void k_front_zero(const int32_t* lev_sn, const SnDev* sn, V* fronts) {
+__global__ void __launch_bounds__(256) k_front_zero(const int32_t* lev_sn, const SnDev* sn, V* fronts) {
   const SnDev S = sn[lev_sn[blockIdx.x]];
-  const int64_t cnt = int64_t(S.m) * S.m;
   V* f = fronts + S.frontoff;
-  for (int64_t e = threadIdx.x; e < cnt; e += blockDim.x) f[e] = czero<V>();
+  for (int j = blockIdx.y * 8 + (threadIdx.x >> 5); j < S.m; j += 8 * gridDim.y)
+    for (int r = j + (threadIdx.x & 31); r < S.m; r += 32) f[int64_t(j) * S.m + r] = czero<V>();
 }
 
+// Copies a level's panels from the fronts to the factor store (grid as above); padding rows
+// are zero.
 template <typename V>
-__global__ void k_panel_copy(const int32_t* lev_sn, const SnDev* sn, const V* fronts, V* panels) {
+__global__ void __launch_bounds__(256) k_panel_copy(const int32_t* lev_sn, const SnDev* sn, const V* fronts,
+                                                    V* panels) {
   const SnDev S = sn[lev_sn[blockIdx.x]];
-  const int64_t cnt = int64_t(S.ld) * S.k;
   const V* src = fronts + S.frontoff;
   V* dst = panels + S.paneloff;
-  for (int64_t e = threadIdx.x; e < cnt; e += blockDim.x) {
-    const int64_t j = e / S.ld, r = e % S.ld;
-    dst[e] = (r < S.m) ? src[r + j * S.m] : czero<V>();    // padding rows are zero
-  }
+  for (int j = blockIdx.y * 8 + (threadIdx.x >> 5); j < S.k; j += 8 * gridDim.y)
+    for (int r = threadIdx.x & 31; r < S.ld; r += 32)
+      dst[int64_t(j) * S.ld + r] = (r >= j && r < S.m) ? src[int64_t(j) * S.m + r] : czero<V>();
 }
 
-static size_t diag_smem(int kmax, size_t vs) { return (size_t(kmax + 1) * kmax + 2 * kmax) * vs; }
+// CTAs per supernode of a level, so that its columns (8 per CTA at a time) and the whole level
+// fill the GPU about twice over
+static unsigned split_for(int64_t nb, int64_t cols) {
+  const int64_t want = std::max<int64_t>(1, 152 * 16 / std::max<int64_t>(nb, 1));
+  return unsigned(std::max<int64_t>(1, std::min(want, (cols + 7) / 8)));
+}
+
 static size_t wg_smem(int kmax, size_t vs) { return (size_t(64) * kmax + kmax) * vs; }
 
 // One tree level of one factorisation group (whole matrices whose fronts share the
@@ -505,7 +459,7 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
   const int32_t* lsn = F.lev_sn + lb;
   if (nb > 0) {
     HZ_COUNT();
-    k_front_zero<V><<<unsigned(nb), 256, 0, st>>>(lsn, F.sn, fronts);
+    k_front_zero<V><<<dim3(unsigned(nb), split_for(nb, F.maxm)), 256, 0, st>>>(lsn, F.sn, fronts);
   }
   int64_t e0, e1;
   range(F.h_ent_g, lev, e0, e1);
@@ -524,14 +478,13 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
     }
   }
   if (nb == 0) return;
-  const size_t ds = diag_smem(F.maxk, sizeof(V));
-  HZ_COUNT();
-  k_diag<V><<<unsigned(nb), 256, ds, st>>>(lsn, F.sn, fronts, status, tiny);
+  const int maxk = F.h_flev_k[size_t(lev)];
+  launch_diag(F.precision, nb, maxk, lsn, F.sn, fronts, status, tiny, st);
   int64_t wb, we;
   range(F.h_wg_g, lev, wb, we);
   if (we > wb) {
     HZ_COUNT();
-    k_wg<V><<<unsigned(we - wb), 256, wg_smem(F.maxk, sizeof(V)), st>>>(F.wg_tasks + wb, F.sn, F.scr_off, fronts,
+    k_wg<V><<<unsigned(we - wb), 256, wg_smem(maxk, sizeof(V)), st>>>(F.wg_tasks + wb, F.sn, F.scr_off, fronts,
                                                                        scratch);
   }
   if constexpr (sizeof(V) == 8) {
@@ -551,7 +504,7 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
     }
   }
   HZ_COUNT();
-  k_panel_copy<V><<<unsigned(nb), 256, 0, st>>>(lsn, F.sn, fronts, (V*)F.panels);
+  k_panel_copy<V><<<dim3(unsigned(nb), split_for(nb, maxk)), 256, 0, st>>>(lsn, F.sn, fronts, (V*)F.panels);
 }
 
 static bool g_attr_done[2] = {false, false};
@@ -559,10 +512,8 @@ static void set_attrs(int prec, int kmax) {
   if (g_attr_done[prec]) return;
   const int lim = 227 * 1024;
   if (prec == 0) {
-    cudaFuncSetAttribute(k_diag<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_wg<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   } else {
-    cudaFuncSetAttribute(k_diag<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_cb_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemFloats * int(sizeof(float)));
     cudaFuncSetAttribute(k_wg<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   }

@@ -29,62 +29,17 @@
 #include <algorithm>
 
 #include "dev.h"
+#include "digits.cuh"
 #include "dmath.cuh"
 
 namespace hz {
 
 namespace {
 
-constexpr int kBias = 1084;               // D = x 2^(kBias - E)
 constexpr int16_t kRowNonFinite = 0x7fff;
-constexpr uint64_t kDigitBias = 0x8080808080808080ull;
-constexpr uint32_t kZeroWord = 0x80808080u;
 constexpr int kPairStride = 24;           // words per column pair of a digit vector (15 used; 24 t mod 32 differ)
 
-__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// digits (with 128 added to each) of x, with x < 2^(E - 1022) for the largest exponent field E
-// of its group; sh = 1 + E - max(exponent field of x, 1)
-__device__ __forceinline__ uint64_t to_digits(double x, int sh) {
-  const int hi = __double2hiint(x);
-  const uint32_t top = (uint32_t(hi) & 0xfffffu) | (((hi >> 20) & 0x7ff) ? 0x100000u : 0u);
-  const uint64_t m = ((uint64_t(top) << 32) | uint32_t(__double2loint(x))) << 10;
-  const uint64_t d = m >> min(sh, 63);
-  return (hi < 0 ? ~d + 1 : d) + kDigitBias;
-}
-
-// 2^e s for a result s of a digit product sum
-__device__ __forceinline__ double scale2(double s, int e) {
-  if (e >= -1000 && e <= 1000) return s * __hiloint2double((e + 1023) << 20, 0);
-  return scalbn(s, e);
-}
-
-__device__ __forceinline__ uint32_t h2sub(uint32_t a) {      // half2 (1024 + b) -> b - 128
-  const __half2 c = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));
-  __half2 v = *reinterpret_cast<__half2*>(&a);
-  v = __hsub2(v, c);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
-
-// the four digits of two 32-bit digit words as half2 (x's digit, y's digit), most significant first
-__device__ __forceinline__ void word_digits(uint32_t x, uint32_t y, uint32_t* out) {
-  const uint32_t p = __byte_perm(x, y, 0x5140), q = __byte_perm(x, y, 0x7362);
-  out[0] = h2sub(__byte_perm(q, 0x64646464u, 0x4342));
-  out[1] = h2sub(__byte_perm(q, 0x64646464u, 0x4140));
-  out[2] = h2sub(__byte_perm(p, 0x64646464u, 0x4342));
-  out[3] = h2sub(__byte_perm(p, 0x64646464u, 0x4140));
-}
-
-__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-               "{%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 __device__ __forceinline__ uint4 ld_panel(const uint4* p) { return __ldg(p); }
-__device__ __forceinline__ uint4 zero_entry() { return make_uint4(kZeroWord, kZeroWord, kZeroWord, kZeroWord); }
-
 // Position of column pair p of a 16-column step in a digit vector: fragment register b0 reads
 // pairs at positions 0-3, b1 at 4-7.  forward: pairs (2t, 2t + 1) and (2t + 8, 2t + 9) as they
 // come; backward: lane t holds four consecutive rows, pairs 2t and 2t + 1.
@@ -486,72 +441,10 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
 }
 
 // ---------------------------------------------------------------------------
-// S right-hand sides (interleaved per row): an MMA's eight columns are the real and
-// imaginary parts of four right-hand sides, and the digit pairs (i, j) with i + j = d add up
-// in accumulator d, so 72 MMAs serve 256 entries x 4 right-hand sides (0.14 SM-clocks per
-// complex product, against 2 on the FP64 units).  Panel digits are unpacked once per warp.
+// S right-hand sides (interleaved per row): step_multi, four right-hand sides per warp.  Panel
+// digits are unpacked once per warp.
 // ---------------------------------------------------------------------------
 namespace {
-
-__device__ __forceinline__ void step_multi(const uint4* raw, const uint32_t* bd, int S2, int pstride, float (*cr)[4],
-                                           float (*ci)[4]) {
-  uint32_t b[8][2];
-#pragma unroll
-  for (int j = 0; j < 8; j++) {
-    b[j][0] = bd[j * S2];
-    b[j][1] = bd[4 * pstride + j * S2];
-  }
-#pragma unroll
-  for (int w = 0; w < 2; w++) {
-#pragma unroll
-    for (int part = 0; part < 2; part++) {
-      uint32_t a[4][4];
-#pragma unroll
-      for (int h = 0; h < 2; h++)
-#pragma unroll
-        for (int kp = 0; kp < 2; kp++) {
-          const uint4 x = raw[(2 * kp) * 2 + h], y = raw[(2 * kp + 1) * 2 + h];
-          uint32_t o[4];
-          if (part == 0) word_digits(w == 0 ? x.y : x.x, w == 0 ? y.y : y.x, o);
-          else word_digits(w == 0 ? x.w : x.z, w == 0 ? y.w : y.z, o);
-#pragma unroll
-          for (int d = 0; d < 4; d++) a[d][2 * kp + h] = o[d];
-        }
-#pragma unroll
-      for (int d = 0; d < 4; d++)
-#pragma unroll
-        for (int j = 0; j < 8 - (4 * w + d); j++) mma16816(part ? ci[4 * w + d + j] : cr[4 * w + d + j], a[d], b[j][0], b[j][1]);
-    }
-  }
-}
-
-// value of the weighted digit sums t[0..7] = result 2^88 2^(exponents)
-__device__ __forceinline__ double digit_value(const int* t) {
-  const int64_t hi = ((int64_t(t[0]) * 256 + t[1]) * 256 + t[2]) * 256 + t[3];
-  const int64_t lo = ((int64_t(t[4]) * 256 + t[5]) * 256 + t[6]) * 256 + t[7];
-  return fma(double(lo), 0x1p-32, double(hi));
-}
-
-// adds the accumulators of one flush to the FP64 sums: acc[h] (row half h) += this lane's
-// right-hand side; exps: right-hand side exponent + row exponents
-__device__ __forceinline__ void flush_multi(float (*cr)[4], float (*ci)[4], double2* acc, int ea, int eb) {
-#pragma unroll
-  for (int h = 0; h < 2; h++) {
-    int tr[8], ti[8];
-#pragma unroll
-    for (int d = 0; d < 8; d++) {
-      tr[d] = __float2int_rn(cr[d][2 * h]) - __float2int_rn(ci[d][2 * h + 1]);
-      ti[d] = __float2int_rn(cr[d][2 * h + 1]) + __float2int_rn(ci[d][2 * h]);
-    }
-    const int sc = 88 + (h ? eb : ea);
-    acc[h].x += scale2(digit_value(tr), sc);
-    acc[h].y += scale2(digit_value(ti), sc);
-  }
-#pragma unroll
-  for (int d = 0; d < 8; d++)
-#pragma unroll
-    for (int q = 0; q < 4; q++) cr[d][q] = ci[d][q] = 0.f;
-}
 
 // Digits of a block of kb values x S right-hand sides (src: row-major kb x S, rows >= cnt are
 // zero) into bd[pair][digit][right-hand side][part]; the exponents of each right-hand side are
