@@ -670,16 +670,15 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
       }
       for (int rb = 0; rb * 32 < r; rb++) wg.push_back(make_int2(s, rb));
       if (precision == 0) {
-        const int T = (r + 31) / 32;
-        for (int ti = 0; ti < T; ti++)
-          for (int tj = 0; tj <= ti; tj++) cbt.push_back(make_int4(s, ti, tj, 0));
+        for (int ti = 0; ti * hz::kCbRows < r; ti++)       // column tiles that reach the row block's last row
+          for (int tj = 0; tj * 16 < std::min(r, (ti + 1) * hz::kCbRows); tj++) cbt.push_back(make_int4(s, ti, tj, 0));
       } else {
         const int T = (r + 127) / 128;
         for (int ti = 0; ti < T; ti++)
           for (int tj = 0; tj <= ti; tj++) tct.push_back(make_int4(s, ti, tj, 0));
       }
       scr_off[s] = lev_scr;
-      lev_scr += int64_t(r) * k;
+      lev_scr += int64_t(r) * (precision == 0 ? k + 1 : k);   // complex128: and a row's exponents
       scratch = std::max(scratch, lev_scr);
     }
     sl.finish(S.lev_ptr[l + 1]);

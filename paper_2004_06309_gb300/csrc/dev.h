@@ -11,6 +11,7 @@ namespace hz {
 constexpr int kMaxSolveK = 448;
 constexpr int kMaxSolveK64 = 512;   // the same for the complex64 sweeps
 constexpr int kMultiBwdRows = 128;  // rows per backward task of the batched sweeps
+constexpr int kCbRows = 128;        // rows per complex128 Schur update task (of 16 columns)
 
 // One supernode of a batched multifrontal factorisation (64 bytes).
 
@@ -74,7 +75,7 @@ struct FactorDev {
   void* bwd_partial = nullptr;   // 32 values per backward partial task (max over levels)
   int2* ea_tasks = nullptr;      // (child sn, col block)
   int2* wg_tasks = nullptr;      // (sn, row block of the off-diagonal part)
-  int4* cb_tasks = nullptr;      // (sn, row tile, col tile, scratch-relative offset unused)
+  int4* cb_tasks = nullptr;      // complex128: (sn, kCbRows-row block, 16-col tile, 0)
   int4* tc_tasks = nullptr;      // complex64 path: (sn, 128-row tile, 128-col tile, 0), tensor-core Schur update
   int64_t* h_tc_ptr = nullptr;   // nlev + 1 (host)
   int64_t* scr_off = nullptr;    // per supernode: offset of its W block in the level scratch
@@ -195,6 +196,14 @@ void launch_factor_level(const FactorDev& F, int lev, int grp, double w, void* f
 // Pivot blocks of one level (diag.cu): F11 = L D L^T, T = L^{-1} in place, D^{-1} on the diagonal.
 void launch_diag(int precision, int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, void* fronts,
                  DevStatus* status, double tiny, cudaStream_t st);
+
+// Complex128 products of one factor level and of the merged solve panels (factor64.cu).
+void launch_wg_dig(int64_t ntask, int maxk, const int2* tasks, const FactorDev& F, double2* fronts, double2* scratch,
+                   DevStatus* status, cudaStream_t st);
+void launch_cb_dig(int64_t ntask, int maxk, const int4* tasks, const FactorDev& F, double2* fronts,
+                   const double2* scratch, cudaStream_t st);
+void launch_merge_dig(double2* M, int ldm, int w, const double2* Ps, int lds, int ks, int ms, const double2* tmp,
+                      cudaStream_t st);
 
 void launch_gather(const FactorDev& F, const double2* src, cudaStream_t st);
 void launch_solve(const FactorDev& F, cudaStream_t st);

@@ -6,8 +6,9 @@
 //     S(J') = sum_q L(J, q) T(q, J') for every J' < J: one product with L's block row J, nbk
 //     tiles of 16 rows whatever J is;
 //   * factors the 16 x 16 block and inverts its unit lower factor in the same 16 pivots;
-//   * applies T(J, J): W(I, J) = A(I, J) T(J, J)^T and T(J, J') = -T(J, J) S(J').  T's row J
-//     overwrites W's, which is not needed any more.
+//   * W(I, J) = A(I, J) L(J, J)^{-T} and T(J, J') = -L(J, J)^{-1} S(J'), a product with T(J, J) in
+//     complex128, by substitution in complex64.  T's row J overwrites W's, which is not needed
+//     any more.
 // The unblocked loop (a barrier pair per column and per row of the inverse) took 1.36 ms per
 // level in complex128 (width 112) and 0.61 ms in complex64 (width 128).  A complex128 product is
 // 4 FP64 instructions of 64 clocks per scheduler, whatever its active lanes, so the block
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
   __shared__ V dinv[16 * kMaxNbk], dval[16 * kMaxNbk];
   __shared__ V wcol2[2][16], lcol2[2][16], trow2[2][16];   // by the pivot's parity
   __shared__ V dcur;
+  __shared__ V ljj[dbl ? 1 : 256];                         // L(J, J), column-major
   __shared__ int aexp[16 * kMaxNbk], bexp[2][16];
   const SnDev S = sn[lev_sn[blockIdx.x]];
   const int k = S.k, m = S.m, nbk = (k + 15) / 16;
@@ -266,7 +268,10 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
         __syncthreads();
         const V di = dcur;
         if (tid == 64) dinv[16 * J + j] = di;
-        if (tid < 16 && i > j) lcol[i] = cmul(wcol[i], di);
+        if (tid < 16 && i > j) {
+          lcol[i] = cmul(wcol[i], di);
+          if constexpr (!dbl) ljj[16 * j + i] = lcol[i];
+        }
         __syncthreads();
         if (i > j) {
           if (c <= j) tv = cmsub(lcol[i], trow[c], tv);
@@ -342,25 +347,25 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
         }
       }
     } else {
-      if (wid < nbk && wid != J) {
-        const int a = wid, r = lane & 15, h = lane >> 4;
-        V* src = a > J ? blk(a, J) : Sb + a * BLK;
-        V acc[8];
+      // by substitution with L(J, J), one thread per vector: multiplying by the inverse instead
+      // raised the error of the complex64 factors by 6 %
+      if (tid < 16 * nbk && (tid >> 4) != J) {
+        const int a = tid >> 4, r = tid & 15;
+        V* src = a > J ? blk(a, J) + r : Sb + a * BLK + P * r;
+        const int step = a > J ? P : 1;
+        V w[16];
 #pragma unroll
-        for (int x = 0; x < 8; x++) acc[x] = czero<V>();
-#pragma unroll 4
-        for (int kk = 0; kk < 16; kk++) {
-          const V av = a > J ? src[r + P * kk] : src[kk + P * r];
-          const V* b = blk(J, J) + P * kk + 8 * h;         // T(n, kk), zero for n <= kk
+        for (int c = 0; c < 16; c++) w[c] = src[c * step];
 #pragma unroll
-          for (int x = 0; x < 8; x++) acc[x] = cmad(av, b[x], acc[x]);
-        }
-        __syncwarp();
+        for (int c = 0; c < 15; c++)
 #pragma unroll
-        for (int x = 0; x < 8; x++) {
-          const int nn = 8 * h + x;
-          if (a > J) src[r + P * nn] = cadd(src[r + P * nn], acc[x]);
-          else blk(J, a)[nn + P * r] = cneg(cadd(src[nn + P * r], acc[x]));
+          for (int i = c + 1; i < 16; i++) w[i] = cmsub(ljj[16 * c + i], w[c], w[i]);
+        if (a > J) {
+#pragma unroll
+          for (int c = 0; c < 16; c++) src[c * step] = w[c];
+        } else {
+#pragma unroll
+          for (int c = 0; c < 16; c++) blk(J, a)[c + P * r] = cneg(w[c]);
         }
       }
     }

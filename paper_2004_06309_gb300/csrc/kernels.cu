@@ -135,57 +135,6 @@ __global__ void __launch_bounds__(256) k_wg(const int2* tasks, const SnDev* sn, 
   }
 }
 
-// Schur update of the contribution block, one 32x32 lower tile per task:
-//   F22[a][b] -= sum_i W[a][i] D^{-1}_i W[b][i].
-template <typename V>
-__global__ void __launch_bounds__(256) k_cb(const int4* tasks, const SnDev* sn, const int64_t* scr_off,
-                                            V* fronts, const V* scratch) {
-  __shared__ V As[16][33];
-  __shared__ V Bs[16][33];
-  const int4 t = tasks[blockIdx.x];
-  const SnDev S = sn[t.x];
-  const int k = S.k, m = S.m, r = m - k;
-  const V* W = scratch + scr_off[t.x];
-  V* F = fronts + S.frontoff;
-  const int a0 = t.y * 32, b0 = t.z * 32;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  V acc[2][2];
-  for (int p = 0; p < 2; p++)
-    for (int q = 0; q < 2; q++) acc[p][q] = czero<V>();
-  for (int i0 = 0; i0 < k; i0 += 16) {
-    for (int e = tid; e < 512; e += 256) {
-      const int rr = e & 31, ii = e >> 5;
-      const int i = i0 + ii;
-      V av = czero<V>(), bv = czero<V>();
-      if (i < k) {
-        if (a0 + rr < r) av = W[(a0 + rr) + int64_t(i) * r];
-        if (b0 + rr < r) bv = cmul(W[(b0 + rr) + int64_t(i) * r], F[i + int64_t(i) * m]);
-      }
-      As[ii][rr] = av;
-      Bs[ii][rr] = bv;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int ii = 0; ii < 16; ii++) {
-      const V x0 = As[ii][ty * 2], x1 = As[ii][ty * 2 + 1];
-      const V y0 = Bs[ii][tx * 2], y1 = Bs[ii][tx * 2 + 1];
-      acc[0][0] = cmad(x0, y0, acc[0][0]);
-      acc[0][1] = cmad(x0, y1, acc[0][1]);
-      acc[1][0] = cmad(x1, y0, acc[1][0]);
-      acc[1][1] = cmad(x1, y1, acc[1][1]);
-    }
-    __syncthreads();
-  }
-  for (int p = 0; p < 2; p++)
-    for (int q = 0; q < 2; q++) {
-      const int a = a0 + ty * 2 + p, b = b0 + tx * 2 + q;
-      if (a < r && b < r && a >= b) {
-        const int64_t pos = (k + a) + int64_t(k + b) * m;
-        F[pos] = csub(F[pos], acc[p][q]);
-      }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Tensor-core (tcgen05) Schur update of complex64 fronts, one 128 x 128 lower
 // tile of the contribution block per CTA (8 warps):
@@ -483,9 +432,13 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
   int64_t wb, we;
   range(F.h_wg_g, lev, wb, we);
   if (we > wb) {
-    HZ_COUNT();
-    k_wg<V><<<unsigned(we - wb), 256, wg_smem(maxk, sizeof(V)), st>>>(F.wg_tasks + wb, F.sn, F.scr_off, fronts,
+    if constexpr (sizeof(V) == 8) {
+      HZ_COUNT();
+      k_wg<V><<<unsigned(we - wb), 256, wg_smem(maxk, sizeof(V)), st>>>(F.wg_tasks + wb, F.sn, F.scr_off, fronts,
                                                                        scratch);
+    } else {
+      launch_wg_dig(we - wb, maxk, F.wg_tasks + wb, F, fronts, scratch, status, st);
+    }
   }
   if constexpr (sizeof(V) == 8) {
     int64_t tb, te;
@@ -498,32 +451,24 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
   } else {
     int64_t cbb, cbe;
     range(F.h_cb_g, lev, cbb, cbe);
-    if (cbe > cbb) {
-      HZ_COUNT();
-      k_cb<V><<<unsigned(cbe - cbb), 256, 0, st>>>(F.cb_tasks + cbb, F.sn, F.scr_off, fronts, scratch);
-    }
+    if (cbe > cbb) launch_cb_dig(cbe - cbb, maxk, F.cb_tasks + cbb, F, fronts, scratch, st);
   }
   HZ_COUNT();
   k_panel_copy<V><<<dim3(unsigned(nb), split_for(nb, maxk)), 256, 0, st>>>(lsn, F.sn, fronts, (V*)F.panels);
 }
 
-static bool g_attr_done[2] = {false, false};
-static void set_attrs(int prec, int kmax) {
-  if (g_attr_done[prec]) return;
-  const int lim = 227 * 1024;
-  if (prec == 0) {
-    cudaFuncSetAttribute(k_wg<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  } else {
+static void set_attrs() {
+  static const bool done = [] {
     cudaFuncSetAttribute(k_cb_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemFloats * int(sizeof(float)));
-    cudaFuncSetAttribute(k_wg<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  }
-  g_attr_done[prec] = true;
-  (void)kmax;
+    cudaFuncSetAttribute(k_wg<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    return true;
+  }();
+  (void)done;
 }
 
 void launch_factor_level(const FactorDev& F, int lev, int grp, double w, void* fronts, void* scratch,
                          DevStatus* status, double tiny, cudaStream_t st) {
-  set_attrs(F.precision, F.maxk);
+  set_attrs();
   if (F.precision == 0)
     factor_level_t<double2>(F, lev, grp, w, (double2*)fronts, (double2*)scratch, status, tiny, st);
   else
@@ -1018,9 +963,13 @@ static void merge_panels_t(const FactorDev& F, cudaStream_t st) {
     if (m.w > 0) {
       HZ_COUNT();
       k_merge_save<<<grid_for(int64_t(m.ks) * m.w, 256), 256, 0, st>>>(M, m.ldm, m.w, m.ks, tmp);
-      HZ_COUNT();
-      k_merge_update<<<dim3(unsigned((m.ms + 63) / 64), unsigned((m.w + 31) / 32)), 256, 0, st>>>(
-          M, m.ldm, m.w, Ps, m.lds, m.ks, m.ms, tmp);
+      if constexpr (sizeof(V) == 16) {
+        launch_merge_dig(M, m.ldm, m.w, Ps, m.lds, m.ks, m.ms, tmp, st);
+      } else {
+        HZ_COUNT();
+        k_merge_update<<<dim3(unsigned((m.ms + 63) / 64), unsigned((m.w + 31) / 32)), 256, 0, st>>>(
+            M, m.ldm, m.w, Ps, m.lds, m.ks, m.ms, tmp);
+      }
     }
     HZ_COUNT();
     k_merge_put<<<grid_for(int64_t(m.ks) * m.ms, 256), 256, 0, st>>>(M, m.ldm, m.w, Ps, m.lds, m.ks, m.ms);
