@@ -759,7 +759,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
     std::vector<int2> mf;
     std::vector<int4> mb, mfin;
     std::vector<int64_t> mf_ptr(ST.nlev + 1), mb_ptr(ST.nlev + 1);
-    F.h_mfwd_rt.assign(size_t(ST.nlev), 64);
+    F.h_mfwd_rt.assign(size_t(ST.nlev), precision == 1 && nrhs_block == 4 ? 128 : 64);   // kFwdRows32
     int64_t max_mb = 0;
     for (int l = 0; l < ST.nlev; l++) {
       mf_ptr[l] = int64_t(mf.size());

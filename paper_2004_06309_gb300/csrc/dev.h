@@ -214,6 +214,8 @@ void launch_merge_panels(const FactorDev& F, cudaStream_t st);
 void launch_to_digits(const FactorDev& F, cudaStream_t st);
 void launch_solve_dig(const FactorDev& F, cudaStream_t st);
 void launch_solve_dig_multi(const FactorDev& F, int S, cudaStream_t st);
+// complex64, S interleaved right-hand sides (multi32.cu)
+void launch_solve_multi32(const FactorDev& F, int S, cudaStream_t st);
 void launch_prolong(const FactorDev& F, const double2* y, double2* z, cudaStream_t st);
 
 void launch_local_multi(const FactorDev& F, int S, const double2* src, const double2* y, double2* dst,

@@ -107,6 +107,87 @@ template <typename V> __device__ __forceinline__ V ldv(const V* p);
 template <> __device__ __forceinline__ float2 ldv<float2>(const float2* p) { return __ldcg(p); }
 template <> __device__ __forceinline__ double2 ldv<double2>(const double2* p) { return __ldcg(p); }
 
+// ---------------------------------------------------------------------------
+// batched sweeps: S right-hand sides per row, moved 16 bytes at a time (one complex128 or two
+// complex64 values), 256 threads.  A row's child contributions are adjacent (cptr); the loads of U
+// rows, their row pointers, and of each row's first two contributions (a nested-dissection
+// supernode has at most two children) are issued together: one after the other, these chains
+// held the forward tasks (22 us each at k = 128, S = 16 in complex64, of which 20 were this).
+// ---------------------------------------------------------------------------
+template <typename V> struct Vec16;
+template <> struct Vec16<float2> { using T = float4; };
+template <> struct Vec16<double2> { using T = double2; };
+__device__ __forceinline__ float4 vadd(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return cadd(a, b); }
+__device__ __forceinline__ float4 vsub(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ double2 vsub(double2 a, double2 b) { return csub(a, b); }
+template <typename T> __device__ __forceinline__ T vzero();
+template <> __device__ __forceinline__ float4 vzero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+template <> __device__ __forceinline__ double2 vzero<double2>() { return make_double2(0.0, 0.0); }
+
+// a[q] + the contributions c0[q] .. c1[q] - 1 of U rows, lane i of LR per row
+template <typename V, int LR, int U, typename T>
+__device__ __forceinline__ void add_contributions(T* a, const uint32_t* c0, const uint32_t* c1, const V* u, int i) {
+  const T* u16 = reinterpret_cast<const T*>(u) + i;
+  T v0[U], v1[U];
+#pragma unroll
+  for (int q = 0; q < U; q++) {
+    v0[q] = c0[q] < c1[q] ? __ldcg(u16 + int64_t(c0[q]) * LR) : vzero<T>();
+    v1[q] = c0[q] + 1 < c1[q] ? __ldcg(u16 + int64_t(c0[q] + 1) * LR) : vzero<T>();
+  }
+#pragma unroll
+  for (int q = 0; q < U; q++) {
+    a[q] = vadd(vadd(a[q], v0[q]), v1[q]);
+    for (uint32_t c = c0[q] + 2; c < c1[q]; c++) a[q] = vadd(a[q], __ldcg(u16 + int64_t(c) * LR));
+  }
+}
+
+// dst[j] = tin[j] + contributions of row j, j < k
+template <typename V, int S>
+__device__ __forceinline__ void gather_rows(V* dst, const V* tin, const uint32_t* cp, const V* u, int k) {
+  using T = typename Vec16<V>::T;
+  constexpr int LR = S * int(sizeof(V)) / 16, RP = 256 / LR, U = 4;
+  const int i = threadIdx.x % LR;
+  const T* t16 = reinterpret_cast<const T*>(tin) + i;
+  for (int j0 = threadIdx.x / LR; j0 < k; j0 += U * RP) {
+    uint32_t c0[U], c1[U];
+    T a[U];
+#pragma unroll
+    for (int q = 0; q < U; q++) {
+      const int j = j0 + q * RP;
+      c0[q] = j < k ? cp[j] : 0u;
+      c1[q] = j < k ? cp[j + 1] : 0u;
+      a[q] = j < k ? __ldcg(t16 + int64_t(j) * LR) : vzero<T>();
+    }
+    add_contributions<V, LR, U>(a, c0, c1, u, i);
+#pragma unroll
+    for (int q = 0; q < U; q++)
+      if (j0 + q * RP < k) reinterpret_cast<T*>(dst)[(j0 + q * RP) * LR + i] = a[q];
+  }
+}
+
+// A forward task's update rows: their contributions and where they go, N 16-byte items per thread
+// (rows row0 + item / LR of RT), loaded before the task's products.
+template <typename V, int S, int RT> struct UpdateRows {
+  using T = typename Vec16<V>::T;
+  static constexpr int LR = S * int(sizeof(V)) / 16, N = (RT * LR + 255) / 256;
+  T b2[N];
+  uint32_t to[N];
+  __device__ __forceinline__ void load(const SnDev& Sn, const uint32_t* cp, const uint32_t* wpos, const V* u, int row0) {
+    uint32_t c0[N], c1[N];
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+      const int e = threadIdx.x + 256 * q, r = row0 + e / LR;
+      const bool ok = e < RT * LR && r >= Sn.k && r < Sn.m;
+      c0[q] = ok ? cp[r] : 0u;
+      c1[q] = ok ? cp[r + 1] : 0u;
+      to[q] = ok ? wpos[Sn.uoff + (r - Sn.k)] : 0u;
+      b2[q] = vzero<T>();
+    }
+    add_contributions<V, LR, N>(b2, c0, c1, u, threadIdx.x % LR);
+  }
+};
+
 // Fused second stage of the backward sweep ("last block done"), for a (supernode,
 // column block) split over several row chunks: every partial-sum CTA of the pair
 // publishes its 32 sums, fences, and bumps the pair's counter; the CTA that brings it

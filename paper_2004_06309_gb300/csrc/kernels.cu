@@ -1025,171 +1025,12 @@ __global__ void k_prolong_multi(int64_t n, const int64_t* pptr, const int32_t* p
   }
 }
 
-// Forward, 64 rows x S right-hand sides per task; 128 threads = 64 rows x 2 column parities.
-template <typename V, int S>
-__global__ void __launch_bounds__(128) k_fwd_multi(const int2* tasks, const SnDev* sn, const uint32_t* cptr,
-                                                   const uint32_t* wpos, const V* panels, const V* tin, V* zout,
-                                                   V* u, int kpad) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* b1 = reinterpret_cast<V*>(smem_raw);               // kpad x S
-  V* part = b1 + kpad * S;                                // 2 x 64 x S
-  const int2 t = tasks[blockIdx.x];
-  const SnDev Sn = sn[t.x];
-  const int k = Sn.k, m = Sn.m, tid = threadIdx.x;
-  const uint32_t* cp = cptr + Sn.rowoff;
-  for (int e = tid; e < k * S; e += blockDim.x) {
-    const int j = e / S, i = e % S;
-    V acc = tin[int64_t(Sn.first + j) * S + i];
-    for (uint32_t c = cp[j]; c < cp[j + 1]; c++) acc = cadd(acc, u[int64_t(c) * S + i]);
-    b1[e] = acc;
-  }
-  __syncthreads();
-  const int rr = tid & 63, cg = tid >> 6;
-  const int r = t.y * 64 + rr;
-  V acc[S];
-#pragma unroll
-  for (int i = 0; i < S; i++) acc[i] = czero<V>();
-  if (r < m) {
-    const int jmax = min(r, k);
-    const V* P = panels + Sn.paneloff + r;
-    for (int j = cg; j < jmax; j += 2) {
-      const V p = P[int64_t(j) * Sn.ld];
-      const V* bj = b1 + j * S;
-#pragma unroll
-      for (int i = 0; i < S; i++) acc[i] = cmad(p, bj[i], acc[i]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < S; i++) part[(cg * 64 + rr) * S + i] = acc[i];
-  __syncthreads();
-  for (int e = tid; e < 64 * S; e += blockDim.x) {
-    const int row = e / S, i = e % S;
-    const int rw = t.y * 64 + row;
-    if (rw >= m) continue;
-    const V tot = cadd(part[row * S + i], part[(64 + row) * S + i]);
-    if (rw < k) {
-      zout[int64_t(Sn.first + rw) * S + i] = cmul(panels[Sn.paneloff + rw + int64_t(rw) * Sn.ld], cadd(b1[rw * S + i], tot));
-    } else {
-      V b2 = czero<V>();
-      for (uint32_t c = cp[rw]; c < cp[rw + 1]; c++) b2 = cadd(b2, u[int64_t(c) * S + i]);
-      u[int64_t(wpos[Sn.uoff + (rw - k)]) * S + i] = csub(b2, tot);
-    }
-  }
-}
-
-// Backward partial sums for S right-hand sides: thread (c, slice) owns pivot column
-// 32 * block + c over a quarter of the chunk's rows; slices are added in a fixed
-// order; the last CTA of a (supernode, column block) finishes x (no waits).
-template <typename V, int S>
-__global__ void __launch_bounds__(128) k_bwd_multi(const int4* tasks, const SnDev* sn, const int32_t* rowlist,
-                                                   const V* panels, const V* zin, V* x, V* partial, int rows,
-                                                   const int4* fins, unsigned int* counters) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* vec = reinterpret_cast<V*>(smem_raw);              // rows x S
-  V* red = vec + rows * S;                                // 4 x 32 x S
-  __shared__ unsigned int ticket;
-  const int4 t = tasks[blockIdx.x];
-  const SnDev Sn = sn[t.x];
-  const int k = Sn.k, m = Sn.m, tid = threadIdx.x, c = tid & 31, sl = tid >> 5;
-  const int r0 = t.z * rows, r1 = min(m, r0 + rows);
-  const int32_t* rl = rowlist + Sn.rowoff;
-  for (int e = tid; e < (r1 - r0) * S; e += blockDim.x) {
-    const int r = r0 + e / S, i = e % S;
-    vec[e] = (r < k) ? zin[int64_t(Sn.first + r) * S + i] : cneg(x[int64_t(rl[r]) * S + i]);
-  }
-  __syncthreads();
-  const int j = t.y * 32 + c;
-  const int slice = (rows + 3) / 4;
-  const int ra = max(r0 + sl * slice, j + 1), rb = min(r1, r0 + (sl + 1) * slice);
-  V acc[S];
-#pragma unroll
-  for (int i = 0; i < S; i++) acc[i] = czero<V>();
-  if (j < k) {
-    const V* col = panels + Sn.paneloff + int64_t(j) * Sn.ld;
-    for (int r = ra; r < rb; r++) {
-      const V p = col[r];
-      const V* vr = vec + (r - r0) * S;
-#pragma unroll
-      for (int i = 0; i < S; i++) acc[i] = cmad(p, vr[i], acc[i]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < S; i++) red[(sl * 32 + c) * S + i] = acc[i];
-  __syncthreads();
-  V* out = partial + int64_t(blockIdx.x) * 32 * S;
-  for (int e = tid; e < 32 * S; e += blockDim.x) {
-    V tot = red[e];
-    for (int q = 1; q < 4; q++) tot = cadd(tot, red[q * 32 * S + e]);
-    out[e] = tot;
-  }
-  // fused second stage
-  const int4 fin = fins[t.w];
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) ticket = atomicAdd(counters + t.w, 1u);
-  __syncthreads();
-  if (ticket != unsigned(fin.w) - 1) return;
-  __threadfence();
-  for (int e = tid; e < 32 * S; e += blockDim.x) {
-    const int cc = e / S, i = e % S;
-    const int jj = fin.y * 32 + cc;
-    if (jj >= k) continue;
-    V a = czero<V>();
-    for (int ch = 0; ch < fin.w; ch++) {
-      const V* pp = partial + (int64_t(fin.z + ch) * 32 + cc) * S + i;
-      V v;
-      if constexpr (sizeof(V) == 8) {
-        const float2 q2 = __ldcg(reinterpret_cast<const float2*>(pp));
-        v.x = q2.x; v.y = q2.y;
-      } else {
-        const double2 q2 = __ldcg(reinterpret_cast<const double2*>(pp));
-        v.x = q2.x; v.y = q2.y;
-      }
-      a = cadd(a, v);
-    }
-    x[int64_t(Sn.first + jj) * S + i] = cadd(zin[int64_t(Sn.first + jj) * S + i], a);
-  }
-  if (tid == 0) counters[t.w] = 0u;
-}
-
-template <int S>
-static void solve_multi_c64(const FactorDev& F, cudaStream_t st) {
-  using V = float2;
-  static const bool attr = [] {
-    cudaFuncSetAttribute(k_fwd_multi<V, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_bwd_multi<V, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    return true;
-  }();
-  (void)attr;
-  const V* P = (const V*)F.panels;
-  V *t = (V*)F.mt_loc, *z = (V*)F.mz_loc, *x = (V*)F.mx_loc, *u = (V*)F.mu_ws;
-  for (int l = 0; l < F.snlev; l++) {
-    const int64_t b = F.h_mfwd_ptr[l], e = F.h_mfwd_ptr[l + 1];
-    if (e > b) {
-      HZ_COUNT();
-      const int kpad = F.h_lev_k[l];
-      const size_t fsm = size_t(kpad * S + 2 * 64 * S) * sizeof(V);
-      k_fwd_multi<V, S><<<unsigned(e - b), 128, fsm, st>>>(F.mfwd_tasks + b, F.ssn, F.cptr, F.wpos, P, t, z, u, kpad);
-    }
-  }
-  const size_t bsm = size_t(kMultiBwdRows * S + 4 * 32 * S) * sizeof(V);
-  for (int l = F.snlev - 1; l >= 0; l--) {
-    const int64_t b = F.h_mbwd_ptr[l], e = F.h_mbwd_ptr[l + 1];
-    if (e > b) {
-      HZ_COUNT();
-      k_bwd_multi<V, S><<<unsigned(e - b), 128, bsm, st>>>(F.mbwd_tasks + b, F.ssn, F.rowlist, P, z, x,
-                                                           (V*)F.mbwd_partial, kMultiBwdRows, F.mbfin_tasks,
-                                                           F.mbwd_counters);
-    }
-  }
-}
-
 template <typename V, int S>
 static void prec_multi_t(const FactorDev& F, const double2* src, const double2* y, double2* dst, cudaStream_t st) {
   V* t = (V*)F.mt_loc;
   HZ_COUNT();
   k_gather_multi<V, S><<<grid_for(F.ntot * S, 256), 256, 0, st>>>(F.ntot, F.gidx, src, t);
-  if constexpr (sizeof(V) == 8) solve_multi_c64<S>(F, st);
+  if constexpr (sizeof(V) == 8) launch_solve_multi32(F, S, st);
   else launch_solve_dig_multi(F, S, st);
   HZ_COUNT();
   k_prolong_multi<V, S><<<grid_for(F.nglob * S, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw,

@@ -553,12 +553,9 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
     nonfin[tid] = 0;
   }
   if (16 * kg < jend) load(kg);
-  for (int e = tid; e < k * S; e += 256) {
-    const int j = e / S, i = e % S;
-    double2 a = ldv(tin + int64_t(Sn.first + j) * S + i);
-    for (uint32_t c = cp[j]; c < cp[j + 1]; c++) a = cadd(a, ldv(u + int64_t(c) * S + i));
-    b1[e] = a;
-  }
+  gather_rows<double2, S>(b1, tin + int64_t(Sn.first) * S, cp, u, k);
+  UpdateRows<double2, S, RT> up;
+  up.load(Sn, cp, wpos, u, tk.y * RT);
   float cr[8][4], ci[8][4];
 #pragma unroll
   for (int d = 0; d < 8; d++)
@@ -585,20 +582,18 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
   part[(kg * RT + mt * 16 + g) * S + rhs] = acc[0];
   part[(kg * RT + mt * 16 + g + 8) * S + rhs] = acc[1];
   __syncthreads();
-  for (int e = tid; e < RT * S; e += 256) {
-    const int i = e % S, r = tk.y * RT + e / S;
-    if (r >= m) continue;
+#pragma unroll
+  for (int n = 0; n < up.N; n++) {
+    const int e = tid + 256 * n, i = e % S, r = tk.y * RT + e / S;
+    if (e >= RT * S || r >= m) continue;
     double2 s = part[e];
 #pragma unroll
     for (int q = 1; q < KG; q++) s = cadd(s, part[q * RT * S + e]);
     if (nonfin[i] || rexp[Sn.eoff + r] == kRowNonFinite) s = make_double2(nan(""), nan(""));
-    if (r < k) {
+    if (r < k)
       zout[int64_t(Sn.first + r) * S + i] = cmul(panels[Sn.paneloff + r + int64_t(r) * Sn.ld], cadd(b1[r * S + i], s));
-    } else {
-      double2 b2 = make_double2(0.0, 0.0);
-      for (uint32_t c = cp[r]; c < cp[r + 1]; c++) b2 = cadd(b2, ldv(u + int64_t(c) * S + i));
-      u[int64_t(wpos[Sn.uoff + (r - k)]) * S + i] = csub(b2, s);
-    }
+    else
+      u[int64_t(up.to[n]) * S + i] = csub(up.b2[n], s);
   }
 }
 
@@ -640,9 +635,21 @@ __global__ void __launch_bounds__(256) k_bwd_dig_multi(const int4* tasks, const 
   if (kg < nst) load(kg);
   const int32_t* rl = rowlist + Sn.rowoff;
   for (int r = tid; r < cnt; r += 256) vex[r] = rexp[Sn.eoff + r0 + r];
-  for (int e = tid; e < cnt * S; e += 256) {
-    const int r = r0 + e / S, i = e % S;
-    vec[e] = r < k ? ldv(zin + int64_t(Sn.first + r) * S + i) : cneg(ldv(x + int64_t(rl[r]) * S + i));
+  {
+    constexpr int U = ROWS * S / 256 < 4 ? ROWS * S / 256 : 4;             // row indices of U values, then the values
+    for (int e0 = tid; e0 < cnt * S; e0 += 256 * U) {
+      int32_t at[U];
+#pragma unroll
+      for (int n = 0; n < U; n++) {
+        const int r = r0 + (e0 + 256 * n) / S;
+        at[n] = r < r1 && r >= k ? rl[r] : 0;
+      }
+#pragma unroll
+      for (int n = 0; n < U; n++) {
+        const int e = e0 + 256 * n, r = r0 + e / S, i = e % S;
+        if (r < r1) vec[e] = r < k ? ldv(zin + int64_t(Sn.first + r) * S + i) : cneg(ldv(x + int64_t(at[n]) * S + i));
+      }
+    }
   }
   float cr[8][4], ci[8][4];
 #pragma unroll
