@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhz.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["setup.cpp", "symbolic.cpp", "kernels.cu", "sweeps64.cu", "diag.cu", "factor64.cu", "multi32.cu", "capi.cu", "noalloc.cu", "server.cpp", "recycle.cpp"]
+SOURCES = ["setup.cpp", "symbolic.cpp", "kernels.cu", "sweeps64.cu", "diag.cu", "factor64.cu", "multi32.cu", "cgs.cu", "capi.cu", "noalloc.cu", "server.cpp", "recycle.cpp"]
 HEADERS = ["host.h", "dev.h", "dmath.cuh", "digits.cuh", "engine.h", "small_la.h"]
 
 

@@ -57,6 +57,7 @@ struct hz_ctx {
   double2 *V = nullptr, *Zs = nullptr, *w = nullptr, *b = nullptr, *x = nullptr, *y = nullptr, *t = nullptr;
   double2 *rH = nullptr, *yH = nullptr;
   double2 *partial = nullptr, *h1 = nullptr, *h2 = nullptr, *nrm = nullptr;
+  unsigned int* ticket = nullptr;          // CGS passes: blocks done, per slot (zero between launches)
   double2 *H = nullptr, *sn = nullptr, *g = nullptr, *ysol = nullptr;
   double *cs = nullptr, *scal = nullptr;   // scal: est, invh, invbeta, beta, |b|
   // one CUDA graph per inner-iteration index j (captured on first use)
@@ -906,6 +907,26 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
   return HZ_OK;
 }
 
+// The Givens update of one vector's Hessenberg column (|b| at scal[bn_off]).
+hz::SlotGivens givens_args(int j, int m, double2* H, double* cs, double2* sn, double2* g, const double2* h1,
+                           const double2* h2, const double2* nrm, double* scal, int bn_off, int* brk) {
+  hz::SlotGivens p{};
+  for (int i = 1; i < 16; i++) p.j[i] = -1;
+  p.m = m;
+  p.bn_off = bn_off;
+  p.j[0] = j;
+  p.H = H;
+  p.cs = cs;
+  p.sn = sn;
+  p.g = g;
+  p.h1 = h1;
+  p.h2 = h2;
+  p.nrm = nrm;
+  p.scal = scal;
+  p.brk = brk;
+  return p;
+}
+
 // y ~ E^{-1} r (iterative coarse solve): one cycle of GMRES(coarse_maxit) on E
 // right-preconditioned by one-level ORAS on the coarse mesh (Eq. 4 with the coarse
 // subdomains), CGS2 and the Givens rotations of the outer solve, x0 = 0, ending when
@@ -915,11 +936,9 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
 void coarse_inner(hz_ctx* c, const double2* r, double2* y) {
   const int64_t nH = c->nH;
   const int mH = c->cmaxit;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   double* pin = c->h_pin + hz_ctx::PIN_CRS;
-  hz::launch_cgs(nH, 0, c->VH, nH, nullptr, const_cast<double2*>(r), 0, c->partial, st);
-  hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+  hz::launch_cgs(nH, 0, c->VH, nH, nullptr, const_cast<double2*>(r), false, c->partial, c->ticket, c->nrm, st);
   cudaMemsetAsync(y, 0, size_t(nH) * 16, st);
   cudaMemcpyAsync(pin, &c->nrm[64].x, sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
@@ -937,14 +956,10 @@ void coarse_inner(hz_ctx* c, const double2* r, double2* y) {
     hz::launch_solve(c->cloc, st);                                                // E_i^{-1}
     hz::launch_prolong(c->cloc, nullptr, zj, st);                                 // sum R^T D x_i
     hz::launch_spmv(nH, c->d_Erp, c->d_Eci, c->d_E, zj, nullptr, c->wH, st);      // E z_j
-    hz::launch_cgs(nH, j + 1, c->VH, nH, nullptr, c->wH, j + 1, c->partial, st);
-    hz::launch_reduce(c->partial, nb, j + 1, c->h1, st);
-    hz::launch_cgs(nH, j + 1, c->VH, nH, c->h1, c->wH, j + 1, c->partial, st);
-    hz::launch_reduce(c->partial, nb, j + 1, c->h2, st);
-    hz::launch_cgs(nH, j + 1, c->VH, nH, c->h2, c->wH, 0, c->partial, st);
-    hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
-    hz::launch_givens(j, mH, c->HH, c->csH, c->snH, c->gH, c->h1, c->h2, c->nrm, c->scalH + 3, c->scalH, c->brkH,
-                      c->scalH + 1, st);
+    hz::launch_cgs(nH, j + 1, c->VH, nH, nullptr, c->wH, true, c->partial, c->ticket, c->h1, st);
+    hz::launch_cgs(nH, j + 1, c->VH, nH, c->h1, c->wH, true, c->partial, c->ticket, c->h2, st);
+    const hz::SlotGivens gv = givens_args(j, mH, c->HH, c->csH, c->snH, c->gH, c->h1, c->h2, c->nrm, c->scalH, 3, c->brkH);
+    hz::launch_cgs(nH, j + 1, c->VH, nH, c->h2, c->wH, false, c->partial, c->ticket, c->nrm, st, &gv);
     hz::launch_scale(nH, c->wH, c->scalH + 1, c->VH + int64_t(j + 1) * nH, st);
     cudaMemcpyAsync(pin + 1, c->scalH, sizeof(double), cudaMemcpyDeviceToHost, st);
     cudaMemcpyAsync(pin + 2, c->brkH, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -990,9 +1005,7 @@ void apply_prec(hz_ctx* c, const double2* v, double2* z) {
 
 
 hz_status norm2(hz_ctx* c, const double2* v, double& out) {
-  const int nb = hz::cgs_blocks();
-  hz::launch_cgs(c->n, 0, c->V, c->n, nullptr, const_cast<double2*>(v), 0, c->partial, c->st);
-  hz::launch_reduce(c->partial, nb, 0, c->nrm, c->st);
+  hz::launch_cgs(c->n, 0, c->V, c->n, nullptr, const_cast<double2*>(v), false, c->partial, c->ticket, c->nrm, c->st);
   CU(cudaMemcpyAsync(c->h_pin + 5, &c->nrm[64].x, sizeof(double), cudaMemcpyDeviceToHost, c->st));
   CU(cudaStreamSynchronize(c->st));
   out = std::sqrt(c->h_pin[5]);
@@ -1006,7 +1019,6 @@ hz_status norm2(hz_ctx* c, const double2* v, double& out) {
 void iteration_kernels(hz_ctx* c, int j) {
   const int64_t n = c->n;
   const int m = c->restart;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   double2* vj = c->V + int64_t(j) * n;
   double2* zj = c->Zs + int64_t(j) * n;
@@ -1015,14 +1027,14 @@ void iteration_kernels(hz_ctx* c, int j) {
   // orthogonalise against [C, v_0..v_j] (C: the recycled space, empty without recycling)
   const int kk = c->ckk, nc = kk + j + 1;
   const double2* base = c->V - int64_t(kk) * n;
-  hz::launch_cgs(n, nc, base, n, nullptr, c->w, nc, c->partial, st);        // h1, |w|
-  hz::launch_reduce(c->partial, nb, nc, c->h1, st);
-  hz::launch_cgs(n, nc, base, n, c->h1, c->w, nc, c->partial, st);          // w -= [C V] h1; h2
-  hz::launch_reduce(c->partial, nb, nc, c->h2, st);
-  hz::launch_cgs(n, nc, base, n, c->h2, c->w, 0, c->partial, st);           // w -= [C V] h2; |w|
-  hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
-  hz::launch_givens(j, m, c->H, c->cs, c->sn, c->g, c->h1, c->h2, c->nrm, c->scal + 4, c->scal, c->brk,
-                    c->scal + 1, st, kk, c->rk ? c->Hraw : nullptr, c->Braw, c->rk);
+  hz::launch_cgs(n, nc, base, n, nullptr, c->w, true, c->partial, c->ticket, c->h1, st);        // h1, |w|
+  hz::launch_cgs(n, nc, base, n, c->h1, c->w, true, c->partial, c->ticket, c->h2, st);          // w -= [C V] h1; h2
+  hz::SlotGivens gv = givens_args(j, m, c->H, c->cs, c->sn, c->g, c->h1, c->h2, c->nrm, c->scal, 4, c->brk);
+  gv.off = kk;
+  gv.raw_h = c->rk ? c->Hraw : nullptr;
+  gv.raw_b = c->Braw;
+  gv.ldb = c->rk;
+  hz::launch_cgs(n, nc, base, n, c->h2, c->w, false, c->partial, c->ticket, c->nrm, st, &gv);   // w -= [C V] h2; |w|
   hz::launch_scale(n, c->w, c->scal + 1, c->V + int64_t(j + 1) * n, st);
   cudaMemcpyAsync(c->h_pin, c->scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaMemcpyAsync(c->h_pin + 4, c->brk, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1065,7 +1077,6 @@ hz_status run_iteration(hz_ctx* c, int j) {
 hz_status fgmres_one(hz_ctx* c, double tol, hz_rhs_info* info) {
   const int64_t n = c->n;
   const int m = c->restart;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   double bnorm = 0;
   TRY(norm2(c, c->b, bnorm));
@@ -1084,8 +1095,7 @@ hz_status fgmres_one(hz_ctx* c, double tol, hz_rhs_info* info) {
   CU(cudaMemcpyAsync(c->scal + 4, c->h_pin + 6, sizeof(double), cudaMemcpyHostToDevice, st));
   // r = b
   hz::launch_axpby_copy(n, c->b, c->w, st);
-  hz::launch_cgs(n, 0, c->V, n, nullptr, c->w, 0, c->partial, st);
-  hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+  hz::launch_cgs(n, 0, c->V, n, nullptr, c->w, false, c->partial, c->ticket, c->nrm, st);
   int its = 0;
   for (;;) {
     hz::launch_init_cycle(c->nrm, c->g, m, d_invbeta, d_beta, st);
@@ -1212,7 +1222,6 @@ hz_status recycle_space(hz_ctx* c, int kk, int kc, int s, const std::vector<cplx
                         double2* V, const double2* Z) {
   const int rk = c->rk;
   const int64_t n = c->n;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   if (kc < 1) return HZ_OK;
   CU(cudaStreamSynchronize(st));
@@ -1256,8 +1265,7 @@ hz_status recycle_space(hz_ctx* c, int kk, int kc, int s, const std::vector<cplx
       double unorm2 = 0.0;
       for (int a = 0; a < ng; a += 64) {
         const int wc = std::min(64, ng - a);
-        hz::launch_cgs(n, wc, Cb + int64_t(a) * n, n, nullptr, ui, wc, c->partial, st);
-        hz::launch_reduce(c->partial, nb, wc, c->h1, st);
+        hz::launch_cgs(n, wc, Cb + int64_t(a) * n, n, nullptr, ui, true, c->partial, c->ticket, c->h1, st);
         CU(cudaStreamSynchronize(st));
         const std::vector<cplx> hv = to_host(c->h1, 65);
         for (int q = 0; q < wc; q++) VW[size_t(i) * ng + a + q] = hv[size_t(q)];
@@ -1379,7 +1387,6 @@ hz_status recycle_rebase(hz_ctx* c) {
 hz_status gcrodr_one(hz_ctx* c, double tol, hz_rhs_info* info) {
   const int64_t n = c->n;
   const int m = c->restart;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   double bnorm = 0;
   TRY(norm2(c, c->b, bnorm));
@@ -1407,10 +1414,8 @@ hz_status gcrodr_one(hz_ctx* c, double tol, hz_rhs_info* info) {
     if (kk > 0) {
       // r orthogonal to C: x += Ux C^H r, r -= C C^H r
       const double2* Cb = c->V - int64_t(kk) * n;
-      hz::launch_cgs(n, kk, Cb, n, nullptr, c->w, kk, c->partial, st);
-      hz::launch_reduce(c->partial, nb, kk, c->h1, st);
-      hz::launch_cgs(n, kk, Cb, n, c->h1, c->w, 0, c->partial, st);
-      hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+      hz::launch_cgs(n, kk, Cb, n, nullptr, c->w, true, c->partial, c->ticket, c->h1, st);
+      hz::launch_cgs(n, kk, Cb, n, c->h1, c->w, false, c->partial, c->ticket, c->nrm, st);
       hz::launch_combo(n, kk, c->Ux, n, 0, nullptr, n, c->h1, 1, c->x, n, 1.0, true, st);
       // b (or the restart residual) inside span(C): x is already the solution
       CU(cudaMemcpyAsync(c->h_pin + 5, &c->nrm[64].x, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1426,8 +1431,7 @@ hz_status gcrodr_one(hz_ctx* c, double tol, hz_rhs_info* info) {
         continue;
       }
     } else {
-      hz::launch_cgs(n, 0, c->V, n, nullptr, c->w, 0, c->partial, st);
-      hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+      hz::launch_cgs(n, 0, c->V, n, nullptr, c->w, false, c->partial, c->ticket, c->nrm, st);
     }
     hz::launch_init_cycle(c->nrm, c->g, m, c->scal + 2, c->scal + 3, st);
     hz::launch_scale(n, c->w, c->scal + 2, c->V, st);
@@ -1583,7 +1587,6 @@ hz_status slot_point_source(hz_ctx* c, int i, const double xyz[3]) {
 void slots_issue(hz_ctx* c) {
   const int S = c->S, m = c->restart;
   const int64_t n = c->n;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   if (c->spmv_lanes) hz::set_spmv_lanes(c->spmv_lanes);
   hz::SlotCols vin, zout, wout;
@@ -1606,6 +1609,7 @@ void slots_issue(hz_ctx* c) {
   hz::SlotGivens pg{};
   hz::SlotScale ps{};
   pg.m = m;
+  pg.bn_off = 4;
   pg.H = c->Hb;
   pg.sn = c->snb;
   pg.g = c->gb;
@@ -1627,11 +1631,11 @@ void slots_issue(hz_ctx* c) {
     ps.s[i] = run ? slot_scal(c, i) + 1 : nullptr;
     ps.out[i] = run ? slot_V(c, i) + int64_t(j + 1) * n : nullptr;
   }
-  hz::launch_cgs_slots(n, S, pc, false, true, c->partial_s, c->h1s, st);    // h1 = V^H w
-  hz::launch_cgs_slots(n, S, pc, true, true, c->partial_s, c->h2s, st);     // w -= V h1; h2 = V^H w
+  pc.ld = n;
+  hz::launch_cgs_slots(n, S, pc, false, true, c->partial_s, c->ticket, c->h1s, st);    // h1 = V^H w
+  hz::launch_cgs_slots(n, S, pc, true, true, c->partial_s, c->ticket, c->h2s, st);     // w -= V h1; h2 = V^H w
   for (int i = 0; i < 16; i++) pc.h[i] = c->h2s + int64_t(i) * 65;
-  hz::launch_cgs_slots(n, S, pc, true, false, c->partial_s, c->nrms, st);   // w -= V h2; |w|^2
-  hz::launch_givens_slots(S, pg, st);
+  hz::launch_cgs_slots(n, S, pc, true, false, c->partial_s, c->ticket, c->nrms, st, &pg);   // w -= V h2; |w|^2; Givens
   hz::launch_scale_slots(n, S, ps, st);
   cudaMemcpyAsync(c->h_pin + hz_ctx::PIN_SLOT, c->scalb, size_t(S) * 8 * sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaMemcpyAsync(c->h_pin + hz_ctx::PIN_FLAGS, c->brkb, size_t(S) * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1772,7 +1776,6 @@ hz_status solve_slots(hz_ctx* c, const double2* rhs, int nrhs, double tol, doubl
 hz_status block_orthonormalise(hz_ctx* c, double2* W, int s, double2* Q, std::vector<cplx>& R, const double* w0,
                                bool& brk) {
   const int64_t n = c->n;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   R.assign(size_t(s) * s, cplx(0.0, 0.0));
   brk = false;
@@ -1780,15 +1783,12 @@ hz_status block_orthonormalise(hz_ctx* c, double2* W, int s, double2* Q, std::ve
   for (int q = 0; q < s; q++) {
     double2* w = W + int64_t(q) * n;
     if (q > 0) {
-      hz::launch_cgs(n, q, Q, n, nullptr, w, q, c->partial, st);
-      hz::launch_reduce(c->partial, nb, q, c->h1, st);
-      hz::launch_cgs(n, q, Q, n, c->h1, w, q, c->partial, st);
-      hz::launch_reduce(c->partial, nb, q, c->h2, st);
-      hz::launch_cgs(n, q, Q, n, c->h2, w, 0, c->partial, st);
+      hz::launch_cgs(n, q, Q, n, nullptr, w, true, c->partial, c->ticket, c->h1, st);
+      hz::launch_cgs(n, q, Q, n, c->h1, w, true, c->partial, c->ticket, c->h2, st);
+      hz::launch_cgs(n, q, Q, n, c->h2, w, false, c->partial, c->ticket, c->nrm, st);
     } else {
-      hz::launch_cgs(n, 0, Q, n, nullptr, w, 0, c->partial, st);
+      hz::launch_cgs(n, 0, Q, n, nullptr, w, false, c->partial, c->ticket, c->nrm, st);
     }
-    hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
     CU(cudaMemcpyAsync(hh.data(), c->h1, 65 * 16, cudaMemcpyDeviceToHost, st));
     CU(cudaMemcpyAsync(hh.data() + 65, c->h2, 65 * 16, cudaMemcpyDeviceToHost, st));
     CU(cudaMemcpyAsync(hh.data() + 130, c->nrm, 65 * 16, cudaMemcpyDeviceToHost, st));
@@ -1831,6 +1831,7 @@ hz_status block_step(hz_ctx* c, int j, int s, int kk, std::vector<cplx>& hcol, b
   const int p = kk + (j + 1) * s;
   const int nch = (p + 63) / 64;
   hz::SlotCgs pc{};
+  pc.ld = n;
   for (int pass = 0; pass < 2; pass++) {
     for (int k = 0; k < nch; k++) {
       for (int i = 0; i < 16; i++) {
@@ -1840,7 +1841,8 @@ hz_status block_step(hz_ctx* c, int j, int s, int kk, std::vector<cplx>& hcol, b
         pc.h[i] = nullptr;
         pc.ncols[i] = on ? std::min(64, p - 64 * k) : -1;
       }
-      hz::launch_cgs_slots(n, S, pc, false, true, c->partial_s, c->hblk + (int64_t(pass) * nch + k) * S * 65, st);
+      hz::launch_cgs_slots(n, S, pc, false, true, c->partial_s, c->ticket,
+                           c->hblk + (int64_t(pass) * nch + k) * S * 65, st);
     }
     for (int k = 0; k < nch; k++) {
       for (int i = 0; i < 16; i++) {
@@ -1850,7 +1852,7 @@ hz_status block_step(hz_ctx* c, int j, int s, int kk, std::vector<cplx>& hcol, b
         pc.h[i] = on ? c->hblk + ((int64_t(pass) * nch + k) * S + i) * 65 : nullptr;
         pc.ncols[i] = on ? std::min(64, p - 64 * k) : -1;
       }
-      hz::launch_cgs_slots(n, S, pc, true, false, c->partial_s, c->nrms, st);
+      hz::launch_cgs_slots(n, S, pc, true, false, c->partial_s, c->ticket, c->nrms, st);
     }
   }
   std::vector<double2> hb(size_t(2) * nch * S * 65);
@@ -1880,7 +1882,6 @@ hz_status block_step(hz_ctx* c, int j, int s, int kk, std::vector<cplx>& hcol, b
 hz_status block_batch(hz_ctx* c, int s, double tol, hz_rhs_info* info) {
   const int64_t n = c->n;
   const int m = c->restart;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   for (int i = 0; i < c->S; i++) c->slots[i].state = i < s ? hz_ctx::SLOT_RUN : hz_ctx::SLOT_FREE;
   std::vector<double> bn(s), rel(s, 0.0);
@@ -1906,9 +1907,8 @@ hz_status block_batch(hz_ctx* c, int s, double tol, hz_rhs_info* info) {
       const double2* Cb = c->Vb - int64_t(kk) * n;
       for (int i = 0; i < s; i++) {
         double2* wi = c->Wc + int64_t(i) * n;
-        hz::launch_cgs(n, kk, Cb, n, nullptr, wi, kk, c->partial, st);
-        hz::launch_reduce(c->partial, nb, kk, c->h1, st);
-        hz::launch_cgs(n, kk, Cb, n, c->h1, wi, 0, c->partial, st);
+        hz::launch_cgs(n, kk, Cb, n, nullptr, wi, true, c->partial, c->ticket, c->h1, st);
+        hz::launch_cgs(n, kk, Cb, n, c->h1, wi, false, c->partial, c->ticket, c->nrm, st);
         hz::launch_combo(n, kk, c->Ux, n, 0, nullptr, n, c->h1, 1, c->Xc + int64_t(i) * n, n, 1.0, true, st);
       }
     }
@@ -2498,6 +2498,7 @@ static hz_status populate(hz_ctx* c, hz::HostProblem& P, int order, const hz_opt
   SETUP_TRY(dalloc(c, &c->y, n));
   SETUP_TRY(dalloc(c, &c->t, n));
   SETUP_TRY(dalloc(c, &c->partial, int64_t(hz::cgs_blocks()) * 65));
+  SETUP_TRY(upload(c, &c->ticket, std::vector<unsigned int>(16, 0u)));
   SETUP_TRY(dalloc(c, &c->h1, 65));
   SETUP_TRY(dalloc(c, &c->h2, 65));
   SETUP_TRY(dalloc(c, &c->nrm, 65));
@@ -2737,14 +2738,12 @@ extern "C" hz_status hz_profile(hz_ctx* c, int32_t reps, hz_profile_out* out) {
   const int64_t n = c->n;
   const int m = c->restart;
   const int jj = std::max(1, m / 2);
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   // finite, normal test data in the vectors and the Krylov basis
   CU(cudaMemsetAsync(c->V, 0x3f, size_t(n) * (m + 1) * 16, st));
   CU(cudaMemsetAsync(c->w, 0x3f, size_t(n) * 16, st));
   CU(cudaMemsetAsync(c->b, 0x3f, size_t(n) * 16, st));
-  hz::launch_cgs(n, 0, c->V, n, nullptr, c->b, 0, c->partial, st);
-  hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+  hz::launch_cgs(n, 0, c->V, n, nullptr, c->b, false, c->partial, c->ticket, c->nrm, st);
   hz::launch_init_cycle(c->nrm, c->g, m, c->scal + 2, c->scal + 3, st);
   c->h_pin[6] = 1.0;
   CU(cudaMemcpyAsync(c->scal + 4, c->h_pin + 6, sizeof(double), cudaMemcpyHostToDevice, st));
@@ -2763,26 +2762,19 @@ extern "C" hz_status hz_profile(hz_ctx* c, int32_t reps, hz_profile_out* out) {
       case HZ_PH_LOCAL_SOLVE: hz::launch_solve(c->loc, st); break;
       case HZ_PH_PROLONG: hz::launch_prolong(c->loc, c->levels == 2 ? c->y : nullptr, c->t, st); break;
       case HZ_PH_CGS2:
-        hz::launch_cgs(n, jj + 1, c->V, n, nullptr, c->w, jj + 1, c->partial, st);
-        hz::launch_reduce(c->partial, nb, jj + 1, c->h1, st);
-        hz::launch_cgs(n, jj + 1, c->V, n, c->h1, c->w, jj + 1, c->partial, st);
-        hz::launch_reduce(c->partial, nb, jj + 1, c->h2, st);
-        hz::launch_cgs(n, jj + 1, c->V, n, c->h2, c->w, 0, c->partial, st);
-        hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+        hz::launch_cgs(n, jj + 1, c->V, n, nullptr, c->w, true, c->partial, c->ticket, c->h1, st);
+        hz::launch_cgs(n, jj + 1, c->V, n, c->h1, c->w, true, c->partial, c->ticket, c->h2, st);
+        hz::launch_cgs(n, jj + 1, c->V, n, c->h2, c->w, false, c->partial, c->ticket, c->nrm, st);
         break;
       case HZ_PH_PRECOND: apply_prec(c, c->b, c->t); break;
       case HZ_PH_ITERATION: {
         double2* zj = c->Zs + int64_t(jj) * n;
         apply_prec(c, c->V + int64_t(jj) * n, zj);
         hz::launch_spmv(n, c->d_rp, c->d_ci, c->d_A, zj, nullptr, c->w, st);
-        hz::launch_cgs(n, jj + 1, c->V, n, nullptr, c->w, jj + 1, c->partial, st);
-        hz::launch_reduce(c->partial, nb, jj + 1, c->h1, st);
-        hz::launch_cgs(n, jj + 1, c->V, n, c->h1, c->w, jj + 1, c->partial, st);
-        hz::launch_reduce(c->partial, nb, jj + 1, c->h2, st);
-        hz::launch_cgs(n, jj + 1, c->V, n, c->h2, c->w, 0, c->partial, st);
-        hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
-        hz::launch_givens(0, m, c->H, c->cs, c->sn, c->g, c->h1, c->h2, c->nrm, c->scal + 4, c->scal, c->brk,
-                          c->scal + 1, st);
+        hz::launch_cgs(n, jj + 1, c->V, n, nullptr, c->w, true, c->partial, c->ticket, c->h1, st);
+        hz::launch_cgs(n, jj + 1, c->V, n, c->h1, c->w, true, c->partial, c->ticket, c->h2, st);
+        const hz::SlotGivens gv = givens_args(0, m, c->H, c->cs, c->sn, c->g, c->h1, c->h2, c->nrm, c->scal, 4, c->brk);
+        hz::launch_cgs(n, jj + 1, c->V, n, c->h2, c->w, false, c->partial, c->ticket, c->nrm, st, &gv);
         hz::launch_scale(n, c->w, c->scal + 1, c->V + int64_t(jj + 1) * n, st);
         break;
       }
@@ -2929,16 +2921,12 @@ extern "C" hz_status hz_cgs2(hz_ctx* c, const void* V, int64_t ldv, int32_t ncol
   if (ncols < 1 || ncols > 64) return fail(c, HZ_ERR_ARG, "ncols must be in [1, 64]");
   if (ldv < c->n) return fail(c, HZ_ERR_ARG, "ldv < n");
   const int64_t n = c->n;
-  const int nb = hz::cgs_blocks();
   cudaStream_t st = c->st;
   const double2* Vd = (const double2*)V;
   double2* wd = (double2*)w;
-  hz::launch_cgs(n, ncols, Vd, ldv, nullptr, wd, ncols, c->partial, st);
-  hz::launch_reduce(c->partial, nb, ncols, c->h1, st);
-  hz::launch_cgs(n, ncols, Vd, ldv, c->h1, wd, ncols, c->partial, st);
-  hz::launch_reduce(c->partial, nb, ncols, c->h2, st);
-  hz::launch_cgs(n, ncols, Vd, ldv, c->h2, wd, 0, c->partial, st);
-  hz::launch_reduce(c->partial, nb, 0, c->nrm, st);
+  hz::launch_cgs(n, ncols, Vd, ldv, nullptr, wd, true, c->partial, c->ticket, c->h1, st);
+  hz::launch_cgs(n, ncols, Vd, ldv, c->h1, wd, true, c->partial, c->ticket, c->h2, st);
+  hz::launch_cgs(n, ncols, Vd, ldv, c->h2, wd, false, c->partial, c->ticket, c->nrm, st);
   hz::launch_add2(ncols, c->h1, c->h2, (double2*)h, st);
   CU(cudaMemcpyAsync(c->h_pin + 5, &c->nrm[64].x, sizeof(double), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));

@@ -145,9 +145,10 @@ struct SlotCols {
   int64_t o[16];
 };
 
-// Per-slot operands of the slot-batched CGS2 passes (ncols < 0: empty slot).
+// Per-slot operands of the CGS passes (ncols < 0: empty slot).
 struct SlotCgs {
-  const double2* V[16];       // the slot's basis, column-major, leading dimension n
+  int64_t ld;                 // leading dimension of the bases
+  const double2* V[16];       // the slot's basis, column-major
   double2* w[16];
   const double2* h[16];       // coefficients of the update pass
   int ncols[16];
@@ -156,11 +157,16 @@ struct SlotCgs {
 // Per-slot Givens update: slot i's arrays at fixed strides from these bases (j < 0: skip).
 struct SlotGivens {
   int m;
+  int bn_off;                      // |b| at scal[bn_off]
+  // GCRO-DR (one slot): the Arnoldi coefficients start at h1/h2[off], after those of the recycled
+  // space; raw_h / raw_b (optional) keep the unrotated column and those coefficients
+  int off, ldb;
+  double2 *raw_h, *raw_b;
   int j[16];
   double2 *H, *sn, *g;
   double* cs;
   const double2 *h1, *h2, *nrm;    // S x 65 each
-  double* scal;                    // S x 8: estimate, 1 / h_{j+1,j}, ..., |b| at 4
+  double* scal;                    // S x 8: estimate, 1 / h_{j+1,j}, ..., |b| at bn_off
   int* brk;
 };
 
@@ -224,10 +230,11 @@ void launch_interleave(int64_t n, int S, const SlotCols& off, const double2* bas
 void launch_deinterleave(int64_t n, int S, const SlotCols& off, const double2* inter, double2* base, cudaStream_t st);
 void launch_point_rhs(const PointRhs& p, double2* out, cudaStream_t st);
 void launch_interleave_put(int64_t n, int S, int i, const double2* col, double2* inter, cudaStream_t st);
-// out (S x 65): per slot, maxpy pass (w -= V h) and / or dot pass (V^H w, |w|^2), reduced.
-void launch_cgs_slots(int64_t n, int S, const SlotCgs& p, bool maxpy, bool dots, double2* partial, double2* out,
-                      cudaStream_t st);
-void launch_givens_slots(int S, const SlotGivens& p, cudaStream_t st);
+// CGS pass (cgs.cu): w -= V h if maxpy, then the dots V^H w if dots, always |w|^2; out (S x 65):
+// the dots per slot, |w|^2 at 64.  ticket: S zeroed words (kept zero) for the short vectors' fused
+// sum, or null; givens: the Givens update that follows, or null.
+void launch_cgs_slots(int64_t n, int S, const SlotCgs& p, bool maxpy, bool dots, double2* partial,
+                      unsigned int* ticket, double2* out, cudaStream_t st, const SlotGivens* givens = nullptr);
 void launch_scale_slots(int64_t n, int S, const SlotScale& p, cudaStream_t st);
 void launch_spmv_multi(int64_t n, int S, const int64_t* rp, const int32_t* ci, const double2* val, const double2* x,
                        const double2* sub, double2* y, cudaStream_t st);
@@ -239,13 +246,10 @@ void launch_spmv(int64_t n, const int64_t* rp, const int32_t* ci, const double2*
 void launch_spmv_real(int64_t n, const int64_t* rp, const int32_t* ci, const double* val, const double2* x,
                       double2* y, cudaStream_t st);
 int cgs_blocks();
-void launch_cgs(int64_t n, int ncols, const double2* V, int64_t ldv, const double2* h, double2* w,
-                int ndot, double2* partial, cudaStream_t st);
-void launch_reduce(const double2* partial, int nblk, int ncols, double2* out, cudaStream_t st);
-void launch_givens(int j, int m, double2* H, double* cs, double2* sn, double2* g, const double2* h1,
-                   const double2* h2, const double2* nrm, const double* bnorm, double* est, int* breakdown,
-                   double* invh, cudaStream_t st, int off = 0, double2* raw_h = nullptr, double2* raw_b = nullptr,
-                   int ldb = 0);
+// the same for one vector; h null: dots only
+void launch_cgs(int64_t n, int ncols, const double2* V, int64_t ldv, const double2* h, double2* w, bool dots,
+                double2* partial, unsigned int* ticket, double2* out, cudaStream_t st,
+                const SlotGivens* givens = nullptr);
 constexpr int kComboMaxCols = 80, kComboMaxOut = 16;
 void launch_combo(int64_t n, int nb1, const double2* B1, int64_t ld1, int nb2, const double2* B2, int64_t ld2,
                   const double2* coef, int nout, double2* out, int64_t ldo, double sign, bool accumulate,

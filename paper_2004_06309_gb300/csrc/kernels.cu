@@ -1220,243 +1220,10 @@ void launch_spmv_real(int64_t n, const int64_t* rp, const int32_t* ci, const dou
 }
 
 // ---------------------------------------------------------------------------
-// GMRES: fused CGS passes and small dense updates
+// GMRES vector updates (the orthogonalisation is in cgs.cu)
 // ---------------------------------------------------------------------------
 constexpr int kMaxCols = 64;
-constexpr int kPartStride = kMaxCols + 1;
-int cgs_blocks() { return 152 * 4; }
 
-// Multi-dot: partial[b][j] = sum over the block's rows of conj(V[r][j]) w[r] (j < ncols);
-// partial[b][64] = sum |w[r]|^2.  One warp per column, lanes over rows.
-__device__ __forceinline__ void mdot_block(int64_t n, int ncols, const double2* __restrict__ V, int64_t ldv,
-                                           const double2* __restrict__ w, double2* out, int64_t chunk, int bx) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t row0 = bx * chunk;
-  const int64_t row1 = min(n, row0 + chunk);
-  for (int j = wid; j < kMaxCols; j += 8) {
-    double2 acc = make_double2(0.0, 0.0);
-    if (j < ncols) {
-      const double2* col = V + int64_t(j) * ldv;
-#pragma unroll 4
-      for (int64_t r = row0 + lane; r < row1; r += 32) acc = cmadc(col[r], w[r], acc);
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) out[j] = acc;
-  }
-  if (wid == 0) {
-    double s = 0.0;
-    for (int64_t r = row0 + lane; r < row1; r += 32) {
-      const double2 v = w[r];
-      s = xfma(v.x, v.x, xfma(v.y, v.y, s));
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[kMaxCols] = make_double2(s, 0.0);
-  }
-}
-__global__ void __launch_bounds__(256) k_mdot(int64_t n, int ncols, const double2* __restrict__ V, int64_t ldv,
-                                              const double2* __restrict__ w, double2* partial, int64_t chunk) {
-  mdot_block(n, ncols, V, ldv, w, partial + int64_t(blockIdx.x) * kPartStride, chunk, blockIdx.x);
-}
-
-// Multi-axpy: w[r] -= sum_j V[r][j] h[j]; partial[b][64] = sum |w[r]|^2 (new w).
-__device__ __forceinline__ void maxpy_block(int64_t n, int ncols, const double2* __restrict__ V, int64_t ldv,
-                                            const double2* __restrict__ h, double2* w, double2* out, int64_t chunk,
-                                            int bx) {
-  __shared__ double2 hs[kMaxCols];
-  __shared__ double red[8];
-  for (int j = threadIdx.x; j < ncols; j += blockDim.x) hs[j] = h[j];
-  __syncthreads();
-  const int64_t row0 = bx * chunk;
-  const int64_t row1 = min(n, row0 + chunk);
-  double s = 0.0;
-  for (int64_t r = row0 + threadIdx.x; r < row1; r += blockDim.x) {
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 4
-    for (int j = 0; j < ncols; j++) acc = cmad(V[r + int64_t(j) * ldv], hs[j], acc);
-    const double2 v = csub(w[r], acc);
-    w[r] = v;
-    s = xfma(v.x, v.x, xfma(v.y, v.y, s));
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int q = 0; q < 8; q++) t += red[q];
-    out[kMaxCols] = make_double2(t, 0.0);
-  }
-}
-__global__ void __launch_bounds__(256) k_maxpy(int64_t n, int ncols, const double2* __restrict__ V, int64_t ldv,
-                                               const double2* __restrict__ h, double2* w, double2* partial,
-                                               int64_t chunk) {
-  maxpy_block(n, ncols, V, ldv, h, w, partial + int64_t(blockIdx.x) * kPartStride, chunk, blockIdx.x);
-}
-
-static int64_t cgs_chunk(int64_t n) {
-  const int nb = cgs_blocks();
-  int64_t chunk = (n + nb - 1) / nb;
-  return (chunk + 31) / 32 * 32;
-}
-
-// ndot > 0 and h == null: dots of w with V (and |w|^2); h != null: w -= V h (and |w|^2),
-// followed by the dots of the updated w when ndot > 0.
-void launch_cgs(int64_t n, int ncols, const double2* V, int64_t ldv, const double2* h, double2* w, int ndot,
-                double2* partial, cudaStream_t st) {
-  const int nb = cgs_blocks();
-  const int64_t chunk = cgs_chunk(n);
-  if (h) {
-    HZ_COUNT();
-    k_maxpy<<<nb, 256, 0, st>>>(n, ncols, V, ldv, h, w, partial, chunk);
-  }
-  if (ndot > 0 || !h) {
-    HZ_COUNT();
-    k_mdot<<<nb, 256, 0, st>>>(n, ndot, V, ldv, w, partial, chunk);
-  }
-}
-
-// out[j] = sum over blocks of partial[b][j]; one CTA per j, fixed-order tree.
-__device__ __forceinline__ void reduce_block(const double2* partial, int nblk, double2* out, int j) {
-  __shared__ double2 red[256];
-  double2 s = make_double2(0.0, 0.0);
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s = cadd(s, partial[int64_t(b) * kPartStride + j]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + o]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[j] = red[0];
-}
-__global__ void __launch_bounds__(256) k_reduce(const double2* partial, int nblk, double2* out) {
-  reduce_block(partial, nblk, out, blockIdx.x);
-}
-
-// Sums all 65 slots (columns and the norm slot 64).
-void launch_reduce(const double2* partial, int nblk, int ncols, double2* out, cudaStream_t st) {
-  (void)ncols;
-  HZ_COUNT();
-  k_reduce<<<kMaxCols + 1, 256, 0, st>>>(partial, nblk, out);
-}
-
-// Complex Givens rotation zeroing b: rho = sqrt(|a|^2+|b|^2), c = |a|/rho,
-// s = (a/|a|) conj(b)/rho; a = 0 gives c = 0, s = 1.
-__device__ void givens_cs(double2 a, double2 b, double& c, double2& s) {
-  const double aa = sqrt(a.x * a.x + a.y * a.y);
-  if (aa == 0.0) {
-    c = 0.0;
-    s = make_double2(1.0, 0.0);
-    return;
-  }
-  const double bb = sqrt(b.x * b.x + b.y * b.y);
-  const double rho = sqrt(aa * aa + bb * bb);
-  c = aa / rho;
-  const double2 u = make_double2(a.x / aa, a.y / aa);
-  const double2 bc = make_double2(b.x / rho, -b.y / rho);
-  s = cmul(u, bc);
-}
-
-// Givens update of column j of the Hessenberg matrix.  The CGS coefficients of the
-// Arnoldi basis start at h1/h2[off] (the first `off` are those of a recycled space,
-// GCRO-DR); raw_h / raw_b (optional) keep the unrotated column and those `off`
-// coefficients for the cycle-end harmonic Ritz problem.
-__device__ void k_givens_body(int j, int m, double2* H, double* cs, double2* sn, double2* g, const double2* h1,
-                              const double2* h2, const double2* nrm, const double* bnorm_p, double* est,
-                              int* breakdown, double* invh, int off = 0, double2* raw_h = nullptr,
-                              double2* raw_b = nullptr, int ldb = 0) {
-  if (threadIdx.x != 0) return;
-  const double bnorm = *bnorm_p;
-  double2* col = H + int64_t(j) * (m + 1);
-  for (int i = 0; i <= j; i++) col[i] = cadd(h1[off + i], h2[off + i]);
-  const double w0 = sqrt(h1[kMaxCols].x);
-  const double hn = sqrt(nrm[kMaxCols].x);
-  col[j + 1] = make_double2(hn, 0.0);
-  if (raw_h) {
-    for (int i = 0; i <= j + 1; i++) raw_h[int64_t(j) * (m + 1) + i] = col[i];
-    for (int i = 0; i < off; i++) raw_b[int64_t(j) * ldb + i] = cadd(h1[i], h2[i]);
-  }
-  for (int i = 0; i < j; i++) {
-    const double2 a = col[i], b = col[i + 1];
-    const double2 sc = make_double2(sn[i].x, -sn[i].y);
-    col[i] = cadd(make_double2(cs[i] * a.x, cs[i] * a.y), cmul(sn[i], b));
-    col[i + 1] = csub(make_double2(cs[i] * b.x, cs[i] * b.y), cmul(sc, a));
-  }
-  double c;
-  double2 s;
-  givens_cs(col[j], col[j + 1], c, s);
-  cs[j] = c;
-  sn[j] = s;
-  col[j] = cadd(make_double2(c * col[j].x, c * col[j].y), cmul(s, col[j + 1]));
-  col[j + 1] = make_double2(0.0, 0.0);
-  const double2 gj = g[j];
-  const double2 sc = make_double2(-s.x, s.y);   // -conj(s)
-  g[j + 1] = cmul(sc, gj);
-  g[j] = make_double2(c * gj.x, c * gj.y);
-  *est = sqrt(g[j + 1].x * g[j + 1].x + g[j + 1].y * g[j + 1].y) / bnorm;
-  *breakdown = (hn <= 1e-14 * w0) ? 1 : 0;
-  *invh = 1.0 / hn;
-}
-__global__ void k_givens(int j, int m, double2* H, double* cs, double2* sn, double2* g, const double2* h1,
-                         const double2* h2, const double2* nrm, const double* bnorm_p, double* est,
-                         int* breakdown, double* invh, int off, double2* raw_h, double2* raw_b, int ldb) {
-  if (blockIdx.x != 0) return;
-  k_givens_body(j, m, H, cs, sn, g, h1, h2, nrm, bnorm_p, est, breakdown, invh, off, raw_h, raw_b, ldb);
-}
-
-void launch_givens(int j, int m, double2* H, double* cs, double2* sn, double2* g, const double2* h1,
-                   const double2* h2, const double2* nrm, const double* bnorm, double* est, int* breakdown,
-                   double* invh, cudaStream_t st, int off, double2* raw_h, double2* raw_b, int ldb) {
-  HZ_COUNT();
-  k_givens<<<1, 32, 0, st>>>(j, m, H, cs, sn, g, h1, h2, nrm, bnorm, est, breakdown, invh, off, raw_h, raw_b, ldb);
-}
-
-// ---------------------------------------------------------------------------
-// The same CGS2 / Givens / scaling steps for the S slots of a pseudo-block solve in one
-// launch each (grid.y = slot); each slot's arithmetic is the single-vector kernels'
-// block for block, so its results do not depend on the other slots.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_cgs_slots(int64_t n, SlotCgs p, double2* partial, int64_t chunk,
-                                                   int mode) {
-  const int i = blockIdx.y, nb = gridDim.x;
-  if (p.ncols[i] < 0) return;
-  double2* out = partial + (int64_t(i) * nb + blockIdx.x) * kPartStride;
-  if (mode == 0)
-    mdot_block(n, p.ncols[i], p.V[i], n, p.w[i], out, chunk, blockIdx.x);
-  else
-    maxpy_block(n, p.ncols[i], p.V[i], n, p.h[i], p.w[i], out, chunk, blockIdx.x);
-}
-__global__ void __launch_bounds__(256) k_reduce_slots(const double2* partial, int nblk, SlotCgs p, double2* out) {
-  const int i = blockIdx.y;
-  if (p.ncols[i] < 0) return;
-  reduce_block(partial + int64_t(i) * nblk * kPartStride, nblk, out + int64_t(i) * kPartStride, blockIdx.x);
-}
-void launch_cgs_slots(int64_t n, int S, const SlotCgs& p, bool maxpy, bool dots, double2* partial, double2* out,
-                      cudaStream_t st) {
-  const int nb = cgs_blocks();
-  const int64_t chunk = cgs_chunk(n);
-  if (maxpy) {
-    HZ_COUNT();
-    k_cgs_slots<<<dim3(nb, S), 256, 0, st>>>(n, p, partial, chunk, 1);
-  }
-  if (dots) {
-    HZ_COUNT();
-    k_cgs_slots<<<dim3(nb, S), 256, 0, st>>>(n, p, partial, chunk, 0);
-  }
-  HZ_COUNT();
-  k_reduce_slots<<<dim3(kMaxCols + 1, S), 256, 0, st>>>(partial, nb, p, out);
-}
-__global__ void k_givens_slots(SlotGivens p) {
-  const int i = blockIdx.x;
-  if (p.j[i] < 0) return;
-  const int m = p.m;
-  k_givens_body(p.j[i], m, p.H + int64_t(i) * (m + 1) * m, p.cs + int64_t(i) * m, p.sn + int64_t(i) * m,
-                p.g + int64_t(i) * (m + 1), p.h1 + int64_t(i) * kPartStride, p.h2 + int64_t(i) * kPartStride,
-                p.nrm + int64_t(i) * kPartStride, p.scal + int64_t(i) * 8 + 4, p.scal + int64_t(i) * 8,
-                p.brk + i, p.scal + int64_t(i) * 8 + 1);
-}
-void launch_givens_slots(int S, const SlotGivens& p, cudaStream_t st) {
-  HZ_COUNT();
-  k_givens_slots<<<S, 32, 0, st>>>(p);
-}
 __global__ void k_scale_slots(int64_t n, SlotScale p) {
   const int i = blockIdx.y;
   if (!p.out[i]) return;
@@ -1531,17 +1298,6 @@ void launch_scale(int64_t n, const double2* w, const double* s, double2* out, cu
   k_scale<<<grid_for(n, 256), 256, 0, st>>>(n, w, s, out);
 }
 
-// y = R^{-1} g (upper triangular k x k of the rotated Hessenberg matrix)
-__global__ void k_backsub(int k, const double2* H, int ldh, const double2* g, double2* y) {
-  if (threadIdx.x != 0) return;
-  for (int i = k - 1; i >= 0; i--) {
-    double2 s = g[i];
-    for (int l = i + 1; l < k; l++) s = cmsub(H[i + int64_t(l) * ldh], y[l], s);
-    const double2 d = H[i + int64_t(i) * ldh];
-    y[i] = cmul(s, cinv(d));
-  }
-}
-
 __global__ void k_gemv_add(int64_t n, int k, const double2* y, const double2* Zs, int64_t ldz, double2* x) {
   __shared__ double2 ys[kMaxCols];
   for (int j = threadIdx.x; j < k; j += blockDim.x) ys[j] = y[j];
@@ -1555,14 +1311,6 @@ __global__ void k_gemv_add(int64_t n, int k, const double2* y, const double2* Zs
 
 // x += Zs[:, 0:k) y (k <= 64)
 void launch_gemv_add(int64_t n, int k, const double2* y, const double2* Zs, int64_t ldz, double2* x, cudaStream_t st) {
-  HZ_COUNT();
-  k_gemv_add<<<grid_for(n, 256), 256, 0, st>>>(n, k, y, Zs, ldz, x);
-}
-
-void launch_update_x(int64_t n, int k, const double2* H, int ldh, const double2* g, double2* y, const double2* Zs,
-                     int64_t ldz, double2* x, cudaStream_t st) {
-  HZ_COUNT();
-  k_backsub<<<1, 32, 0, st>>>(k, H, ldh, g, y);
   HZ_COUNT();
   k_gemv_add<<<grid_for(n, 256), 256, 0, st>>>(n, k, y, Zs, ldz, x);
 }

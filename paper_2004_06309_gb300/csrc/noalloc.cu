@@ -93,12 +93,10 @@ extern "C" hz_status hz_cgs2_noalloc(const void* V, int64_t n, int64_t ldv, int3
   double2* wd = static_cast<double2*>(w);
   // Every slot read below is written earlier in the same call, so nothing from a
   // previous call (which leaves its values in the array) leaks into this one.
-  hz::launch_cgs(n, ncols, Vd, ldv, nullptr, wd, ncols, partial, cs);
-  hz::launch_reduce(partial, kBlocks, ncols, h1, cs);
-  hz::launch_cgs(n, ncols, Vd, ldv, h1, wd, ncols, partial, cs);
-  hz::launch_reduce(partial, kBlocks, ncols, h2, cs);
-  hz::launch_cgs(n, ncols, Vd, ldv, h2, wd, 0, partial, cs);
-  hz::launch_reduce(partial, kBlocks, 0, nrm, cs);
+  // no ticket words in the static scratch: every pass sums its blocks in a launch of its own
+  hz::launch_cgs(n, ncols, Vd, ldv, nullptr, wd, true, partial, nullptr, h1, cs);
+  hz::launch_cgs(n, ncols, Vd, ldv, h1, wd, true, partial, nullptr, h2, cs);
+  hz::launch_cgs(n, ncols, Vd, ldv, h2, wd, false, partial, nullptr, nrm, cs);
   hz::launch_add2(ncols, h1, h2, static_cast<double2*>(h), cs);
   k_sqrt_norm<<<1, 32, 0, cs>>>(nrm, static_cast<double*>(wnorm));
   const cudaError_t e = cudaGetLastError();
