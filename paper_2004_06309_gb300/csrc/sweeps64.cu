@@ -11,8 +11,8 @@
 //   * the right-hand side of a task is written in digits too, with one exponent per task
 //     and right-hand side;
 //   * a digit product sum runs on mma.sync m16n8k16 (f16 in, f32 accumulators): a digit and
-//     a product of digits are exact, and at most 8 digit pairs x 64 columns x 2 products of
-//     at most 2^14 meet in one accumulator, at most 2^24, so every sum is exact too.
+//     a product of digits are exact, and at most 8 digit pairs x 128 columns of products of
+//     at most 2^14 meet in one accumulator: at most 2^24, so every sum is exact too.
 //     Digit pairs (i, j) with i + j <= 7 are kept; what is dropped is below 2^-59 (rms) of
 //     the largest product for 64 columns.
 // The digits of one operand hold 62 bits below the row's largest entry, against the 53 of a
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
     }
     step_single(raw, bre, bim, (8 * s + t) * kPairStride + g + 7, c);
     issue(s + kRing * CG, slot);                                         // the slot's entries are in use above
-    if ((it & 3) == 3) flush_single(c, tot);                             // at most 64 columns per accumulator
+    if ((it & 7) == 7) flush_single(c, tot);                             // at most 128 columns per accumulator
   }
   flush_single(c, tot);
   const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
     }
     step_single(raw, vre, vim, (8 * s + t) * kPairStride + g + 7, c);
     issue(s + 2 * kRing, slot);
-    if ((it & 3) == 3) flush_single(c, tot);
+    if ((it & 7) == 7) flush_single(c, tot);
   }
   flush_single(c, tot);
   const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
@@ -510,9 +510,10 @@ __device__ __forceinline__ void block_exponents(const double2* src, int cnt, int
 
 }  // namespace
 
-// columns (forward) or rows (backward) whose digits are in shared memory at once: 64 per
-// group of steps, so that no accumulator takes more
-template <int KG> constexpr int kMultiKb = 16 * (KG > 4 ? KG : 4);
+// columns (forward) or rows (backward) whose digits are in shared memory at once, at most 128 per
+// group of steps, so that no accumulator takes more.  Each such block costs three barriers, the
+// conversion and a flush (20 FP64 instructions a warp), so it is as long as a supernode is wide.
+template <int S> constexpr int kMultiKb = S == 4 ? 256 : 128;
 template <int S> constexpr int kMultiPairStride = 16 * S + 8;     // words; 8 t mod 32 differ
 
 // Forward: 16 MT rows x S right-hand sides per task; 8 warps = S / 4 groups of four
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
                                                        const uint32_t* wpos, const double2* panels,
                                                        const int16_t* rexp, const double2* tin, double2* zout,
                                                        double2* u, int kpad) {
-  constexpr int NT = S / 4, KG = 8 / (NT * MT), KB = kMultiKb<KG>, PS = kMultiPairStride<S>, RT = 16 * MT;
+  constexpr int NT = S / 4, KG = 8 / (NT * MT), KB = kMultiKb<S>, PS = kMultiPairStride<S>, RT = 16 * MT;
   static_assert(NT * MT * KG == 8, "eight warps");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* b1 = reinterpret_cast<double2*>(smem_raw);                    // kpad x S
@@ -569,7 +570,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
     int* exb = ex[blk & 1];
     block_exponents<S, false>(b1 + j0 * S, min(KB, k - j0), exb, nonfin, nullptr);
     __syncthreads();
-    put_digits_multi<S, false>(bd, PS, b1 + j0 * S, min(KB, k - j0), KB, exb, nullptr);
+    put_digits_multi<S, false>(bd, PS, b1 + j0 * S, min(KB, k - j0), min(KB, (jend - j0 + 15) / 16 * 16), exb, nullptr);
     if (tid < S) ex[(blk + 1) & 1][tid] = 1;
     __syncthreads();
     for (int s = j0 / 16 + kg; s < (j0 + KB) / 16 && 16 * s < jend; s += KG) {
@@ -603,7 +604,7 @@ __global__ void __launch_bounds__(256) k_bwd_dig_multi(const int4* tasks, const 
                                                        const double2* panels, const int16_t* rexp,
                                                        const double2* zin, double2* x, double2* partial,
                                                        const int4* fins, unsigned int* counters) {
-  constexpr int NT = S / 4, KG = 4 / NT, KB = 64, PS = kMultiPairStride<S>, ROWS = kMultiBwdRows;
+  constexpr int NT = S / 4, KG = 4 / NT, KB = kMultiBwdRows, PS = kMultiPairStride<S>, ROWS = kMultiBwdRows;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* vec = reinterpret_cast<double2*>(smem_raw);                   // ROWS x S; then KG x 32 x S partial sums
   uint32_t* bd = reinterpret_cast<uint32_t*>(vec + ROWS * S);            // KB / 2 x PS
@@ -664,7 +665,7 @@ __global__ void __launch_bounds__(256) k_bwd_dig_multi(const int4* tasks, const 
     const int nr = min(KB, cnt - q0);
     block_exponents<S, true>(vec + q0 * S, nr, exb, nonfin, vex + q0);
     __syncthreads();
-    put_digits_multi<S, true>(bd, PS, vec + q0 * S, nr, KB, exb, vex + q0);
+    put_digits_multi<S, true>(bd, PS, vec + q0 * S, nr, (nr + 15) / 16 * 16, exb, vex + q0);
     if (tid < S) ex[(blk + 1) & 1][tid] = -4000;
     __syncthreads();
     for (int s = q0 / 16 + kg; s < (q0 + KB) / 16 && s < nst; s += KG) {
@@ -719,10 +720,10 @@ size_t fwd_smem(int kpad) { return kRingBytes + size_t(kpad) * 16 + size_t(kpad)
 size_t bwd_smem(int rpad) { return kRingBytes + size_t(rpad) * 20 + size_t(rpad) * kPairStride * 4; }
 template <int S, int MT> size_t fwd_multi_smem(int kpad) {
   constexpr int KG = 8 / (S / 4 * MT);
-  return size_t(kpad) * S * 16 + size_t(KG) * 16 * MT * S * 16 + size_t(kMultiKb<KG> / 2) * kMultiPairStride<S> * 4;
+  return size_t(kpad) * S * 16 + size_t(KG) * 16 * MT * S * 16 + size_t(kMultiKb<S> / 2) * kMultiPairStride<S> * 4;
 }
 template <int S> size_t bwd_multi_smem() {
-  return size_t(kMultiBwdRows) * S * 16 + size_t(32) * kMultiPairStride<S> * 4;
+  return size_t(kMultiBwdRows) * S * 16 + size_t(kMultiBwdRows / 2) * kMultiPairStride<S> * 4;
 }
 template <typename K> void allow_smem(K kern) {
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
