@@ -192,6 +192,7 @@ std::vector<double2> to_d2(const std::vector<cplx>& v) {
 // sweep_tasks (hz_options) forces wide (1) or narrow (2) shapes on every level.
 struct SweepPlan {
   std::vector<int> fwd_rt, bwd_rows;   // per level: forward task rows, backward chunk rows
+  std::vector<int> bwd_cb;             // 32-column blocks per backward task
   int32_t fwd_wide = 0, fwd_narrow = 0, bwd_wide = 0, bwd_narrow = 0;
   int64_t bwd_split = 0, tc_tiles = 0, tc_multi = 0;
   int32_t tc_kstages = 0, max_k = 0;
@@ -294,6 +295,7 @@ SweepPlan plan_sweeps(const TreeView& S, int precision, int bwd_rows, int sweep_
   const int wide = precision == 0 ? 64 : 256;
   sp.fwd_rt.assign(nlev, wide);
   sp.bwd_rows.assign(nlev, bwd_rows);
+  sp.bwd_cb.assign(nlev, 1);
   for (int l = 0; l < nlev; l++) {
     int64_t nf = 0, nbk = 0;
     for (int32_t q = S.lev_ptr[l]; q < S.lev_ptr[l + 1]; q++) {
@@ -306,6 +308,24 @@ SweepPlan plan_sweeps(const TreeView& S, int precision, int bwd_rows, int sweep_
     const bool narrow_b = sweep_tasks == 2 || (sweep_tasks == 0 && nbk < sparse);
     if (narrow_f) sp.fwd_rt[l] = precision == 0 ? 16 : 64;
     if (narrow_b) sp.bwd_rows[l] = std::min(bwd_rows, precision == 0 ? 64 : 128);
+    if (precision == 0 && sweep_tasks == 0) {
+      // complex128, wide levels: a task takes up to 256 rows (four 32-column blocks backward) while
+      // that leaves three waves of tasks (4 CTAs per SM), and gathers and converts its right-hand
+      // side once: subdomain sweeps 31.4 -> 28.9 ms on the 5 Hz workload, 3.83 -> 3.75 on the
+      // 349,461-dof survey model, few of whose levels have that many tasks
+      const int64_t enough = 3 * 4 * 152;
+      auto count = [&](int rows, int cb) {
+        int64_t t = 0;
+        for (int32_t q = S.lev_ptr[l]; q < S.lev_ptr[l + 1]; q++) {
+          const int s = S.lev_sn[q];
+          t += rows > 0 ? (S.sn_m[s] + rows - 1) / rows
+                        : int64_t(((S.sn_k[s] + 31) / 32 + cb - 1) / cb) * ((S.sn_m[s] + bwd_rows - 1) / bwd_rows);
+        }
+        return t;
+      };
+      while (!narrow_f && sp.fwd_rt[l] < 256 && count(2 * sp.fwd_rt[l], 0) >= enough) sp.fwd_rt[l] *= 2;
+      while (!narrow_b && sp.bwd_cb[l] < 4 && count(0, 2 * sp.bwd_cb[l]) >= enough) sp.bwd_cb[l] *= 2;
+    }
     if (S.lev_ptr[l + 1] == S.lev_ptr[l]) continue;
     // the launchers pick the narrow kernels by shape (forward rows; chunk <= 128 / 64 rows)
     (narrow_f ? sp.fwd_narrow : sp.fwd_wide)++;
@@ -337,8 +357,9 @@ hz_status build_sweep_tasks(hz_ctx* c, hz::FactorDev& F, const SweepPlan& sp) {
   std::vector<int2> fwd;
   std::vector<int4> bwd, bfin;
   std::vector<int64_t> fwd_ptr(nlev + 1), bwd_ptr(nlev + 1), bfin_ptr(nlev + 1);
-  int64_t max_bwd_level = 0;
+  int64_t max_bwd_level = 0;                           // partial sums: 32 per column block and chunk
   for (int l = 0; l < nlev; l++) {
+    int64_t parts = 0;
     fwd_ptr[l] = int64_t(fwd.size());
     bwd_ptr[l] = int64_t(bwd.size());
     bfin_ptr[l] = int64_t(bfin.size());
@@ -350,11 +371,13 @@ hz_status build_sweep_tasks(hz_ctx* c, hz::FactorDev& F, const SweepPlan& sp) {
       const int nch = (m + sp.bwd_rows[l] - 1) / sp.bwd_rows[l];
       for (int cb = 0; cb * 32 < k; cb++) {
         const int fin = int(bfin.size());          // global index: its counter and its record
-        bfin.push_back(make_int4(s, cb, int(int64_t(bwd.size()) - bwd_ptr[l]), nch));
-        for (int ch = 0; ch < nch; ch++) bwd.push_back(make_int4(s, cb, ch, fin));
+        bfin.push_back(make_int4(s, cb, int(parts), nch));
+        parts += nch;
+        if (cb % sp.bwd_cb[l] == 0)                // a task's column blocks have consecutive records
+          for (int ch = 0; ch < nch; ch++) bwd.push_back(make_int4(s, cb, ch, fin));
       }
     }
-    max_bwd_level = std::max(max_bwd_level, int64_t(bwd.size()) - bwd_ptr[l]);
+    max_bwd_level = std::max(max_bwd_level, parts);
   }
   fwd_ptr[nlev] = int64_t(fwd.size());
   bwd_ptr[nlev] = int64_t(bwd.size());
@@ -406,6 +429,7 @@ hz_status build_sweep_tasks(hz_ctx* c, hz::FactorDev& F, const SweepPlan& sp) {
   F.h_bwd_rows = new int[nlev];
   std::copy(sp.fwd_rt.begin(), sp.fwd_rt.end(), F.h_fwd_rt);
   std::copy(sp.bwd_rows.begin(), sp.bwd_rows.end(), F.h_bwd_rows);
+  F.h_bwd_cb = sp.bwd_cb;
   F.v_fwd_wide = sp.fwd_wide;
   F.v_fwd_narrow = sp.fwd_narrow;
   F.v_bwd_wide = sp.bwd_wide;
@@ -671,7 +695,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
         sc.enter(gs, int64_t(cbt.size()));
         st.enter(gs, int64_t(tct.size()));
       }
-      for (int rb = 0; rb * 32 < r; rb++) wg.push_back(make_int2(s, rb));
+      for (int rb = 0; rb * (precision == 0 ? 32 : hz::kWgRows) < r; rb++) wg.push_back(make_int2(s, rb));
       if (precision == 0) {
         for (int ti = 0; ti * hz::kCbRows < r; ti++)       // column tiles that reach the row block's last row
           for (int tj = 0; tj * 16 < std::min(r, (ti + 1) * hz::kCbRows); tj++) cbt.push_back(make_int4(s, ti, tj, 0));

@@ -11,6 +11,7 @@ namespace hz {
 constexpr int kMaxSolveK = 448;
 constexpr int kMaxSolveK64 = 512;   // the same for the complex64 sweeps
 constexpr int kMultiBwdRows = 128;  // rows per backward task of the batched sweeps
+constexpr int kWgRows = 64;          // rows per complex64 off-diagonal task (32 in complex128)
 constexpr int kCbRows = 128;        // rows per complex128 Schur update task (of 16 columns)
 
 // One supernode of a batched multifrontal factorisation (64 bytes).
@@ -74,7 +75,7 @@ struct FactorDev {
   unsigned int* bwd_counters = nullptr;  // one per bfin task: partial-sum CTAs done (reset by the last)
   void* bwd_partial = nullptr;   // 32 values per backward partial task (max over levels)
   int2* ea_tasks = nullptr;      // (child sn, col block)
-  int2* wg_tasks = nullptr;      // (sn, row block of the off-diagonal part)
+  int2* wg_tasks = nullptr;      // (sn, row block of the off-diagonal part: 32 rows, kWgRows in complex64)
   int4* cb_tasks = nullptr;      // complex128: (sn, kCbRows-row block, 16-col tile, 0)
   int4* tc_tasks = nullptr;      // complex64 path: (sn, 128-row tile, 128-col tile, 0), tensor-core Schur update
   int64_t* h_tc_ptr = nullptr;   // nlev + 1 (host)
@@ -99,6 +100,7 @@ struct FactorDev {
   // per solve level: widest supernode (rounded up to 16 columns), tallest one, and the rows
   // of the batched forward tasks
   std::vector<int> h_lev_k, h_lev_m, h_mfwd_rt;
+  std::vector<int> h_bwd_cb;          // per solve level: 32-column blocks per backward task
   std::vector<int> h_flev_k;          // per factor level: widest supernode
   int32_t max_slot = 0;
   // kernel variants of the schedule (host-side counts, reported through hz_stats)

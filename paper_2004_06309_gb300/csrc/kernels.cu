@@ -92,47 +92,105 @@ __global__ void __launch_bounds__(256) k_extend_add(const int2* tasks, const SnD
   }
 }
 
-// Off-diagonal block, 32 rows per task:
+// Off-diagonal panel of a complex64 supernode, kWgRows rows per task:
 //   W = F21 T^T  (= L21 D), saved to the level scratch for the Schur update,
 //   G = W D^{-1} T  (= F21 F11^{-1} = L21 L11^{-1}), written over F21.
-template <typename V>
-__global__ void __launch_bounds__(256) k_wg(const int2* tasks, const SnDev* sn, const int64_t* scr_off,
-                                            V* fronts, V* scratch) {
+// Bound: FP32 arithmetic.  A thread owns 8 rows x 4 columns; T is staged 16 columns (rows) at a
+// time, and a warp skips the stages that hold only zeros for its 16 columns.  One element per
+// thread and step, T read from global memory inside the loop, took 530 us per level on the
+// 349,461-dof survey model.  Every sum keeps that order.
+constexpr int kWgPitch = kWgRows + 2, kWgTPitch = kMaxK + 2;
+__global__ void __launch_bounds__(256, 2) k_wg32(const int2* tasks, const SnDev* sn, const int64_t* scr_off,
+                                                 float2* fronts, float2* scratch, int kpad) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* Fs = reinterpret_cast<float2*>(smem_raw);          // kpad x kWgPitch: F21, then L21
+  float2* Tt = Fs + kpad * kWgPitch;                         // 16 x kWgTPitch
+  __shared__ float2 di[kMaxK];
   const int2 t = tasks[blockIdx.x];
   const SnDev S = sn[t.x];
-  const int k = S.k, m = S.m, r = m - k;
-  V* Fs = reinterpret_cast<V*>(smem_raw);  // 32 x k, ld 32
-  V* Ws = Fs + 32 * k;
-  V* di = Ws + 32 * k;
-  V* F = fronts + S.frontoff;
-  const int R0 = t.y * 32;                 // first row within the off-diagonal part
-  const int nr = min(32, r - R0);
-  const int tid = threadIdx.x, rr = tid & 31, g = tid >> 5;
-  for (int e = tid; e < 32 * k; e += blockDim.x) {
-    const int i = e & 31, j = e >> 5;
-    Fs[e] = (i < nr) ? F[(k + R0 + i) + int64_t(j) * m] : czero<V>();
+  const int k = S.k, m = S.m, r = m - k, tid = threadIdx.x;
+  float2* F = fronts + S.frontoff;
+  const int R0 = t.y * kWgRows, nr = min(kWgRows, r - R0);
+  float2* F21 = F + k + R0;
+  // the warp's 16 columns: warps w and w + 4 share a scheduler, so the second four count down
+  // and each scheduler gets the same share of T's triangle
+  const int wid = tid >> 5, wj0 = 16 * (wid < 4 ? wid : 11 - wid);
+  const int rg = tid & 7, j0 = wj0 + 4 * ((tid >> 3) & 3);   // rows 8 rg .., columns j0 ..
+  const int K16 = (k + 15) / 16 * 16;
+  const float2 z = make_float2(0.f, 0.f);
+  for (int e = tid; e < K16 * kWgRows; e += 256) {
+    const int i = e % kWgRows, j = e / kWgRows;
+    Fs[j * kWgPitch + i] = (i < nr && j < k) ? F21[i + int64_t(j) * m] : z;
   }
-  for (int j = tid; j < k; j += blockDim.x) di[j] = F[j + int64_t(j) * m];
+  for (int j = tid; j < k; j += 256) di[j] = F[j + int64_t(j) * m];
+  float2 acc[8][4];
+  auto product = [&](int i0) {
+#pragma unroll 4
+    for (int ii = 0; ii < 16; ii++) {
+      const float4* a4 = reinterpret_cast<const float4*>(Fs + (i0 + ii) * kWgPitch + 8 * rg);
+      const float4* b4 = reinterpret_cast<const float4*>(Tt + ii * kWgTPitch + j0);
+      const float4 b0 = b4[0], b1 = b4[1];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const float4 a = a4[q];
+        const float2 x = make_float2(a.x, a.y), y = make_float2(a.z, a.w);
+        acc[2 * q][0] = cmad(x, make_float2(b0.x, b0.y), acc[2 * q][0]);
+        acc[2 * q][1] = cmad(x, make_float2(b0.z, b0.w), acc[2 * q][1]);
+        acc[2 * q][2] = cmad(x, make_float2(b1.x, b1.y), acc[2 * q][2]);
+        acc[2 * q][3] = cmad(x, make_float2(b1.z, b1.w), acc[2 * q][3]);
+        acc[2 * q + 1][0] = cmad(y, make_float2(b0.x, b0.y), acc[2 * q + 1][0]);
+        acc[2 * q + 1][1] = cmad(y, make_float2(b0.z, b0.w), acc[2 * q + 1][1]);
+        acc[2 * q + 1][2] = cmad(y, make_float2(b1.x, b1.y), acc[2 * q + 1][2]);
+        acc[2 * q + 1][3] = cmad(y, make_float2(b1.z, b1.w), acc[2 * q + 1][3]);
+      }
+    }
+  };
+  auto start = [&]() {
+#pragma unroll
+    for (int a = 0; a < 8; a++)
+#pragma unroll
+      for (int b = 0; b < 4; b++) acc[a][b] = j0 + b < K16 ? Fs[(j0 + b) * kWgPitch + 8 * rg + a] : z;
+  };
   __syncthreads();
-  for (int j = g; j < k; j += 8) {
-    V acc = Fs[rr + 32 * j];
-    for (int i = 0; i < j; i++) acc = cmad(Fs[rr + 32 * i], F[j + int64_t(i) * m], acc);
-    Ws[rr + 32 * j] = acc;
+  start();
+  for (int i0 = 0; i0 < k; i0 += 16) {                       // W: T(j, i), i < j
+    __syncthreads();
+    for (int e = tid; e < 16 * K16; e += 256) {
+      const int j = e % K16, i = i0 + e / K16;
+      Tt[(e / K16) * kWgTPitch + j] = (j < k && i < j) ? F[j + int64_t(i) * m] : z;
+    }
+    __syncthreads();
+    if (wj0 < K16 && wj0 + 15 > i0) product(i0);
   }
   __syncthreads();
-  V* W = scratch + scr_off[t.x];
-  for (int e = tid; e < 32 * k; e += blockDim.x) {
-    const int i = e & 31, j = e >> 5;
-    if (i < nr) W[(R0 + i) + int64_t(j) * r] = Ws[e];
-    Fs[e] = cmul(Ws[e], di[j]);             // L21
+  float2* W = scratch + scr_off[t.x];
+#pragma unroll
+  for (int b = 0; b < 4; b++) {
+    const int j = j0 + b;
+    if (j >= k) continue;
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+      const int i = 8 * rg + a;
+      if (i < nr) W[(R0 + i) + int64_t(j) * r] = acc[a][b];
+      Fs[j * kWgPitch + i] = cmul(acc[a][b], di[j]);         // L21
+    }
   }
   __syncthreads();
-  for (int j = g; j < k; j += 8) {
-    V acc = Fs[rr + 32 * j];
-    for (int i = j + 1; i < k; i++) acc = cmad(Fs[rr + 32 * i], F[i + int64_t(j) * m], acc);
-    if (rr < nr) F[(k + R0 + rr) + int64_t(j) * m] = acc;
+  start();
+  for (int i0 = 0; i0 < k; i0 += 16) {                       // G: T(i, j), i > j
+    __syncthreads();
+    for (int e = tid; e < 16 * K16; e += 256) {
+      const int ii = e % 16, i = i0 + ii, j = e / 16;
+      Tt[ii * kWgTPitch + j] = (i < k && i > j) ? F[i + int64_t(j) * m] : z;
+    }
+    __syncthreads();
+    if (wj0 < K16 && wj0 < i0 + 15) product(i0);
   }
+#pragma unroll
+  for (int b = 0; b < 4; b++)
+#pragma unroll
+    for (int a = 0; a < 8; a++)
+      if (j0 + b < k && 8 * rg + a < nr) F21[(8 * rg + a) + int64_t(j0 + b) * m] = acc[a][b];
 }
 
 // ---------------------------------------------------------------------------
@@ -166,6 +224,13 @@ __device__ __forceinline__ float tf32_rna(float x) {
   uint32_t y;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(x));
   return __uint_as_float(y);
+}
+// TF32 high parts and remainders of four values, stored as vectors
+__device__ __forceinline__ void tc_split(float4 v, float* hi, float* lo) {
+  const float4 h = make_float4(tf32_rna(v.x), tf32_rna(v.y), tf32_rna(v.z), tf32_rna(v.w));
+  *reinterpret_cast<float4*>(hi) = h;
+  *reinterpret_cast<float4*>(lo) =
+      make_float4(tf32_rna(v.x - h.x), tf32_rna(v.y - h.y), tf32_rna(v.z - h.z), tf32_rna(v.w - h.w));
 }
 // float offset of element (row r, k) in a 128 x 32 K-major tile of core matrices
 constexpr int kTcCols = 8;                      // complex columns per stage
@@ -274,27 +339,18 @@ __global__ void __launch_bounds__(256) k_cb_tc(const int4* tasks, const SnDev* s
     float* B1l = B1h + kTcTile;
     float* B2h = B1l + kTcTile;
     float* B2l = B2h + kTcTile;
+    // two complex columns fill a 16-byte core-matrix row: one conflict-free vector store per operand
 #pragma unroll
-    for (int q = 0; q < QH; q++) {
+    for (int q = 0; q < QH; q += 2) {
       const int i = kTcCols * st + QH * half + q;
-      const float2 a = av[q];
-      const float2 bv = i < k ? cmul(bw[q], dinv[i]) : make_float2(0.f, 0.f);
-      const int kk = 2 * (QH * half + q);
-      const int o0 = tc_off(row, kk), o1 = tc_off(row, kk + 1);
-      const float arh = tf32_rna(a.x), aih = tf32_rna(a.y);
-      const float brh = tf32_rna(bv.x), bih = tf32_rna(bv.y), nbih = tf32_rna(-bv.y);
-      Ah[o0] = arh;
-      Al[o0] = tf32_rna(a.x - arh);
-      Ah[o1] = aih;
-      Al[o1] = tf32_rna(a.y - aih);
-      B1h[o0] = brh;
-      B1l[o0] = tf32_rna(bv.x - brh);
-      B1h[o1] = nbih;
-      B1l[o1] = tf32_rna(-bv.y - nbih);
-      B2h[o0] = bih;
-      B2l[o0] = tf32_rna(bv.y - bih);
-      B2h[o1] = brh;
-      B2l[o1] = tf32_rna(bv.x - brh);
+      const float2 b0 = i < k ? cmul(bw[q], dinv[i]) : make_float2(0.f, 0.f);
+      const float2 b1 = i + 1 < k ? cmul(bw[q + 1], dinv[i + 1]) : make_float2(0.f, 0.f);
+      const int o = tc_off(row, 2 * (QH * half + q));
+      const float4 a = make_float4(av[q].x, av[q].y, av[q + 1].x, av[q + 1].y);
+      const float4 c1 = make_float4(b0.x, -b0.y, b1.x, -b1.y), c2 = make_float4(b0.y, b0.x, b1.y, b1.x);
+      tc_split(a, Ah + o, Al + o);
+      tc_split(c1, B1h + o, B1l + o);
+      tc_split(c2, B2h + o, B2l + o);
     }
     asm volatile("fence.proxy.async.shared::cta;");
     __syncthreads();
@@ -390,7 +446,6 @@ static unsigned split_for(int64_t nb, int64_t cols) {
   return unsigned(std::max<int64_t>(1, std::min(want, (cols + 7) / 8)));
 }
 
-static size_t wg_smem(int kmax, size_t vs) { return (size_t(64) * kmax + kmax) * vs; }
 
 // One tree level of one factorisation group (whole matrices whose fronts share the
 // workspace at once): each task list holds, per level, the groups' tasks in order.
@@ -434,8 +489,9 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
   if (we > wb) {
     if constexpr (sizeof(V) == 8) {
       HZ_COUNT();
-      k_wg<V><<<unsigned(we - wb), 256, wg_smem(maxk, sizeof(V)), st>>>(F.wg_tasks + wb, F.sn, F.scr_off, fronts,
-                                                                       scratch);
+      const int kpad = (maxk + 15) / 16 * 16;
+      k_wg32<<<unsigned(we - wb), 256, size_t(kpad * kWgPitch + 16 * kWgTPitch) * 8, st>>>(F.wg_tasks + wb, F.sn,
+                                                                                           F.scr_off, fronts, scratch, kpad);
     } else {
       launch_wg_dig(we - wb, maxk, F.wg_tasks + wb, F, fronts, scratch, status, st);
     }
@@ -460,7 +516,7 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
 static void set_attrs() {
   static const bool done = [] {
     cudaFuncSetAttribute(k_cb_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemFloats * int(sizeof(float)));
-    cudaFuncSetAttribute(k_wg<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_wg32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     return true;
   }();
   (void)done;

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) k_to_digits(const int2* tasks, const SnDe
   __shared__ int red[CG][RT];
   const int2 t = tasks[blockIdx.x];
   const SnDev S = sn[t.x];
-  const int rr = threadIdx.x % RT, cg = threadIdx.x / RT, r = t.y * RT + rr;
+  const int rr = threadIdx.x % RT, cg = threadIdx.x / RT, r = (t.y * gridDim.y + blockIdx.y) * RT + rr;
   const int jmax = r < S.m ? min(r, S.k) : 0;
   double2* P = panels + S.paneloff + r;
   int e = 1;
@@ -177,15 +177,16 @@ __global__ void __launch_bounds__(256) k_to_digits(const int2* tasks, const SnDe
 // the other blocks of the SM cover only in part.
 constexpr int kRing = 2;
 
-// Forward, 16 MT rows of one supernode per task (rows < k: z = D^{-1} (T b1); rows >= k:
-// u = children's updates - G b1); 4 warps = MT row tiles x 4 / MT groups of 16-column steps.
-// What the last step needs (children's updates of the update rows, D^{-1}, row exponents) is
-// loaded with the right-hand side.
+// Forward, npass blocks of 16 MT rows of one supernode per task (rows < k: z = D^{-1} (T b1); rows
+// >= k: u = children's updates - G b1); 4 warps = MT row tiles x 4 / MT groups of 16-column steps.
+// The right-hand side is gathered and converted once per task; the ring runs through the blocks,
+// and what a block's last step needs (children's updates of its rows, D^{-1}, row exponents) is
+// loaded one block ahead.
 template <int MT>
 __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnDev* sn, const uint32_t* cptr,
                                                     const uint32_t* wpos, const double2* panels,
                                                     const int16_t* rexp, const double2* tin, double2* zout,
-                                                    double2* u, int kpad) {
+                                                    double2* u, int kpad, int npass) {
   pdl_trigger();
   constexpr int CG = 4 / MT, RT = 16 * MT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -193,58 +194,80 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
   double* b1 = reinterpret_cast<double*>(ring + 4 * kRing * 256);        // kpad x 2
   uint32_t* bre = reinterpret_cast<uint32_t*>(b1 + 2 * kpad);            // kpad / 2 pairs x kPairStride
   uint32_t* bim = bre + (kpad / 2) * kPairStride;
-  __shared__ int64_t sums[CG][RT][2][2];                                 // [group][row][part][half]
+  __shared__ int64_t sums[2][CG][RT][2][2];                              // [block parity][group][row][part][half]
   __shared__ int red[4];
   const int2 tk = tasks[blockIdx.x];
   const SnDev S = sn[tk.x];
   const int k = S.k, m = S.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int g = lane >> 2, t = lane & 3, mt = wid % MT, cg = wid / MT;
   const uint32_t* cp = cptr + S.rowoff;
-  const int row0 = tk.y * RT + mt * 16;
-  const int ra = row0 + g, rb = ra + 8;
-  const int ja = ra < m ? min(ra, k) : 0, jb = rb < m ? min(rb, k) : 0;
-  const int nst = row0 < m ? (min(row0 + 15, k) + 15) / 16 : 0;          // 16-column steps of this tile
-  const int nfull = row0 + 15 < m ? min(row0, k) / 16 : 0;               // steps without a masked entry
+  const int base = tk.y * RT * npass, np = min(npass, (m - base + RT - 1) / RT);
   const uint4* P = reinterpret_cast<const uint4*>(panels + S.paneloff);
   uint4* myring = ring + wid * (kRing * 256) + lane;
-  auto issue = [&](int s, int slot) {
-    if (s < nst) {
+  auto nsteps = [&](int p) {                                             // 16-column steps of this warp's tile in block p
+    const int row0 = base + p * RT + mt * 16;
+    return row0 < m ? (min(row0 + 15, k) + 15) / 16 : 0;
+  };
+  int ip = 0, is = cg;                                                   // next step to copy: block, step
+  auto issue = [&](int slot) {
+    while (ip < np && is >= nsteps(ip)) {
+      ip++;
+      is = cg;
+    }
+    if (ip < np) {
+      const int ra = base + ip * RT + mt * 16 + g, rb = ra + 8;
+      const int ja = ra < m ? min(ra, k) : 0, jb = rb < m ? min(rb, k) : 0;
 #pragma unroll
       for (int q = 0; q < 4; q++) {
-        const int j = 16 * s + 2 * t + (q & 1) + 8 * (q >> 1);
+        const int j = 16 * is + 2 * t + (q & 1) + 8 * (q >> 1);
         const uint4* col = P + int64_t(j) * S.ld;
         if (j < ja) cp_async16(myring + slot * 256 + (2 * q) * 32, col + ra);
         if (j < jb) cp_async16(myring + slot * 256 + (2 * q + 1) * 32, col + rb);
       }
+      is += CG;
     }
     cp_async_commit();
   };
 #pragma unroll
-  for (int q = 0; q < kRing; q++) issue(cg + q * CG, q);
-  // this thread's result: row tid / 2 of the task, part tid & 1
-  const int r = tk.y * RT + (tid >> 1), pt = tid & 1;
-  const bool mine = tid < 2 * RT && r < m;
-  double2 dinv = make_double2(0.0, 0.0);
+  for (int q = 0; q < kRing; q++) issue(q);
+  // this thread's result of a block: row tid / 2, part tid & 1; where its child contributions lie
+  // and where its update goes
+  const int pt = tid & 1;
   int re = 0;
-  const bool upd = mine && r >= k;
-  if (mine) {
-    re = rexp[S.eoff + r];
-    if (r < k) dinv = panels[S.paneloff + r + int64_t(r) * S.ld];
-  }
-  // where this thread's child contributions lie and where its update goes
-  const uint32_t h0 = upd ? cp[r] : 0u, h1 = upd ? cp[r + 1] : 0u, uw = upd ? wpos[S.uoff + (r - k)] : 0u;
+  uint32_t h0 = 0, h1 = 0, uw = 0;
+  double2 dinv = make_double2(0.0, 0.0);
+  auto load_row = [&](int p) {
+    const int r = base + p * RT + (tid >> 1);
+    const bool mine = tid < 2 * RT && p < np && r < m, upd = mine && r >= k;
+    re = mine ? rexp[S.eoff + r] : 0;
+    if (mine && r < k) dinv = panels[S.paneloff + r + int64_t(r) * S.ld];
+    h0 = upd ? cp[r] : 0u;
+    h1 = upd ? cp[r + 1] : 0u;
+    uw = upd ? wpos[S.uoff + (r - k)] : 0u;
+  };
+  load_row(0);
   const uint32_t g0 = tid < 2 * k ? cp[tid >> 1] : 0u, g1 = tid < 2 * k ? cp[(tid >> 1) + 1] : 0u;
+  const int q1 = tid + 128;
+  const uint32_t g2 = q1 < 2 * k ? cp[q1 >> 1] : 0u, g3 = q1 < 2 * k ? cp[(q1 >> 1) + 1] : 0u;
   pdl_wait();
   const double *tind = reinterpret_cast<const double*>(tin + S.first), *ud = reinterpret_cast<const double*>(u);
   int e = 1;
-  for (int q = tid; q < 2 * k; q += 128) {
-    const int j = q >> 1;
-    const uint32_t c0 = q == tid ? g0 : cp[j], c1 = q == tid ? g1 : cp[j + 1];
-    const double a = add_updates_part(__ldcg(tind + q), ud, c0, c1, q & 1);
+  {
+    // the first two rounds (64 columns each) have their row pointers and load together
+    double a0 = 0.0, a1 = 0.0;
+    if (tid < 2 * k) a0 = __ldcg(tind + tid);
+    if (q1 < 2 * k) a1 = __ldcg(tind + q1);
+    a0 = add_updates_part(a0, ud, g0, g1, pt);
+    a1 = add_updates_part(a1, ud, g2, g3, pt);
+    if (tid < 2 * k) b1[tid] = a0;
+    if (q1 < 2 * k) b1[q1] = a1;
+    e = max(e, max(exp_field(a0), exp_field(a1)));
+  }
+  for (int q = tid + 256; q < 2 * k; q += 128) {
+    const double a = add_updates_part(__ldcg(tind + q), ud, cp[q >> 1], cp[(q >> 1) + 1], pt);
     b1[q] = a;
     e = max(e, exp_field(a));
   }
-  const double b2 = add_updates_part(0.0, ud, h0, h1, pt);
   const int E = block_max(e, red);                                       // publishes b1 too
   const int kp = (k + 15) / 16 * 16;
   for (int q = tid; q < kp; q += 128) {                                  // pair q / 2, part q & 1
@@ -254,71 +277,81 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
              to_digits(y, 1 + E - max(exp_field(y), 1)));
   }
   __syncthreads();
-  float c[4][4];
-  int tot[2][4];
-#pragma unroll
-  for (int q = 0; q < 4; q++) {
-    c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
-    tot[0][q] = tot[1][q] = 0;
-  }
   int it = 0;
-  for (int s = cg; s < nst; s += CG, it++) {
-    cp_async_wait<kRing - 1>();
-    const int slot = it % kRing;
-    uint4 raw[8];
+  for (int p = 0; p < np; p++) {
+    const int row0 = base + p * RT + mt * 16, ra = row0 + g, rb = ra + 8;
+    const int ja = ra < m ? min(ra, k) : 0, jb = rb < m ? min(rb, k) : 0;
+    const int nst = nsteps(p), nfull = row0 + 15 < m ? min(row0, k) / 16 : 0;   // steps without a masked entry
+    const double b2 = add_updates_part(0.0, ud, h0, h1, pt);
+    float c[4][4];
+    int tot[2][4];
 #pragma unroll
-    for (int q = 0; q < 8; q++) raw[q] = myring[slot * 256 + q * 32];
-    if (s >= nfull) {
+    for (int q = 0; q < 4; q++) {
+      c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
+      tot[0][q] = tot[1][q] = 0;
+    }
+    int since = 0;
+    for (int s = cg; s < nst; s += CG, it++) {
+      cp_async_wait<kRing - 1>();
+      const int slot = it % kRing;
+      uint4 raw[8];
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const int j = 16 * s + 2 * t + (q & 1) + 8 * (q >> 1);
-        if (j >= ja) raw[2 * q] = zero_entry();
-        if (j >= jb) raw[2 * q + 1] = zero_entry();
+      for (int q = 0; q < 8; q++) raw[q] = myring[slot * 256 + q * 32];
+      if (s >= nfull) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const int j = 16 * s + 2 * t + (q & 1) + 8 * (q >> 1);
+          if (j >= ja) raw[2 * q] = zero_entry();
+          if (j >= jb) raw[2 * q + 1] = zero_entry();
+        }
+      }
+      step_single(raw, bre, bim, (8 * s + t) * kPairStride + g + 7, c);
+      issue(slot);                                                       // the slot's entries are in use above
+      if ((++since & 7) == 0) flush_single(c, tot);                      // at most 128 columns per accumulator
+    }
+    flush_single(c, tot);
+    const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
+    const int64_t v2 = quad_half(tot[0][2], tot[0][3]), v3 = quad_half(tot[1][2], tot[1][3]);
+    int64_t(*sum)[RT][2][2] = sums[p & 1];
+    if ((t & 1) == 0) {
+      sum[cg][mt * 16 + g][0][t >> 1] = v0;
+      sum[cg][mt * 16 + g][1][t >> 1] = v1;
+      sum[cg][mt * 16 + g + 8][0][t >> 1] = v2;
+      sum[cg][mt * 16 + g + 8][1][t >> 1] = v3;
+    }
+    __syncthreads();
+    if (tid < 2 * RT) {                                                  // whole warps
+      int64_t hi = 0, lo = 0;
+#pragma unroll
+      for (int q = 0; q < CG; q++) {
+        hi += sum[q][tid >> 1][pt][0];
+        lo += sum[q][tid >> 1][pt][1];
+      }
+      const int r = base + p * RT + (tid >> 1);
+      double s = scale2(halves_value(hi, lo), 88 + re + E - kBias);
+      if (E == 0x7ff || re == kRowNonFinite) s = nan("");
+      const double a = s + (r < k ? b1[2 * r + pt] : 0.0);
+      const double o = __shfl_xor_sync(0xffffffffu, a, 1);               // the other part
+      if (r < m) {
+        // D^{-1} (a, o): real part dx a - dy o, imaginary part dx a + dy o (a, o swapped)
+        if (r < k)
+          reinterpret_cast<double*>(zout + S.first + r)[pt] = fma(dinv.x, a, pt ? dinv.y * o : -dinv.y * o);
+        else
+          reinterpret_cast<double*>(u + uw)[pt] = b2 - s;
       }
     }
-    step_single(raw, bre, bim, (8 * s + t) * kPairStride + g + 7, c);
-    issue(s + kRing * CG, slot);                                         // the slot's entries are in use above
-    if ((it & 7) == 7) flush_single(c, tot);                             // at most 128 columns per accumulator
-  }
-  flush_single(c, tot);
-  const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
-  const int64_t v2 = quad_half(tot[0][2], tot[0][3]), v3 = quad_half(tot[1][2], tot[1][3]);
-  if ((t & 1) == 0) {
-    sums[cg][mt * 16 + g][0][t >> 1] = v0;
-    sums[cg][mt * 16 + g][1][t >> 1] = v1;
-    sums[cg][mt * 16 + g + 8][0][t >> 1] = v2;
-    sums[cg][mt * 16 + g + 8][1][t >> 1] = v3;
-  }
-  __syncthreads();
-  if (tid < 2 * RT) {                                                    // whole warps
-    int64_t hi = 0, lo = 0;
-#pragma unroll
-    for (int q = 0; q < CG; q++) {
-      hi += sums[q][tid >> 1][pt][0];
-      lo += sums[q][tid >> 1][pt][1];
-    }
-    double s = scale2(halves_value(hi, lo), 88 + re + E - kBias);
-    if (E == 0x7ff || re == kRowNonFinite) s = nan("");
-    const double a = s + (mine && r < k ? b1[2 * r + pt] : 0.0);
-    const double o = __shfl_xor_sync(0xffffffffu, a, 1);                 // the other part
-    if (mine) {
-      // D^{-1} (a, o): real part dx a - dy o, imaginary part dx a + dy o (a, o swapped)
-      if (r < k)
-        reinterpret_cast<double*>(zout + S.first + r)[pt] = fma(dinv.x, a, pt ? dinv.y * o : -dinv.y * o);
-      else
-        reinterpret_cast<double*>(u + uw)[pt] = b2 - s;
-    }
+    load_row(p + 1);
   }
 }
 
-// Backward, 32 pivot columns x one row chunk per task: sums over the chunk's rows r > j of
-// P[r][j] vec[r], vec = (z, -x[ancestor rows]), with each panel row's exponent folded into
-// vec's.  4 warps = 2 column tiles x 2 groups of 16-row steps.  A supernode of one chunk is
-// finished here, else by the last CTA of the column block (bwd_finish).
+// Backward, ncol blocks of 32 pivot columns x one row chunk per task: sums over the chunk's rows r > j
+// of P[r][j] vec[r], vec = (z, -x[ancestor rows]), with each panel row's exponent folded into vec's,
+// gathered and converted once per task.  4 warps = 2 column tiles x 2 groups of 16-row steps.  A
+// supernode of one chunk is finished here, else by the last CTA of each column block (bwd_finish).
 __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnDev* sn, const int32_t* rowlist,
                                                     const double2* panels, const int16_t* rexp,
                                                     const double2* zin, double2* x, double2* partial, int rows,
-                                                    int rpad, const int4* fins, unsigned int* counters) {
+                                                    int rpad, int ncol, const int4* fins, unsigned int* counters) {
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4* ring = reinterpret_cast<uint4*>(smem_raw);                      // 4 warps x kRing x 8 x 32
@@ -326,42 +359,52 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
   uint32_t* vre = reinterpret_cast<uint32_t*>(vec + 2 * rpad);
   uint32_t* vim = vre + (rpad / 2) * kPairStride;
   int* vex = reinterpret_cast<int*>(vim + (rpad / 2) * kPairStride);     // rpad
-  __shared__ int64_t sums[2][32][2][2];                                  // [group][column][part][half]
+  __shared__ int64_t sums[2][2][32][2][2];                               // [block parity][group][column][part][half]
   __shared__ int red[4];
   const int4 tk = tasks[blockIdx.x];
   const SnDev S = sn[tk.x];
   const int k = S.k, m = S.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int g = lane >> 2, t = lane & 3, ct = wid & 1, sl = wid >> 1;
   const int r0 = tk.z * rows, r1 = min(m, r0 + rows);
-  const int j0 = tk.y * 32 + ct * 16;
-  const int ja = j0 + g, jb = ja + 8;
+  const int nblk = min(ncol, (k - tk.y * 32 + 31) / 32);
   const uint4* P = reinterpret_cast<const uint4*>(panels + S.paneloff);
-  const uint4* Pa = P + int64_t(ja < k ? ja : 0) * S.ld;
-  const uint4* Pb = P + int64_t(jb < k ? jb : 0) * S.ld;
   const int nst = (r1 - r0 + 15) / 16;
-  // steps whose rows all lie at or above the tile's first column hold nothing
-  const int sfirst = j0 < k ? max(0, (j0 + 1 - r0) / 16) : nst;
-  const bool fullcols = j0 + 15 < k;
   uint4* myring = ring + wid * (kRing * 256) + lane;
-  auto issue = [&](int s, int slot) {
-    if (s < nst) {
+  // first step of this warp in block p: those whose rows all lie at or above the tile's first
+  // column hold nothing
+  auto first = [&](int p) {
+    const int j0 = (tk.y + p) * 32 + ct * 16;
+    const int f = j0 < k ? max(0, (j0 + 1 - r0) / 16) : nst;
+    return f + ((sl - f) & 1);
+  };
+  int ip = 0, is = first(0);                                             // next step to copy: block, step
+  auto issue = [&](int slot) {
+    while (ip < nblk && is >= nst) {
+      ip++;
+      is = first(ip);
+    }
+    if (ip < nblk) {
+      const int ja = (tk.y + ip) * 32 + ct * 16 + g, jb = ja + 8;
+      const uint4 *Pa = P + int64_t(ja) * S.ld, *Pb = P + int64_t(jb) * S.ld;
 #pragma unroll
       for (int q = 0; q < 4; q++) {
-        const int r = r0 + 16 * s + 4 * t + q;
+        const int r = r0 + 16 * is + 4 * t + q;
         if (ja < k && r < r1 && r > ja) cp_async16(myring + slot * 256 + (2 * q) * 32, Pa + r);
         if (jb < k && r < r1 && r > jb) cp_async16(myring + slot * 256 + (2 * q + 1) * 32, Pb + r);
       }
+      is += 2;
     }
     cp_async_commit();
   };
-  const int s0 = sfirst + ((sl - sfirst) & 1);
 #pragma unroll
-  for (int q = 0; q < kRing; q++) issue(s0 + 2 * q, q);
+  for (int q = 0; q < kRing; q++) issue(q);
   const int32_t* rl = rowlist + S.rowoff;
   int e = -4000, bad = 0;
   pdl_wait();
+  const int pt = tid & 1;
+#pragma unroll 4
   for (int q = tid; q < 2 * (r1 - r0); q += 128) {
-    const int r = r0 + (q >> 1), pt = q & 1;
+    const int r = r0 + (q >> 1);
     const double v = r < k ? __ldcg(reinterpret_cast<const double*>(zin + S.first + r) + pt)
                            : -__ldcg(reinterpret_cast<const double*>(x + rl[r]) + pt);
     const int re = rexp[S.eoff + r];
@@ -374,7 +417,7 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
   const bool nonfinite = __syncthreads_or(bad) != 0;
   const int E = block_max(e, red);
   for (int q = tid; q < 16 * nst; q += 128) {
-    const int p = q >> 1, r = 2 * p, pt = q & 1;
+    const int p = q >> 1, r = 2 * p;
     double x0 = 0.0, x1 = 0.0;
     int e0 = 0, e1 = 0;
     if (r < r1 - r0) {
@@ -389,55 +432,66 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
     put_pair(dst, to_digits(x0, 1 + E - max(exp_field(x0), 1) - e0), to_digits(x1, 1 + E - max(exp_field(x1), 1) - e1));
   }
   __syncthreads();
-  float c[4][4];
-  int tot[2][4];
-#pragma unroll
-  for (int q = 0; q < 4; q++) {
-    c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
-    tot[0][q] = tot[1][q] = 0;
-  }
-  int it = 0;
-  for (int s = s0; s < nst; s += 2, it++) {
-    cp_async_wait<kRing - 1>();
-    const int slot = it % kRing;
-    uint4 raw[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) raw[q] = myring[slot * 256 + q * 32];
-    const int rs = r0 + 16 * s;
-    if (!fullcols || rs + 16 > r1 || rs <= j0 + 15) {
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const int r = rs + 4 * t + q;
-        if (ja >= k || r >= r1 || r <= ja) raw[2 * q] = zero_entry();
-        if (jb >= k || r >= r1 || r <= jb) raw[2 * q + 1] = zero_entry();
-      }
-    }
-    step_single(raw, vre, vim, (8 * s + t) * kPairStride + g + 7, c);
-    issue(s + 2 * kRing, slot);
-    if ((it & 7) == 7) flush_single(c, tot);
-  }
-  flush_single(c, tot);
-  const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
-  const int64_t v2 = quad_half(tot[0][2], tot[0][3]), v3 = quad_half(tot[1][2], tot[1][3]);
-  if ((t & 1) == 0) {
-    sums[sl][ct * 16 + g][0][t >> 1] = v0;
-    sums[sl][ct * 16 + g][1][t >> 1] = v1;
-    sums[sl][ct * 16 + g + 8][0][t >> 1] = v2;
-    sums[sl][ct * 16 + g + 8][1][t >> 1] = v3;
-  }
-  __syncthreads();
   const bool single = m <= rows;
-  if (tid < 64) {
-    const int j = tk.y * 32 + (tid >> 1), pt = tid & 1;
-    double s = scale2(halves_value(sums[0][tid >> 1][pt][0] + sums[1][tid >> 1][pt][0],
-                                   sums[0][tid >> 1][pt][1] + sums[1][tid >> 1][pt][1]), 88 + E - kBias);
-    if (nonfinite) s = nan("");
-    if (!single)
-      reinterpret_cast<double*>(partial)[int64_t(blockIdx.x) * 64 + tid] = s;
-    else if (j < k)
-      reinterpret_cast<double*>(x + S.first + j)[pt] = __ldcg(reinterpret_cast<const double*>(zin + S.first + j) + pt) + s;
+  int it = 0;
+  for (int p = 0; p < nblk; p++) {
+    const int j0 = (tk.y + p) * 32 + ct * 16, ja = j0 + g, jb = ja + 8;
+    const bool fullcols = j0 + 15 < k;
+    const int j = (tk.y + p) * 32 + (tid >> 1);
+    const double zj = single && tid < 64 && j < k ? __ldcg(reinterpret_cast<const double*>(zin + S.first + j) + pt) : 0.0;
+    float c[4][4];
+    int tot[2][4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
+      tot[0][q] = tot[1][q] = 0;
+    }
+    int since = 0;
+    for (int s = first(p); s < nst; s += 2, it++) {
+      cp_async_wait<kRing - 1>();
+      const int slot = it % kRing;
+      uint4 raw[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) raw[q] = myring[slot * 256 + q * 32];
+      const int rs = r0 + 16 * s;
+      if (!fullcols || rs + 16 > r1 || rs <= j0 + 15) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const int r = rs + 4 * t + q;
+          if (ja >= k || r >= r1 || r <= ja) raw[2 * q] = zero_entry();
+          if (jb >= k || r >= r1 || r <= jb) raw[2 * q + 1] = zero_entry();
+        }
+      }
+      step_single(raw, vre, vim, (8 * s + t) * kPairStride + g + 7, c);
+      issue(slot);
+      if ((++since & 7) == 0) flush_single(c, tot);
+    }
+    flush_single(c, tot);
+    const int64_t v0 = quad_half(tot[0][0], tot[0][1]), v1 = quad_half(tot[1][0], tot[1][1]);
+    const int64_t v2 = quad_half(tot[0][2], tot[0][3]), v3 = quad_half(tot[1][2], tot[1][3]);
+    int64_t(*sum)[32][2][2] = sums[p & 1];
+    if ((t & 1) == 0) {
+      sum[sl][ct * 16 + g][0][t >> 1] = v0;
+      sum[sl][ct * 16 + g][1][t >> 1] = v1;
+      sum[sl][ct * 16 + g + 8][0][t >> 1] = v2;
+      sum[sl][ct * 16 + g + 8][1][t >> 1] = v3;
+    }
+    __syncthreads();
+    if (tid < 64) {
+      double s = scale2(halves_value(sum[0][tid >> 1][pt][0] + sum[1][tid >> 1][pt][0],
+                                     sum[0][tid >> 1][pt][1] + sum[1][tid >> 1][pt][1]), 88 + E - kBias);
+      if (nonfinite) s = nan("");
+      if (!single)
+        reinterpret_cast<double*>(partial)[(int64_t(fins[tk.w + p].z) + tk.z) * 64 + tid] = s;
+      else if (j < k)
+        reinterpret_cast<double*>(x + S.first + j)[pt] = zj + s;
+    }
   }
-  if (!single) bwd_finish<double2>(fins[tk.w], S, zin, partial, x, counters + tk.w);
+  if (!single)
+    for (int p = 0; p < nblk; p++) {
+      bwd_finish<double2>(fins[tk.w + p], S, zin, partial, x, counters + tk.w + p);
+      __syncthreads();                                                   // its shared ticket is used again
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -757,7 +811,8 @@ void launch_to_digits(const FactorDev& F, cudaStream_t st) {
     if (F.h_fwd_rt[l] == 16)
       k_to_digits<16><<<unsigned(e - b), 256, 0, st>>>(F.fwd_tasks + b, F.ssn, (double2*)F.panels, F.rexp);
     else
-      k_to_digits<64><<<unsigned(e - b), 256, 0, st>>>(F.fwd_tasks + b, F.ssn, (double2*)F.panels, F.rexp);
+      k_to_digits<64><<<dim3(unsigned(e - b), unsigned(F.h_fwd_rt[l] / 64)), 256, 0, st>>>(F.fwd_tasks + b, F.ssn,
+                                                                                           (double2*)F.panels, F.rexp);
   }
 }
 
@@ -774,10 +829,10 @@ void launch_solve_dig(const FactorDev& F, cudaStream_t st) {
       const int kpad = F.h_lev_k[l];
       if (F.h_fwd_rt[l] == 16)
         launch_level(k_fwd_dig<1>, e - b, 128, fwd_smem(kpad), st, pdl, F.fwd_tasks + b, F.ssn, F.cptr, F.wpos, P,
-                     F.rexp, t, z, u, kpad);
+                     F.rexp, t, z, u, kpad, 1);
       else
         launch_level(k_fwd_dig<4>, e - b, 128, fwd_smem(kpad), st, pdl, F.fwd_tasks + b, F.ssn, F.cptr, F.wpos, P,
-                     F.rexp, t, z, u, kpad);
+                     F.rexp, t, z, u, kpad, F.h_fwd_rt[l] / 64);
     }
     if (F.level_events) cudaEventRecord(F.level_events[1 + l], st);
   }
@@ -787,7 +842,7 @@ void launch_solve_dig(const FactorDev& F, cudaStream_t st) {
       add_launches(1);
       const int rows = F.h_bwd_rows[l], rpad = (std::min(rows, F.h_lev_m[l]) + 15) / 16 * 16;
       launch_level(k_bwd_dig, e - b, 128, bwd_smem(rpad), st, pdl, F.bwd_tasks + b, F.ssn, F.rowlist, P, F.rexp, z, x,
-                   (double2*)F.bwd_partial, rows, rpad, F.bfin_tasks, F.bwd_counters);
+                   (double2*)F.bwd_partial, rows, rpad, F.h_bwd_cb[size_t(l)], F.bfin_tasks, F.bwd_counters);
     }
     if (F.level_events) cudaEventRecord(F.level_events[1 + F.snlev + (F.snlev - 1 - l)], st);
   }
