@@ -199,7 +199,10 @@ typedef struct {
   int64_t nsupernodes;      /* local supernodes over all subdomains                  */
   int32_t nlevels;          /* local assembly-tree levels                            */
   int32_t nlevels_coarse;
-  int64_t front_bytes;      /* transient device bytes of the frontal workspace       */
+  int64_t front_bytes;      /* transient device bytes of the frontal workspace.  With a
+                               direct coarse solve hz_factor also holds the coarse
+                               factor's, to run both at once, where that fits hbm_budget
+                               and a quarter of the free device memory                */
   int64_t device_bytes;     /* device bytes held by the context after hz_factor      */
   double factor_flops;      /* real flops of the numeric local factorisation         */
   double setup_seconds;     /* host wall time of hz_setup_mesh                        */

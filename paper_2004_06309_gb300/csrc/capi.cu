@@ -23,6 +23,8 @@ struct hz_ctx {
   std::string err;
   hz_options opt{};
   cudaStream_t st = nullptr;
+  cudaStream_t side = nullptr;      // direct coarse solve: the coarse factorisation beside the subdomains'
+  cudaEvent_t side_ev = nullptr;
   int device = 0;
   int order = 1, levels = 1, restart = 30, precision = 0, max_iter = 1000;
   hz::Mesh mesh;       // kept for point location
@@ -881,47 +883,79 @@ void free_host_ptrs(hz::FactorDev& F) {
   F.h_bfin_ptr = F.h_lev_ptr = F.h_fwd_ptr = F.h_bwd_ptr = F.h_wg_ptr = F.h_cb_ptr = F.h_ea_ptr = F.h_ent_ptr = nullptr;
 }
 
-hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[3], double& min_pivot) {
-  if (F.nsn == 0) return HZ_OK;
-  static const bool verbose = std::getenv("HZ_VERBOSE") != nullptr;
-  auto t0 = std::chrono::steady_clock::now();
-  const size_t vs = F.precision == 0 ? 16 : 8;
+// One numeric factorisation on a stream: its workspace and its status word.
+struct FactorRun {
+  hz::FactorDev* F = nullptr;
+  cudaStream_t st = nullptr;
+  hz::DevStatus* status = nullptr;
   char *fronts = nullptr, *scratch = nullptr;
-  TRY(dalloc(c, &fronts, F.front_elems * int64_t(vs)));
-  hz_status s = dalloc(c, &scratch, std::max<int64_t>(F.scratch_elems, 1) * int64_t(vs));
+};
+
+int64_t factor_workspace(const hz::FactorDev& F) {
+  return (F.front_elems + std::max<int64_t>(F.scratch_elems, 1)) * (F.precision == 0 ? 16 : 8);
+}
+
+bool factor_verbose() {
+  static const bool verbose = std::getenv("HZ_VERBOSE") != nullptr;
+  return verbose;
+}
+
+hz_status factor_alloc(hz_ctx* c, FactorRun& r) {
+  const hz::FactorDev& F = *r.F;
+  if (F.nsn == 0) return HZ_OK;
+  auto t0 = std::chrono::steady_clock::now();
+  const int64_t vs = F.precision == 0 ? 16 : 8;
+  TRY(dalloc(c, &r.fronts, F.front_elems * vs));
+  const hz_status s = dalloc(c, &r.scratch, std::max<int64_t>(F.scratch_elems, 1) * vs);
   if (s != HZ_OK) {
-    dfree(c, fronts);
+    dfree(c, r.fronts);
+    r.fronts = nullptr;
     return s;
   }
+  if (factor_verbose())
+    std::fprintf(stderr, "[hz] factor: workspace %.2f GB allocated in %.3f s\n", double(F.front_elems) * double(vs) / 1e9,
+                 std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
+  return HZ_OK;
+}
+
+hz_status factor_launch(hz_ctx* c, FactorRun& r, double w, const double maxabs[3]) {
+  hz::FactorDev& F = *r.F;
+  if (F.nsn == 0) return HZ_OK;
+  const bool verbose = factor_verbose();
+  auto t0 = std::chrono::steady_clock::now();
   hz::DevStatus init{0u, 0u, 0.0};   // zero_pivot, timeout, min_pivot
   const double big = 1e300;
   std::memcpy(&init.min_pivot, &big, sizeof(double));
-  CU(cudaMemcpyAsync(c->status, &init, sizeof(init), cudaMemcpyHostToDevice, c->st));
+  CU(cudaMemcpyAsync(r.status, &init, sizeof(init), cudaMemcpyHostToDevice, r.st));
   const double tiny = 1e-13 * (maxabs[0] + w * w * maxabs[1] + w * maxabs[2]);
   if (verbose) {
-    cudaStreamSynchronize(c->st);
-    std::fprintf(stderr, "[hz] factor: workspace %.2f GB allocated in %.3f s\n",
-                 double(F.front_elems) * double(vs) / 1e9,
-                 std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
+    cudaStreamSynchronize(r.st);
     t0 = std::chrono::steady_clock::now();
   }
   for (int g = 0; g < F.ngrp; g++)                 // groups one after the other in one workspace
-    for (int l = 0; l < F.nlev; l++) hz::launch_factor_level(F, l, g, w, fronts, scratch, c->status, tiny, c->st);
-  hz::launch_merge_panels(F, c->st);              // merged solve supernodes of the sweeps
-  if (F.precision == 0) hz::launch_to_digits(F, c->st);
+    for (int l = 0; l < F.nlev; l++) hz::launch_factor_level(F, l, g, w, r.fronts, r.scratch, r.status, tiny, r.st);
+  hz::launch_merge_panels(F, r.st);               // merged solve supernodes of the sweeps
+  if (F.precision == 0) hz::launch_to_digits(F, r.st);
   if (verbose) {
-    cudaStreamSynchronize(c->st);
+    cudaStreamSynchronize(r.st);
     std::fprintf(stderr, "[hz] factor: %d levels in %.3f s\n", F.nlev,
                  std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
-    t0 = std::chrono::steady_clock::now();
   }
   CU(cudaGetLastError());
+  return HZ_OK;
+}
+
+// Waits for the factorisation, gives its workspace back and judges it.
+hz_status factor_finish(hz_ctx* c, FactorRun& r, double& min_pivot) {
+  if (r.F->nsn == 0) return HZ_OK;
+  auto t0 = std::chrono::steady_clock::now();
   hz::DevStatus out{};
-  CU(cudaMemcpyAsync(&out, c->status, sizeof(out), cudaMemcpyDeviceToHost, c->st));
-  CU(cudaStreamSynchronize(c->st));
-  dfree(c, fronts);
-  dfree(c, scratch);
-  if (verbose)
+  CU(cudaMemcpyAsync(&out, r.status, sizeof(out), cudaMemcpyDeviceToHost, r.st));
+  CU(cudaStreamSynchronize(r.st));
+  dfree(c, r.fronts);
+  dfree(c, r.scratch);
+  r.fronts = r.scratch = nullptr;
+  if (factor_verbose())
     std::fprintf(stderr, "[hz] factor: status read and workspace freed in %.3f s\n",
                  std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
   min_pivot = std::min(min_pivot, out.min_pivot);
@@ -931,6 +965,63 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
                                        : "a tensor-core completion wait ran out in the factorisation");
   if (out.zero_pivot) return fail(c, HZ_ERR_ZERO_PIVOT, "tiny pivot in a local LDL^T factor");
   return HZ_OK;
+}
+
+hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[3], double& min_pivot) {
+  FactorRun r;
+  r.F = &F;
+  r.st = c->st;
+  r.status = c->status;
+  TRY(factor_alloc(c, r));
+  TRY(factor_launch(c, r, w, maxabs));
+  return factor_finish(c, r, min_pivot);
+}
+
+// The subdomain factors on the context's stream and the coarse factor on its side stream at the
+// same time.  The coarse factor is one matrix: above the first few of its tree levels a launch holds
+// a handful of CTAs, whose serial pivot blocks set the time while the subdomains' launches fill
+// the GPU.  The side stream has the higher priority, so that this chain is not queued behind them.
+// The subdomain factor's workspace comes first, as without the side stream; the coarse one's is
+// then taken only if it leaves three quarters of the free memory and fits the context's limit,
+// else coarse_follows is set and nothing of the coarse factor has run.
+// 349,461 dofs, mixed (coarse factor 54,925 dofs, 36 levels): hz_factor 105.1 -> 86.8 ms; 64,009
+// dofs, FP64: 41.2 -> 36.0 ms.
+hz_status factor_both(hz_ctx* c, double w, double& min_pivot, bool& coarse_follows) {
+  FactorRun a, b;
+  a.F = &c->loc;
+  a.st = c->st;
+  a.status = c->status;
+  b.F = &c->crs;
+  b.st = c->side;
+  b.status = c->status + 1;
+  coarse_follows = true;
+  TRY(factor_alloc(c, a));
+  const int64_t need = factor_workspace(c->crs);
+  size_t free_bytes = 0, total_bytes = 0;
+  CU(cudaMemGetInfo(&free_bytes, &total_bytes));
+  const bool fits = need <= int64_t(free_bytes / 4) &&
+                    (!c->opt.hbm_budget || uint64_t(c->bytes) + uint64_t(need) <= c->opt.hbm_budget);
+  if (fits && factor_alloc(c, b) == HZ_OK) coarse_follows = false;
+  if (coarse_follows) {
+    TRY(factor_launch(c, a, w, c->loc_max));
+    return factor_finish(c, a, min_pivot);
+  }
+  hz_status s = HZ_OK;
+  if (cudaEventRecord(c->side_ev, c->st) != cudaSuccess || cudaStreamWaitEvent(c->side, c->side_ev, 0) != cudaSuccess)
+    s = fail(c, HZ_ERR_CUDA, "ordering the coarse factorisation after the context's stream");
+  if (s == HZ_OK) s = factor_launch(c, b, w, c->crs_max);
+  if (s == HZ_OK) s = factor_launch(c, a, w, c->loc_max);
+  // both are waited for whatever either gives: their workspaces go back.  The host wait for
+  // the side stream orders it before anything that the context's stream does next.
+  const hz_status sa = factor_finish(c, a, min_pivot);
+  const std::string ea = c->err;
+  const hz_status sb = factor_finish(c, b, min_pivot);
+  if (s != HZ_OK) return s;
+  if (sa != HZ_OK) {
+    c->err = ea;                                   // the subdomains' failure is the one reported, as in serial order
+    return sa;
+  }
+  return sb;
 }
 
 // The Givens update of one vector's Hessenberg column (|b| at scal[bn_off]).
@@ -2162,6 +2253,8 @@ void hz_free(hz_ctx* c) {
   c->sizes.clear();
   for (cudaGraphExec_t g : c->gexec)
     if (g) cudaGraphExecDestroy(g);
+  if (c->side_ev) cudaEventDestroy(c->side_ev);
+  if (c->side) cudaStreamDestroy(c->side);
   if (c->h_pin) cudaFreeHost(c->h_pin);
   free_host_ptrs(c->loc);
   free_host_ptrs(c->crs);
@@ -2553,7 +2646,14 @@ static hz_status populate(hz_ctx* c, hz::HostProblem& P, int order, const hz_opt
   // the iterative coarse solve waits on the host inside each preconditioner application
   c->graphs = std::getenv("HZ_NO_GRAPHS") == nullptr && !c->coarse_oras;
   SETUP_TRY(dalloc(c, &c->brk, 1));
-  SETUP_TRY(dalloc(c, &c->status, 1));
+  SETUP_TRY(dalloc(c, &c->status, 2));            // the subdomains' factor, the coarse factor
+  if (c->levels == 2 && !c->coarse_oras) {
+    int lo = 0, hi = 0;
+    cudaDeviceGetStreamPriorityRange(&lo, &hi);
+    if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->side_ev, cudaEventDisableTiming) != cudaSuccess)
+      SETUP_TRY(fail(c, HZ_ERR_CUDA, "creating the coarse factorisation's stream"));
+  }
   if (c->S) {
     const int S = c->S;
     // block GCRO-DR keeps its recycled space C in the rk columns right before Vb
@@ -2657,8 +2757,12 @@ extern "C" hz_status hz_factor(hz_ctx* c, double freq_hz) {
   }
   hz::set_spmv_lanes(c->spmv_lanes);
   double minp = 1e300;
-  TRY(factor_one(c, c->loc, w, c->loc_max, minp));
   const bool tune = c->opt.tune_sweeps && !c->sweeps_tuned && c->opt.sweep_tasks == 0 && c->opt.bwd_chunk == 0;
+  bool coarse_follows = true;
+  if (c->side && !tune)                           // the sweeps are timed with nothing beside them
+    TRY(factor_both(c, w, minp, coarse_follows));
+  else
+    TRY(factor_one(c, c->loc, w, c->loc_max, minp));
   if (tune) {
     TRY(tune_sweeps(c, c->loc));
     hz_stats& st = c->stats;
@@ -2674,7 +2778,7 @@ extern "C" hz_status hz_factor(hz_ctx* c, double freq_hz) {
     hz::launch_fill_values(c->nnzH, c->d_EK, c->d_EM, c->d_EB, w, c->d_E, c->st);
     TRY(factor_one(c, c->cloc, w, c->cloc_max, minp));
     c->stats.coarse_solves = c->stats.coarse_iterations = 0;
-  } else if (c->levels == 2) {
+  } else if (c->levels == 2 && coarse_follows) {
     TRY(factor_one(c, c->crs, w, c->crs_max, minp));
     if (tune) TRY(tune_sweeps(c, c->crs));
   }
