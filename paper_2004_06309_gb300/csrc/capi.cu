@@ -984,7 +984,7 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
 // The subdomain factor's workspace comes first, as without the side stream; the coarse one's is
 // then taken only if it leaves three quarters of the free memory and fits the context's limit,
 // else coarse_follows is set and nothing of the coarse factor has run.
-// 349,461 dofs, mixed (coarse factor 54,925 dofs, 36 levels): hz_factor 105.1 -> 86.8 ms; 64,009
+// 349,461 dofs, mixed (coarse factor 54,925 dofs, 36 levels): hz_factor 105.1 -> 86.8 ms; 54,925
 // dofs, FP64: 41.2 -> 36.0 ms.
 hz_status factor_both(hz_ctx* c, double w, double& min_pivot, bool& coarse_follows) {
   FactorRun a, b;
