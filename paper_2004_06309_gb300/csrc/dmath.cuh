@@ -91,6 +91,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\
 __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(sdst)), "l"(gsrc) : "memory");
 }
+// 8 bytes, or zeros if !in (gsrc is not read then)
+__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem_addr(sdst)), "l"(gsrc), "r"(in ? 8 : 0)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // returns when at most N of the thread's committed groups are still in flight
 template <int N> __device__ __forceinline__ void cp_async_wait() {
