@@ -94,11 +94,6 @@ __device__ __forceinline__ int64_t quad_half(int hi, int lo) {
   const int64_t v = int64_t(hi) * 256 + lo;
   return v * 65536 + __shfl_xor_sync(0xffffffffu, v, 1);
 }
-// value of the two halves: result 2^88 2^(exponents)
-__device__ __forceinline__ double halves_value(int64_t hi, int64_t lo) {
-  return fma(double(lo), 0x1p-32, double(hi));
-}
-
 // a + the pt-th parts of u[c0 .. c1), in order; the first two loads are issued together
 __device__ __forceinline__ double add_updates_part(double a, const double* ud, uint32_t c0, uint32_t c1, int pt) {
   double v0 = 0.0, v1 = 0.0;
@@ -328,7 +323,7 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
         lo += sum[q][tid >> 1][pt][1];
       }
       const int r = base + p * RT + (tid >> 1);
-      double s = scale2(halves_value(hi, lo), 88 + re + E - kBias);
+      double s = scaled_sum(hi, lo, 88 + re + E - kBias);
       if (E == 0x7ff || re == kRowNonFinite) s = nan("");
       const double a = s + (r < k ? b1[2 * r + pt] : 0.0);
       const double o = __shfl_xor_sync(0xffffffffu, a, 1);               // the other part
@@ -478,8 +473,8 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
     }
     __syncthreads();
     if (tid < 64) {
-      double s = scale2(halves_value(sum[0][tid >> 1][pt][0] + sum[1][tid >> 1][pt][0],
-                                     sum[0][tid >> 1][pt][1] + sum[1][tid >> 1][pt][1]), 88 + E - kBias);
+      double s = scaled_sum(sum[0][tid >> 1][pt][0] + sum[1][tid >> 1][pt][0],
+                            sum[0][tid >> 1][pt][1] + sum[1][tid >> 1][pt][1], 88 + E - kBias);
       if (nonfinite) s = nan("");
       if (!single)
         reinterpret_cast<double*>(partial)[(int64_t(fins[tk.w + p].z) + tk.z) * 64 + tid] = s;
