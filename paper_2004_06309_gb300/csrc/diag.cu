@@ -13,8 +13,9 @@
 // level in complex128 (width 112) and 0.61 ms in complex64 (width 128).  A complex128 product is
 // 4 FP64 instructions of 64 clocks per scheduler, whatever its active lanes, so the block
 // products run in exact digits on mma.sync (digits.cuh) and only the 16 x 16 blocks on the FP64
-// units; the pivots' chain (reciprocal, column, update) is what remains: 0.36 ms per level in
-// complex128 and 0.14 ms in complex64 on the same models.
+// units.  The next pivot's chain (diagonal entry, reciprocal, column) runs in its own warp beside the
+// update, its two parts in different lanes of the same instructions; one after the other a pivot took 2,500
+// clocks.  0.27 ms per level in complex128 and 0.12 ms in complex64 on the same models.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -80,8 +81,7 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
   constexpr bool dbl = sizeof(V) == 16;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ V dinv[16 * kMaxNbk], dval[16 * kMaxNbk];
-  __shared__ V wcol2[2][16], lcol2[2][16], trow2[2][16];   // by the pivot's parity
-  __shared__ V dcur;
+  __shared__ V wcol2[2][16], trow2[2][16], xdiag[2], lcol[16];   // [2]: by the pivot's parity
   __shared__ V ljj[dbl ? 1 : 256];                         // L(J, J), column-major
   __shared__ int aexp[16 * kMaxNbk], bexp[2][16];
   const SnDev S = sn[lev_sn[blockIdx.x]];
@@ -237,46 +237,90 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
       }
       __syncthreads();
     }
-    // 16 x 16 block: thread (i, c) holds entry (i, c) of the update for c > pivot and of T for
-    // c < pivot
+    // 16 x 16 block.  Warps 2, 3, 6 and 7 hold its entries (row, c), two row pairs each: of the update
+    // for c > pivot, of T from pivot c on.  Warp 0 does what the next pivot waits for beside them:
+    // column of L, next diagonal entry, its reciprocal, real and imaginary parts in different lanes.
     {
-      const int i = tid & 15, c = tid >> 4;
-      V x = blk(J, J)[i + P * c], tv = czero<V>();
-      for (int j = 0; j < 16; j++) {
-        V *wcol = wcol2[j & 1], *lcol = lcol2[j & 1], *trow = trow2[j & 1];
-        if (c == j && i >= j) wcol[i] = x;
-        if (i == j && c <= j) {
-          if (c == j) {
-            tv = czero<V>();
-            tv.x = 1;
-          }
-          trow[c] = tv;
-        }
-        __syncthreads();
-        if (tid == 0 || tid == 32) {                       // the two parts on two schedulers
-          const V d = wcol[j];
-          const auto q = d.x * d.x + d.y * d.y;
-          if (tid == 0) {
-            dcur.x = d.x / q;
-            dval[16 * J + j] = d;
-          } else {
-            dcur.y = -d.y / q;
-          }
-        }
-        __syncthreads();
-        const V di = dcur;
-        if (tid == 64) dinv[16 * J + j] = di;
-        if (tid < 16 && i > j) {
-          lcol[i] = cmul(wcol[i], di);
-          if constexpr (!dbl) ljj[16 * j + i] = lcol[i];
-        }
-        __syncthreads();
-        if (i > j) {
-          if (c <= j) tv = cmsub(lcol[i], trow[c], tv);
-          else if (i >= c) x = cmsub(wcol[i], lcol[c], x);
+      using R = decltype(V().x);
+      const int c = lane & 15, uw = (wid & 2) ? (wid & 1) + 2 * (wid >> 2) : -1;
+      const int part = lane >> 4;                          // warp 0: lanes (i = c, part)
+      int row[2] = {0, 0};
+      V y[2] = {czero<V>(), czero<V>()};
+      if (uw >= 0) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const int r = row[h] = 2 * (uw + 4 * h) + part;
+          y[h] = blk(J, J)[r + P * c];
+          if (c == 0) wcol2[0][r] = y[h];
+          if (r == 1 && c == 1) xdiag[1] = y[h];
         }
       }
-      blk(J, J)[i + P * c] = i > c ? tv : czero<V>();
+      if (tid == 0) {
+        V one = czero<V>();
+        one.x = 1;
+        trow2[0][0] = one;
+      }
+      __syncthreads();
+      V d = czero<V>(), di = czero<V>();
+      auto reciprocal = [&]() {                            // warp 0: 1 / d
+        const R q = d.x * d.x + d.y * d.y;
+        const R v = (part ? -d.y : d.x) / q;
+        di.x = __shfl_sync(0xffffffffu, v, 0);
+        di.y = __shfl_sync(0xffffffffu, v, 16);
+      };
+      if (wid == 0) {
+        d = wcol2[0][0];
+        reciprocal();
+      }
+      for (int j = 0; j < 16; j++) {
+        V *wcol = wcol2[j & 1], *trow = trow2[j & 1];
+        if (wid == 0) {
+          const V w = wcol[c];                             // w di, one part per lane
+          const R v = xfma(w.x, part ? di.y : di.x, (part ? w.y : -w.y) * (part ? di.x : di.y));
+          if (c > j) {
+            reinterpret_cast<R*>(lcol + c)[part] = v;
+            if constexpr (!dbl) reinterpret_cast<R*>(ljj + 16 * j + c)[part] = v;
+          }
+          if (lane == 0) {
+            dval[16 * J + j] = d;
+            dinv[16 * J + j] = di;
+          }
+        }
+        __syncthreads();
+        if (j == 15) break;
+        if (uw >= 0) {
+#pragma unroll
+          for (int h = 0; h < 2; h++) {
+            const int r = row[h];
+            if (r <= j) continue;
+            const bool t = c <= j;
+            y[h] = cmsub(t ? lcol[r] : wcol[r], t ? trow[c] : lcol[c], c == j ? czero<V>() : y[h]);
+            if (c == j + 1) wcol2[(j + 1) & 1][r] = y[h];
+            if (r == j + 1 && c <= j + 1) {
+              V v = y[h];
+              if (c == j + 1) {
+                v = czero<V>();
+                v.x = 1;
+              }
+              trow2[(j + 1) & 1][c] = v;
+            }
+            if (r == j + 2 && c == j + 2) xdiag[j & 1] = y[h];
+          }
+        } else if (wid == 0) {
+          const V w = wcol[j + 1], l = lcol[j + 1], x = xdiag[(j + 1) & 1];
+          // one part per lane: x - w l
+          R v = xfma(-w.x, part ? l.y : l.x, part ? x.y : x.x);
+          v = xfma(part ? -w.y : w.y, part ? l.x : l.y, v);
+          d.x = __shfl_sync(0xffffffffu, v, 0);
+          d.y = __shfl_sync(0xffffffffu, v, 16);
+          reciprocal();
+        }
+        __syncthreads();
+      }
+      if (uw >= 0) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) blk(J, J)[row[h] + P * c] = row[h] > c ? y[h] : czero<V>();
+      }
       __syncthreads();
     }
     // W(I, J) = A(I, J) T^T for I > J and T(J, J') = -T S(J') for J' < J
