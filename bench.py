@@ -66,9 +66,9 @@ def workload_dofs(name):
     return (4 * nx + 1) * (4 * ny + 1) * (4 * nz + 1)
 # kernels of each timed phase (hz_profile)
 PHASE_KERNELS = {
-    "local_solve": "k_fwd_c64 / k_bwd_partial_c64 (k_fwd / k_bwd_partial_c128 in FP64), one launch per tree level",
+    "local_solve": "k_fwd_c64 / k_bwd_partial_c64 (k_fwd_dig / k_bwd_dig in FP64), one launch per tree level",
     "coarse": "k_spmv_real, coarse sweeps (or the inner GMRES of the iterative coarse solve), k_spmv_real",
-    "cgs2": "k_mdot, k_maxpy, k_reduce",
+    "cgs2": "k_cgs, k_cgs_sum",
     "spmv": "k_spmv",
 }
 # DRAM traffic / panel bytes of the complex64 local sweeps (ncu, medium workload, three launches

@@ -368,7 +368,7 @@ hz_status build_sweep_tasks(hz_ctx* c, hz::FactorDev& F, const SweepPlan& sp) {
     for (int32_t q = lev_ptr[l]; q < lev_ptr[l + 1]; q++) {
       const int s = lev_sn[q];
       const int k = sn_k[s], m = sn_m[s];
-      const int frows = sp.fwd_rt[l];                  // forward task rows (k_fwd / k_fwd_c64)
+      const int frows = sp.fwd_rt[l];                  // forward task rows (k_fwd_dig / k_fwd_c64)
       for (int rb = 0; rb * frows < m; rb++) fwd.push_back(make_int2(s, rb));
       const int nch = (m + sp.bwd_rows[l] - 1) / sp.bwd_rows[l];
       for (int cb = 0; cb * 32 < k; cb++) {
