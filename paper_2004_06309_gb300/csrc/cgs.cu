@@ -13,6 +13,10 @@
 // pass, runs the Givens update, so an orthogonalisation takes three launches instead of eight.
 // Measured (dots, update): 101, 80 us before, on 25 columns of 349,461 rows; 27, 8.6 us on 13
 // columns of 2,197 rows with 6 us for each sum over blocks and 14 for Givens.
+// A warp's loop is compiled for its own number of columns, and with at most four columns the warps
+// share the rows.  With loops of 1, 2, 4 or 8 columns, unused ones skipped, CGS2 of 33 columns took
+// 577 us at 349,461 rows and 3.45 ms at 2,368,333 (388 us and 2.22 ms so; 485 us and 2.51 ms with one
+// launch per update and dot), of one column 105 and 422 us (69 and 166; 119 and 253).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -31,13 +35,16 @@ constexpr int kMinChunk = 64;
 // the last block's own sum over this many blocks takes about as long as the launch it saves
 constexpr int kFusedBlocks = 160;
 
-// sums NC complex values over a warp's lanes; the sum of value c ends in the lanes whose bits from
-// 16 down spell c (most significant first)
-template <int NC> __device__ __forceinline__ double2 sum_columns(double2* v, int lane, int& c) {
+// smallest power of two that holds NC values
+template <int NC> constexpr int kPow2 = NC <= 1 ? 1 : (NC <= 2 ? 2 : (NC <= 4 ? 4 : 8));
+
+// sums P (a power of two) complex values over a warp's lanes; the sum of value c ends in the lanes
+// whose bits from 16 down spell c (most significant first)
+template <int P> __device__ __forceinline__ double2 sum_columns(double2* v, int lane, int& c) {
   c = 0;
   int o = 16;
 #pragma unroll
-  for (int half = NC / 2; half > 0; half >>= 1, o >>= 1) {
+  for (int half = P / 2; half > 0; half >>= 1, o >>= 1) {
     const bool up = (lane & o) != 0;
 #pragma unroll
     for (int i = 0; i < half; i++) {
@@ -49,6 +56,27 @@ template <int NC> __device__ __forceinline__ double2 sum_columns(double2* v, int
   double2 s = v[0];
   for (; o > 0; o >>= 1) s = cadd(s, shfl_xor(s, o));
   return s;
+}
+
+// acc[c] += the dots of column c (of C, every eighth one of the basis) over rows q0, q0 + step, .. < cnt
+template <int C>
+__device__ __forceinline__ void dot_rows(double2* acc, const double2* __restrict__ V, int64_t ld8, const double2* ws,
+                                         int q0, int cnt, int step) {
+  constexpr int U = C == 1 ? 8 : (C == 2 ? 4 : 2);
+#pragma unroll U
+  for (int q = q0; q < cnt; q += step) {
+    const double2 x = ws[q];
+#pragma unroll
+    for (int c = 0; c < C; c++) acc[c] = cmadc(V[q + c * ld8], x, acc[c]);
+  }
+}
+// the same for a warp that holds `mine` of at most C columns: a loop for each count.  Skipping columns
+// inside one loop of C kept the FP64 units as busy as C of them
+template <int C>
+__device__ __forceinline__ void dot_rows_of(int mine, double2* acc, const double2* V, int64_t ld8, const double2* ws,
+                                            int q0, int cnt, int step) {
+  if (mine == C) dot_rows<C>(acc, V, ld8, ws, q0, cnt, step);
+  else if constexpr (C > 1) dot_rows_of<C - 1>(mine, acc, V, ld8, ws, q0, cnt, step);
 }
 
 // Givens update of column j, one warp.  The chain over the earlier rotations is sequential; lanes 0-3
@@ -132,8 +160,9 @@ static int64_t cgs_chunk(int64_t n) {
 enum { kAxpy = 1, kDots = 2 };
 
 // One pass over a chunk of rows: the update (thread per row), then the dots (warp wid holds columns
-// wid + 8 c, lanes over the rows kept in shared memory).  ticket != null: the slot's last block adds
-// the blocks' sums into out (columns, and |w|^2 at 64) and runs the Givens update if asked.
+// wid + 8 c, lanes over the rows kept in shared memory; with at most four columns the warps share
+// the rows of each).  ticket != null: the slot's last block adds the blocks' sums into out (columns,
+// and |w|^2 at 64) and runs the Givens update if asked.  NC: columns per warp of the widest slot.
 template <int NC>
 __global__ void __launch_bounds__(256) k_cgs(int64_t n, SlotCgs p, int mode, int64_t chunk, int sub, double2* partial,
                                              unsigned int* ticket, double2* out, SlotGivens gv, int givens) {
@@ -141,8 +170,9 @@ __global__ void __launch_bounds__(256) k_cgs(int64_t n, SlotCgs p, int mode, int
   if (ncols < 0) return;
   __shared__ double2 hs[kMaxCols];
   __shared__ double2 ws[256];
+  __shared__ double2 gsum[8];
   __shared__ double red[8];
-  __shared__ unsigned int mine;
+  __shared__ unsigned int order;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const double2* __restrict__ V = p.V[i];
   double2* w = p.w[i];
@@ -152,9 +182,13 @@ __global__ void __launch_bounds__(256) k_cgs(int64_t n, SlotCgs p, int mode, int
     __syncthreads();
   }
   const int64_t row0 = blockIdx.x * chunk, row1 = min(n, row0 + chunk);
-  double2 acc[NC];
+  constexpr int P = kPow2<NC>;
+  double2 acc[P];
 #pragma unroll
-  for (int c = 0; c < NC; c++) acc[c] = make_double2(0.0, 0.0);
+  for (int c = 0; c < P; c++) acc[c] = make_double2(0.0, 0.0);
+  // cw columns side by side in the warps, 8 / cw groups of warps over a column's rows
+  const int cw = ncols > 4 ? 8 : (ncols > 2 ? 4 : (ncols > 1 ? 2 : 1)), col = wid & (cw - 1);
+  const int q0 = lane + 32 * (wid / cw), step = 32 * (8 / cw), mine = col < ncols ? (ncols - col + 7) / 8 : 0;
   double nn = 0.0;
   for (int64_t base = row0; base < row1; base += sub) {
     const int cnt = int(min(int64_t(sub), row1 - base));
@@ -174,21 +208,19 @@ __global__ void __launch_bounds__(256) k_cgs(int64_t n, SlotCgs p, int mode, int
     if (mode & kDots) {
       ws[tid] = v;
       __syncthreads();
-#pragma unroll 2
-      for (int q = lane; q < cnt; q += 32) {
-        const double2 x = ws[q];
-#pragma unroll
-        for (int c = 0; c < NC; c++)
-          if (wid + 8 * c < ncols) acc[c] = cmadc(V[base + q + (wid + 8 * c) * ld], x, acc[c]);
-      }
+      dot_rows_of<NC>(mine, acc, V + base + col * ld, 8 * ld, ws, q0, cnt, step);
       __syncthreads();
     }
   }
   double2* part = partial + (int64_t(i) * nb + blockIdx.x) * kPartStride;
   if (mode & kDots) {
     int c;
-    const double2 s = sum_columns<NC>(acc, lane, c);
-    if ((lane & (32 / NC - 1)) == 0 && wid + 8 * c < ncols) part[wid + 8 * c] = s;
+    const double2 s = sum_columns<P>(acc, lane, c);
+    if (cw < 8) {
+      if (lane == 0) gsum[wid] = s;
+    } else if ((lane & (32 / P - 1)) == 0 && wid + 8 * c < ncols) {
+      part[wid + 8 * c] = s;
+    }
   }
   for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
   if (lane == 0) red[wid] = nn;
@@ -198,12 +230,17 @@ __global__ void __launch_bounds__(256) k_cgs(int64_t n, SlotCgs p, int mode, int
     for (int q = 0; q < 8; q++) s += red[q];
     part[kMaxCols] = make_double2(s, 0.0);
   }
+  if ((mode & kDots) && cw < 8 && tid < ncols) {
+    double2 s = gsum[tid];
+    for (int q = tid + cw; q < 8; q += cw) s = cadd(s, gsum[q]);
+    part[tid] = s;
+  }
   if (!ticket) return;
   __threadfence();
   __syncthreads();
-  if (tid == 0) mine = atomicAdd(ticket + i, 1u);
+  if (tid == 0) order = atomicAdd(ticket + i, 1u);
   __syncthreads();
-  if (mine != unsigned(nb) - 1) return;
+  if (order != unsigned(nb) - 1) return;
   __threadfence();
   const double2* all = partial + int64_t(i) * nb * kPartStride;
   double2* o = out + int64_t(i) * kPartStride;
@@ -265,10 +302,18 @@ void launch_cgs_slots(int64_t n, int S, const SlotCgs& p, bool maxpy, bool dots,
   if (givens) gv = *givens;
   const dim3 grid(unsigned(std::max(nb, 1)), unsigned(S));
   add_launches(1);
-  if (!dots || cols <= 8) k_cgs<1><<<grid, 256, 0, st>>>(n, p, mode, chunk, sub, partial, tk, out, gv, gfused);
-  else if (cols <= 16) k_cgs<2><<<grid, 256, 0, st>>>(n, p, mode, chunk, sub, partial, tk, out, gv, gfused);
-  else if (cols <= 32) k_cgs<4><<<grid, 256, 0, st>>>(n, p, mode, chunk, sub, partial, tk, out, gv, gfused);
-  else k_cgs<8><<<grid, 256, 0, st>>>(n, p, mode, chunk, sub, partial, tk, out, gv, gfused);
+  const int nc = dots ? std::max((cols + 7) / 8, 1) : 1;
+  auto pass = [&](auto* kern) { kern<<<grid, 256, 0, st>>>(n, p, mode, chunk, sub, partial, tk, out, gv, gfused); };
+  switch (nc) {
+    case 1: pass(k_cgs<1>); break;
+    case 2: pass(k_cgs<2>); break;
+    case 3: pass(k_cgs<3>); break;
+    case 4: pass(k_cgs<4>); break;
+    case 5: pass(k_cgs<5>); break;
+    case 6: pass(k_cgs<6>); break;
+    case 7: pass(k_cgs<7>); break;
+    default: pass(k_cgs<8>); break;
+  }
   if (fused) return;
   add_launches(1);
   k_cgs_sum<<<dim3(unsigned(dots ? cols + 1 : 1), unsigned(S)), 256, 0, st>>>(partial, int(grid.x), p, mode, out);
