@@ -567,6 +567,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
         rows += d.m;
       }
       TRY(dalloc(c, &F.rexp, std::max<int64_t>(rows, 1)));
+      TRY(dalloc(c, &F.colnz, std::max<int64_t>(F.ntot, 1)));
     }
     TRY(upload(c, &F.ssn, ssn));
   }

@@ -52,6 +52,7 @@ struct FactorDev {
   int64_t merge_tmp_elems = 0;
   void* merge_tmp = nullptr;
   int16_t* rexp = nullptr;            // complex128: exponent of each solve panel row's digits (sweeps64.cu)
+  uint8_t* colnz = nullptr;           // complex128: columns (vector index) of solve panels with entries below the diagonal
   int32_t* rowlist = nullptr;
   uint32_t* cptr = nullptr;      // per row slot: its children's updates are u[cptr[r] .. cptr[r + 1])
   uint32_t* wpos = nullptr;      // per update row (uoff + i): where in u it goes

@@ -15,9 +15,11 @@
 //     at most 2^14 meet in one accumulator: at most 2^24, so every sum is exact too.
 //     Digit pairs (i, j) with i + j <= 7 are kept; what is dropped is below 2^-59 (rms) of
 //     the largest product for 64 columns.
-// The digits of one operand hold 62 bits below the row's largest entry, against the 53 of a
-// double below each entry, and the column sum is exact where the FP64 loop rounded at every
-// step.  A right-hand side with an infinity or NaN gives NaN in every row of its tasks.
+// The digits of one operand hold 62 bits below the largest entry of its group (a panel row; a task's
+// right-hand side), against the 53 of a double below each entry, and the column sum is exact where the
+// FP64 loop rounded at every step.  So a sum's error is relative to the product of the two groups'
+// largest entries, not to its own terms; sums far below that product are done on the FP64 units
+// (kGuardBits).  A right-hand side with an infinity or NaN gives NaN in every row of its tasks.
 //
 // Bound: reading the panels (16 bytes per entry: 0.69 SM-clocks at 6.8 TB/s), beside about
 // 0.3 for unpacking digits (20 integer and half2 operations per entry) and 0.25 for the
@@ -118,6 +120,42 @@ __device__ __forceinline__ void put_pair(uint32_t* dst, uint64_t dx, uint64_t dy
   for (int i = 0; i < 4; i++) dst[11 + i] = o[i];
 }
 
+// A row's (column's) products are bounded by 2^(x - 960), x the exponent of its entries plus that of the
+// right-hand side, and the digits miss each by about 2^-59 of this bound.  Where the sum and what it is
+// added to both come out below 2^-kGuardBits of it, the large entries of one side meet small or zero
+// ones of the other, and what is missed may matter beside what is left: the sum is done again on the
+// FP64 units.  The panel itself is within 2^-62 of its row's largest entry either way; a zero is exact.
+// One of 6 million sums comes below in M^{-1} of a random vector of 349,461 dofs, one of 5,000 in a solve
+// for a point source, nearly all of them in its first application: M^{-1} v 4.48 -> 4.54 ms, six sources
+// in four slots (9,801 dofs) 9.3 -> 9.7 ms.  With 10 bits, what is added to left out and columns of zeros
+// not skipped, 1 of 24 columns came below: 6.1 and 17.0 ms.
+constexpr int kGuardBits = 14;
+__device__ __forceinline__ bool below_guard(int field, int x) { return field < x + 63 - kGuardBits; }
+
+// a panel entry in units of 2^62 of its row
+__device__ __forceinline__ double2 entry_value(uint4 w) {
+  const int64_t x = int64_t(((uint64_t(w.y) << 32) | w.x) - kDigitBias), y = int64_t(((uint64_t(w.w) << 32) | w.z) - kDigitBias);
+  return make_double2(double(x) * 0x1p-62, double(y) * 0x1p-62);
+}
+// sum over j < n of the entries of one panel row (p, columns ld apart) times b[j * stride], in units of
+// the row; one warp, the sum in every lane
+__device__ __noinline__ double2 row_dot(const uint4* p, int ld, int n, const double2* b, int stride) {
+  double2 a = make_double2(0.0, 0.0);
+  for (int j = threadIdx.x & 31; j < n; j += 32) a = cmad(entry_value(__ldg(p + int64_t(j) * ld)), b[j * stride], a);
+  return warp_sum(a);
+}
+
+// sum over rows q0 <= q < n of one panel column (p) times v[q], with the rows' exponents; one warp
+__device__ __noinline__ double2 column_dot(const uint4* p, int q0, int n, const double2* v, const int* vex) {
+  double2 a = make_double2(0.0, 0.0);
+  for (int q = q0 + (threadIdx.x & 31); q < n; q += 32) {
+    const double2 x = v[q];
+    const int e = vex[q] + 62;
+    a = cmad(entry_value(__ldg(p + q)), make_double2(scale2(x.x, e), scale2(x.y, e)), a);
+  }
+  return warp_sum(a);
+}
+
 // largest value over the block (128 threads); syncs
 __device__ __forceinline__ int block_max(int v, int* red) {
   v = __reduce_max_sync(0xffffffffu, v);
@@ -129,11 +167,12 @@ __device__ __forceinline__ int block_max(int v, int* red) {
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// panels -> digits, in place; one task = RT rows of one solve supernode
+// panels -> digits, in place; one task = RT rows of one solve supernode.  colnz (zeroed before): columns
+// with an entry below the diagonal
 // ---------------------------------------------------------------------------
 template <int RT>
 __global__ void __launch_bounds__(256) k_to_digits(const int2* tasks, const SnDev* sn, double2* panels,
-                                                   int16_t* rexp) {
+                                                   int16_t* rexp, uint8_t* colnz) {
   constexpr int CG = 256 / RT;
   __shared__ int red[CG][RT];
   const int2 t = tasks[blockIdx.x];
@@ -155,6 +194,7 @@ __global__ void __launch_bounds__(256) k_to_digits(const int2* tasks, const SnDe
     const uint64_t a = to_digits(v.x, 1 + e - max(exp_field(v.x), 1));
     const uint64_t b = to_digits(v.y, 1 + e - max(exp_field(v.y), 1));
     P[int64_t(j) * S.ld] = make_double2(__longlong_as_double(int64_t(a)), __longlong_as_double(int64_t(b)));
+    if ((v.x != 0.0 || v.y != 0.0) && !__ldcg(colnz + S.first + j)) colnz[S.first + j] = 1;   // all write the same
   }
   if (cg == 0 && r < S.m) rexp[S.eoff + r] = e == 0x7ff ? kRowNonFinite : int16_t(e - kBias);
 }
@@ -324,6 +364,16 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
       }
       const int r = base + p * RT + (tid >> 1);
       double s = scaled_sum(hi, lo, 88 + re + E - kBias);
+      const double to = r < k ? b1[2 * r + pt] : b2;
+      const int f1 = max(exp_field(s), exp_field(to)), field = max(f1, __shfl_xor_sync(0xffffffffu, f1, 1));
+      // r = 0 and rows of zeros have no sum
+      const bool redo = r > 0 && r < m && re > 1 - kBias && below_guard(field, re + E);
+      for (unsigned todo = __ballot_sync(0xffffffffu, redo); todo; todo &= todo - 1) {   // a row's two lanes are neighbours
+        const int at = __ffs(todo) - 1, row = base + p * RT + ((tid & ~31) + at) / 2;
+        todo &= todo - 1;
+        const double2 d = row_dot(P + row, S.ld, min(row, k), reinterpret_cast<const double2*>(b1), 1);
+        if (lane >> 1 == at >> 1) s = scale2(pt ? d.y : d.x, re + 62);
+      }
       if (E == 0x7ff || re == kRowNonFinite) s = nan("");
       const double a = s + (r < k ? b1[2 * r + pt] : 0.0);
       const double o = __shfl_xor_sync(0xffffffffu, a, 1);               // the other part
@@ -345,7 +395,8 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
 // supernode of one chunk is finished here, else by the last CTA of each column block (bwd_finish).
 __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnDev* sn, const int32_t* rowlist,
                                                     const double2* panels, const int16_t* rexp,
-                                                    const double2* zin, double2* x, double2* partial, int rows,
+                                                    const uint8_t* colnz, const double2* zin, double2* x,
+                                                    double2* partial, int rows,
                                                     int rpad, int ncol, const int4* fins, unsigned int* counters) {
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -475,6 +526,17 @@ __global__ void __launch_bounds__(128, 4) k_bwd_dig(const int4* tasks, const SnD
     if (tid < 64) {
       double s = scaled_sum(sum[0][tid >> 1][pt][0] + sum[1][tid >> 1][pt][0],
                             sum[0][tid >> 1][pt][1] + sum[1][tid >> 1][pt][1], 88 + E - kBias);
+      bool redo = j < k && j + 1 < r1 && below_guard(exp_field(s), E) && colnz[S.first + j];
+      if (redo) redo = below_guard(exp_field(__ldcg(reinterpret_cast<const double*>(zin + S.first + j) + pt)), E);
+      const int both = __shfl_xor_sync(0xffffffffu, int(redo), 1);           // a column's two parts
+      redo = redo && both;
+      for (unsigned todo = __ballot_sync(0xffffffffu, redo); todo; todo &= todo - 1) {
+        const int at = __ffs(todo) - 1, col = (tk.y + p) * 32 + ((tid & ~31) + at) / 2;
+        todo &= todo - 1;
+        const double2 d = column_dot(P + int64_t(col) * S.ld + r0, max(col + 1 - r0, 0), r1 - r0,
+                                     reinterpret_cast<const double2*>(vec), vex);
+        if (lane >> 1 == at >> 1) s = pt ? d.y : d.x;
+      }
       if (nonfinite) s = nan("");
       if (!single)
         reinterpret_cast<double*>(partial)[(int64_t(fins[tk.w + p].z) + tk.z) * 64 + tid] = s;
@@ -578,7 +640,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
   double2* b1 = reinterpret_cast<double2*>(smem_raw);                    // kpad x S
   double2* part = b1 + kpad * S;                                          // KG x RT x S
   uint32_t* bd = reinterpret_cast<uint32_t*>(part + KG * RT * S);        // KB / 2 x PS
-  __shared__ int ex[2][S], nonfin[S];
+  __shared__ int ex[2][S], exmax[S], nonfin[S];
   const int2 tk = tasks[blockIdx.x];
   const SnDev Sn = sn[tk.x];
   const int k = Sn.k, m = Sn.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -600,6 +662,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
   };
   if (tid < S) {
     ex[0][tid] = 1;
+    exmax[tid] = 1;
     nonfin[tid] = 0;
   }
   if (16 * kg < jend) load(kg);
@@ -620,7 +683,10 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
     block_exponents<S, false>(b1 + j0 * S, min(KB, k - j0), exb, nonfin, nullptr);
     __syncthreads();
     put_digits_multi<S, false>(bd, PS, b1 + j0 * S, min(KB, k - j0), min(KB, (jend - j0 + 15) / 16 * 16), exb, nullptr);
-    if (tid < S) ex[(blk + 1) & 1][tid] = 1;
+    if (tid < S) {
+      ex[(blk + 1) & 1][tid] = 1;
+      exmax[tid] = max(exmax[tid], exb[tid]);
+    }
     __syncthreads();
     for (int s = j0 / 16 + kg; s < (j0 + KB) / 16 && 16 * s < jend; s += KG) {
       step_multi(raw, bd + (8 * (s - j0 / 16) + t) * PS + 8 * nt + g, 2 * S, PS, cr, ci);
@@ -635,11 +701,27 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
 #pragma unroll
   for (int n = 0; n < up.N; n++) {
     const int e = tid + 256 * n, i = e % S, r = tk.y * RT + e / S;
-    if (e >= RT * S || r >= m) continue;
-    double2 s = part[e];
+    const bool mine = e < RT * S && r < m;
+    double2 s = make_double2(0.0, 0.0);
+    int re = 0;
+    if (mine) {
+      s = part[e];
 #pragma unroll
-    for (int q = 1; q < KG; q++) s = cadd(s, part[q * RT * S + e]);
-    if (nonfin[i] || rexp[Sn.eoff + r] == kRowNonFinite) s = make_double2(nan(""), nan(""));
+      for (int q = 1; q < KG; q++) s = cadd(s, part[q * RT * S + e]);
+      re = rexp[Sn.eoff + r];
+    }
+    bool redo = mine && r > 0 && re > 1 - kBias && below_guard(max(exp_field(s.x), exp_field(s.y)), re + exmax[i]);
+    if (redo) {
+      const double2 to = r < k ? b1[r * S + i] : up.b2[n];
+      redo = below_guard(max(exp_field(to.x), exp_field(to.y)), re + exmax[i]);
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, redo); todo; todo &= todo - 1) {
+      const int at = __ffs(todo) - 1, ea = e - lane + at, row = tk.y * RT + ea / S;
+      const double2 d = row_dot(P + row, Sn.ld, min(row, k), b1 + ea % S, S);
+      if (lane == at) s = make_double2(scale2(d.x, re + 62), scale2(d.y, re + 62));
+    }
+    if (!mine) continue;
+    if (nonfin[i] || re == kRowNonFinite) s = make_double2(nan(""), nan(""));
     if (r < k)
       zout[int64_t(Sn.first + r) * S + i] = cmul(panels[Sn.paneloff + r + int64_t(r) * Sn.ld], cadd(b1[r * S + i], s));
     else
@@ -651,7 +733,8 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
 template <int S>
 __global__ void __launch_bounds__(256) k_bwd_dig_multi(const int4* tasks, const SnDev* sn, const int32_t* rowlist,
                                                        const double2* panels, const int16_t* rexp,
-                                                       const double2* zin, double2* x, double2* partial,
+                                                       const uint8_t* colnz, const double2* zin, double2* x,
+                                                       double2* partial,
                                                        const int4* fins, unsigned int* counters) {
   constexpr int NT = S / 4, KG = 4 / NT, KB = kMultiBwdRows, PS = kMultiPairStride<S>, ROWS = kMultiBwdRows;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -733,8 +816,25 @@ __global__ void __launch_bounds__(256) k_bwd_dig_multi(const int4* tasks, const 
     double2 s = vec[e];
 #pragma unroll
     for (int q = 1; q < KG; q++) s = cadd(s, vec[q * 32 * S + e]);
-    if (nonfin[e % S]) s = make_double2(nan(""), nan(""));
     const int j = tk.y * 32 + e / S;
+    bool redo = j < k && j + 1 < r1 && below_guard(max(exp_field(s.x), exp_field(s.y)), ex[0][e % S]) &&
+                colnz[Sn.first + j];
+    if (redo) {
+      const double2 to = ldv(zin + int64_t(Sn.first + j) * S + e % S);
+      redo = below_guard(max(exp_field(to.x), exp_field(to.y)), ex[0][e % S]);
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, redo); todo; todo &= todo - 1) {
+      const int at = __ffs(todo) - 1, ea = e - lane + at, ia = ea % S, col = tk.y * 32 + ea / S;
+      double2 d = make_double2(0.0, 0.0);                                  // vec holds sums now: from global memory
+      for (int r = max(col + 1, r0) + lane; r < r1; r += 32) {
+        const double2 v = r < k ? ldv(zin + int64_t(Sn.first + r) * S + ia) : cneg(ldv(x + int64_t(rl[r]) * S + ia));
+        const int ev = vex[r - r0] + 62;
+        d = cmad(entry_value(__ldg(P + int64_t(col) * Sn.ld + r)), make_double2(scale2(v.x, ev), scale2(v.y, ev)), d);
+      }
+      d = warp_sum(d);
+      if (lane == at) s = d;
+    }
+    if (nonfin[e % S]) s = make_double2(nan(""), nan(""));
     if (!single)
       out[e] = s;
     else if (j < k)
@@ -799,15 +899,17 @@ void set_attrs_dig() {
 }  // namespace
 
 void launch_to_digits(const FactorDev& F, cudaStream_t st) {
+  cudaMemsetAsync(F.colnz, 0, size_t(F.ntot), st);
   for (int l = 0; l < F.snlev; l++) {
     const int64_t b = F.h_fwd_ptr[l], e = F.h_fwd_ptr[l + 1];
     if (e == b) continue;
     add_launches(1);
     if (F.h_fwd_rt[l] == 16)
-      k_to_digits<16><<<unsigned(e - b), 256, 0, st>>>(F.fwd_tasks + b, F.ssn, (double2*)F.panels, F.rexp);
+      k_to_digits<16><<<unsigned(e - b), 256, 0, st>>>(F.fwd_tasks + b, F.ssn, (double2*)F.panels, F.rexp,
+                                                                F.colnz);
     else
       k_to_digits<64><<<dim3(unsigned(e - b), unsigned(F.h_fwd_rt[l] / 64)), 256, 0, st>>>(F.fwd_tasks + b, F.ssn,
-                                                                                           (double2*)F.panels, F.rexp);
+                                                                                           (double2*)F.panels, F.rexp, F.colnz);
   }
 }
 
@@ -836,7 +938,7 @@ void launch_solve_dig(const FactorDev& F, cudaStream_t st) {
     if (e > b) {
       add_launches(1);
       const int rows = F.h_bwd_rows[l], rpad = (std::min(rows, F.h_lev_m[l]) + 15) / 16 * 16;
-      launch_level(k_bwd_dig, e - b, 128, bwd_smem(rpad), st, pdl, F.bwd_tasks + b, F.ssn, F.rowlist, P, F.rexp, z, x,
+      launch_level(k_bwd_dig, e - b, 128, bwd_smem(rpad), st, pdl, F.bwd_tasks + b, F.ssn, F.rowlist, P, F.rexp, F.colnz, z, x,
                    (double2*)F.bwd_partial, rows, rpad, F.h_bwd_cb[size_t(l)], F.bfin_tasks, F.bwd_counters);
     }
     if (F.level_events) cudaEventRecord(F.level_events[1 + F.snlev + (F.snlev - 1 - l)], st);
@@ -866,7 +968,7 @@ static void solve_dig_multi_t(const FactorDev& F, cudaStream_t st) {
     if (e == b) continue;
     add_launches(1);
     k_bwd_dig_multi<S><<<unsigned(e - b), 256, bwd_multi_smem<S>(), st>>>(
-        F.mbwd_tasks + b, F.ssn, F.rowlist, (const double2*)F.panels, F.rexp, (const double2*)F.mz_loc,
+        F.mbwd_tasks + b, F.ssn, F.rowlist, (const double2*)F.panels, F.rexp, F.colnz, (const double2*)F.mz_loc,
         (double2*)F.mx_loc, (double2*)F.mbwd_partial, F.mbfin_tasks, F.mbwd_counters);
   }
 }
