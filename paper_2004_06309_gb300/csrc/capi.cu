@@ -128,8 +128,10 @@ hz_status fail(hz_ctx* c, hz_status s, const std::string& msg) {
 #define CU(call)                                                                          \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
-    if (e_ != cudaSuccess)                                                                \
+    if (e_ != cudaSuccess) {                                                              \
+      cudaGetLastError(); /* reported here, not again by the next call's check */         \
       return fail(c, HZ_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_));   \
+    }                                                                                     \
   } while (0)
 
 template <typename T>
@@ -884,12 +886,29 @@ void free_host_ptrs(hz::FactorDev& F) {
   F.h_bfin_ptr = F.h_lev_ptr = F.h_fwd_ptr = F.h_bwd_ptr = F.h_wg_ptr = F.h_cb_ptr = F.h_ea_ptr = F.h_ent_ptr = nullptr;
 }
 
-// One numeric factorisation on a stream: its workspace and its status word.
+// One numeric factorisation on a stream: its workspace, given back however it ends, and its status word.
 struct FactorRun {
-  hz::FactorDev* F = nullptr;
-  cudaStream_t st = nullptr;
-  hz::DevStatus* status = nullptr;
+  hz_ctx* c;
+  hz::FactorDev* F;
+  cudaStream_t st;
+  hz::DevStatus* status;
   char *fronts = nullptr, *scratch = nullptr;
+  FactorRun(hz_ctx* c_, hz::FactorDev& F_, cudaStream_t st_, hz::DevStatus* status_)
+      : c(c_), F(&F_), st(st_), status(status_) {}
+  FactorRun(const FactorRun&) = delete;
+  FactorRun& operator=(const FactorRun&) = delete;
+  ~FactorRun() {
+    if (fronts || scratch) {                       // an error on the way: kernels may still use them
+      cudaStreamSynchronize(st);
+      release();
+      cudaGetLastError();
+    }
+  }
+  void release() {
+    dfree(c, fronts);
+    dfree(c, scratch);
+    fronts = scratch = nullptr;
+  }
 };
 
 int64_t factor_workspace(const hz::FactorDev& F) {
@@ -901,7 +920,8 @@ bool factor_verbose() {
   return verbose;
 }
 
-hz_status factor_alloc(hz_ctx* c, FactorRun& r) {
+hz_status factor_alloc(FactorRun& r) {
+  hz_ctx* c = r.c;
   const hz::FactorDev& F = *r.F;
   if (F.nsn == 0) return HZ_OK;
   auto t0 = std::chrono::steady_clock::now();
@@ -909,8 +929,7 @@ hz_status factor_alloc(hz_ctx* c, FactorRun& r) {
   TRY(dalloc(c, &r.fronts, F.front_elems * vs));
   const hz_status s = dalloc(c, &r.scratch, std::max<int64_t>(F.scratch_elems, 1) * vs);
   if (s != HZ_OK) {
-    dfree(c, r.fronts);
-    r.fronts = nullptr;
+    r.release();
     return s;
   }
   if (factor_verbose())
@@ -919,7 +938,8 @@ hz_status factor_alloc(hz_ctx* c, FactorRun& r) {
   return HZ_OK;
 }
 
-hz_status factor_launch(hz_ctx* c, FactorRun& r, double w, const double maxabs[3]) {
+hz_status factor_launch(FactorRun& r, double w, const double maxabs[3]) {
+  hz_ctx* c = r.c;
   hz::FactorDev& F = *r.F;
   if (F.nsn == 0) return HZ_OK;
   const bool verbose = factor_verbose();
@@ -947,15 +967,14 @@ hz_status factor_launch(hz_ctx* c, FactorRun& r, double w, const double maxabs[3
 }
 
 // Waits for the factorisation, gives its workspace back and judges it.
-hz_status factor_finish(hz_ctx* c, FactorRun& r, double& min_pivot) {
+hz_status factor_finish(FactorRun& r, double& min_pivot) {
+  hz_ctx* c = r.c;
   if (r.F->nsn == 0) return HZ_OK;
   auto t0 = std::chrono::steady_clock::now();
   hz::DevStatus out{};
   CU(cudaMemcpyAsync(&out, r.status, sizeof(out), cudaMemcpyDeviceToHost, r.st));
   CU(cudaStreamSynchronize(r.st));
-  dfree(c, r.fronts);
-  dfree(c, r.scratch);
-  r.fronts = r.scratch = nullptr;
+  r.release();
   if (factor_verbose())
     std::fprintf(stderr, "[hz] factor: status read and workspace freed in %.3f s\n",
                  std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
@@ -969,13 +988,10 @@ hz_status factor_finish(hz_ctx* c, FactorRun& r, double& min_pivot) {
 }
 
 hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[3], double& min_pivot) {
-  FactorRun r;
-  r.F = &F;
-  r.st = c->st;
-  r.status = c->status;
-  TRY(factor_alloc(c, r));
-  TRY(factor_launch(c, r, w, maxabs));
-  return factor_finish(c, r, min_pivot);
+  FactorRun r(c, F, c->st, c->status);
+  TRY(factor_alloc(r));
+  TRY(factor_launch(r, w, maxabs));
+  return factor_finish(r, min_pivot);
 }
 
 // The subdomain factors on the context's stream and the coarse factor on its side stream at the
@@ -988,36 +1004,36 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
 // 349,461 dofs, mixed (coarse factor 54,925 dofs, 36 levels): hz_factor 105.1 -> 86.8 ms; 54,925
 // dofs, FP64: 41.2 -> 36.0 ms.
 hz_status factor_both(hz_ctx* c, double w, double& min_pivot, bool& coarse_follows) {
-  FactorRun a, b;
-  a.F = &c->loc;
-  a.st = c->st;
-  a.status = c->status;
-  b.F = &c->crs;
-  b.st = c->side;
-  b.status = c->status + 1;
+  FactorRun a(c, c->loc, c->st, c->status), b(c, c->crs, c->side, c->status + 1);
   coarse_follows = true;
-  TRY(factor_alloc(c, a));
+  TRY(factor_alloc(a));
   const int64_t need = factor_workspace(c->crs);
   size_t free_bytes = 0, total_bytes = 0;
   CU(cudaMemGetInfo(&free_bytes, &total_bytes));
   const bool fits = need <= int64_t(free_bytes / 4) &&
                     (!c->opt.hbm_budget || uint64_t(c->bytes) + uint64_t(need) <= c->opt.hbm_budget);
-  if (fits && factor_alloc(c, b) == HZ_OK) coarse_follows = false;
+  const std::string before = c->err;
+  if (fits && factor_alloc(b) == HZ_OK) coarse_follows = false;
   if (coarse_follows) {
-    TRY(factor_launch(c, a, w, c->loc_max));
-    return factor_finish(c, a, min_pivot);
+    c->err = before;                               // no room for both is no error
+    TRY(factor_launch(a, w, c->loc_max));
+    return factor_finish(a, min_pivot);
   }
   hz_status s = HZ_OK;
   if (cudaEventRecord(c->side_ev, c->st) != cudaSuccess || cudaStreamWaitEvent(c->side, c->side_ev, 0) != cudaSuccess)
     s = fail(c, HZ_ERR_CUDA, "ordering the coarse factorisation after the context's stream");
-  if (s == HZ_OK) s = factor_launch(c, b, w, c->crs_max);
-  if (s == HZ_OK) s = factor_launch(c, a, w, c->loc_max);
+  if (s == HZ_OK) s = factor_launch(b, w, c->crs_max);
+  if (s == HZ_OK) s = factor_launch(a, w, c->loc_max);
+  const std::string es = c->err;
   // both are waited for whatever either gives: their workspaces go back.  The host wait for
   // the side stream orders it before anything that the context's stream does next.
-  const hz_status sa = factor_finish(c, a, min_pivot);
+  const hz_status sa = factor_finish(a, min_pivot);
   const std::string ea = c->err;
-  const hz_status sb = factor_finish(c, b, min_pivot);
-  if (s != HZ_OK) return s;
+  const hz_status sb = factor_finish(b, min_pivot);
+  if (s != HZ_OK) {
+    c->err = es;
+    return s;
+  }
   if (sa != HZ_OK) {
     c->err = ea;                                   // the subdomains' failure is the one reported, as in serial order
     return sa;
