@@ -185,12 +185,16 @@ std::vector<double2> to_d2(const std::vector<cplx>& v) {
   return o;
 }
 
-// Device copy of a symbolic set with its task lists.
+bool verbose_log() {
+  static const bool verbose = std::getenv("HZ_VERBOSE") != nullptr;
+  return verbose;
+}
+
 // Task shapes of the batched triangular sweeps per assembly-tree level, and the kernel
 // variants they imply (host-only; shared by the device upload and hz_plan).
-// Sparse tree levels get narrow tasks.  complex128 (FP64 arithmetic bound): fewer
-// tasks than two per SM -> 16-row forward tasks, 64-row backward chunks, so that such a
-// level reaches every SM.  complex64: fewer tasks than one resident wave (8 CTAs per
+// Sparse tree levels get narrow tasks.  complex128: fewer tasks than two per SM -> 16-row
+// forward tasks, 64-row backward chunks, so that such a level reaches every SM; enough for three
+// waves -> tasks of up to 256 rows or four 32-column blocks.  complex64: fewer tasks than one resident wave (8 CTAs per
 // SM) -> 64-row forward tasks and 128-row backward chunks, which shorten each task's
 // serial walk over its columns and rows (the time of a latency-bound level).
 // sweep_tasks (hz_options) forces wide (1) or narrow (2) shapes on every level.
@@ -346,6 +350,12 @@ SweepPlan plan_sweeps(const TreeView& S, int precision, int bwd_rows, int sweep_
         sp.tc_kstages = std::max(sp.tc_kstages, (2 * k + 31) / 32);
       }
     }
+  }
+  if (precision == 0 && verbose_log()) {
+    auto levels = [](const std::vector<int>& v, int x) { return int(std::count(v.begin(), v.end(), x)); };
+    std::fprintf(stderr, "[hz] sweep tasks: levels of 16/64/128/256 rows %d/%d/%d/%d, of 1/2/4 column blocks %d/%d/%d\n",
+                 levels(sp.fwd_rt, 16), levels(sp.fwd_rt, 64), levels(sp.fwd_rt, 128), levels(sp.fwd_rt, 256),
+                 levels(sp.bwd_cb, 1), levels(sp.bwd_cb, 2), levels(sp.bwd_cb, 4));
   }
   return sp;
 }
@@ -915,11 +925,6 @@ int64_t factor_workspace(const hz::FactorDev& F) {
   return (F.front_elems + std::max<int64_t>(F.scratch_elems, 1)) * (F.precision == 0 ? 16 : 8);
 }
 
-bool factor_verbose() {
-  static const bool verbose = std::getenv("HZ_VERBOSE") != nullptr;
-  return verbose;
-}
-
 hz_status factor_alloc(FactorRun& r) {
   hz_ctx* c = r.c;
   const hz::FactorDev& F = *r.F;
@@ -932,7 +937,7 @@ hz_status factor_alloc(FactorRun& r) {
     r.release();
     return s;
   }
-  if (factor_verbose())
+  if (verbose_log())
     std::fprintf(stderr, "[hz] factor: workspace %.2f GB allocated in %.3f s\n", double(F.front_elems) * double(vs) / 1e9,
                  std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
   return HZ_OK;
@@ -942,7 +947,7 @@ hz_status factor_launch(FactorRun& r, double w, const double maxabs[3]) {
   hz_ctx* c = r.c;
   hz::FactorDev& F = *r.F;
   if (F.nsn == 0) return HZ_OK;
-  const bool verbose = factor_verbose();
+  const bool verbose = verbose_log();
   auto t0 = std::chrono::steady_clock::now();
   hz::DevStatus init{0u, 0u, 0.0};   // zero_pivot, timeout, min_pivot
   const double big = 1e300;
@@ -975,7 +980,7 @@ hz_status factor_finish(FactorRun& r, double& min_pivot) {
   CU(cudaMemcpyAsync(&out, r.status, sizeof(out), cudaMemcpyDeviceToHost, r.st));
   CU(cudaStreamSynchronize(r.st));
   r.release();
-  if (factor_verbose())
+  if (verbose_log())
     std::fprintf(stderr, "[hz] factor: status read and workspace freed in %.3f s\n",
                  std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
   min_pivot = std::min(min_pivot, out.min_pivot);
