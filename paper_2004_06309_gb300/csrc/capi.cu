@@ -528,12 +528,12 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
     sn[s].rowoff = S.sn_rowoff[s];
     // complex64 panels: columns padded to 4 rows (32 bytes) for 16-byte vector loads
     sn[s].ld = precision == 0 ? S.sn_m[s] : (S.sn_m[s] + 3) / 4 * 4;
-    sn[s].pad_ = 0;
+    sn[s].id = s;
     sn[s].paneloff = panel_off;
     panel_off += int64_t(sn[s].ld) * S.sn_k[s];
-    sn[s].uoff = S.sn_uoff[s];
     sn[s].frontoff = S.sn_frontoff[s];
-    sn[s].eoff = 0;
+    sn[s].ubase = S.cptr[size_t(S.sn_rowoff[s])];
+    sn[s].wbase = S.sn_parent[s] < 0 ? 0 : S.cptr[size_t(S.sn_rowoff[S.sn_parent[s]])];
     F.maxk = std::max(F.maxk, S.sn_k[s]);
     F.maxm = std::max(F.maxm, S.sn_m[s]);
   }
@@ -560,7 +560,7 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
       d.m = ST.m[ci];
       d.ld = precision == 0 ? d.m : (d.m + 3) / 4 * 4;     // complex64: 16-byte aligned row pairs
       d.parent = S.sn_parent[ch.back()];
-      d.uoff = S.sn_uoff[ch.back()];
+      d.wbase = sn[size_t(ch.back())].wbase;
       d.paneloff = off;
       int w = 0;
       for (int32_t s : ch) {
@@ -587,11 +587,17 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
   {
     // update vectors are stored in the order in which the parents' rows read them (a parent row's
     // child contributions are adjacent): u index of row slot r, child rank q = cptr[r] + q, and
-    // wpos gives the index that each update row writes
-    if (S.cptr.back() >= int64_t(1) << 32 || S.u_elems >= int64_t(1) << 32)
-      return fail(c, HZ_ERR_OOM, "more update rows than a device holds");
-    std::vector<uint32_t> p32(S.cptr.begin(), S.cptr.end()), w(size_t(S.u_elems), 0u);
-    for (size_t q = 0; q < S.cidx.size(); q++) w[size_t(S.cidx[q])] = uint32_t(q);
+    // wpos gives the index that each update row writes, both from the start of the parent's
+    std::vector<uint32_t> p32(size_t(S.sn_rowoff[ns] + ns)), to(size_t(S.u_elems)), w(size_t(S.sn_rowoff[ns]), 0u);
+    for (int s = 0; s < ns; s++) {
+      const int64_t* cp = S.cptr.data() + S.sn_rowoff[s];
+      for (int r = 0; r <= S.sn_m[s]; r++) p32[size_t(S.sn_rowoff[s] + s + r)] = uint32_t(cp[r] - cp[0]);
+      for (int64_t q = cp[0]; q < cp[S.sn_m[s]]; q++) to[size_t(S.cidx[size_t(q)])] = uint32_t(q - cp[0]);
+    }
+    for (size_t ci = 0; ci < ST.chains.size(); ci++) {   // a chain's update rows are its last member's
+      const int32_t a = ST.chains[ci].front(), b = ST.chains[ci].back();
+      std::copy_n(to.begin() + S.sn_uoff[b], ST.m[ci] - ST.k[ci], w.begin() + S.sn_rowoff[a] + ST.k[ci]);
+    }
     TRY(upload(c, &F.cptr, p32));
     TRY(upload(c, &F.wpos, w));
   }

@@ -14,17 +14,21 @@ constexpr int kMultiBwdRows = 128;  // rows per backward task of the batched swe
 constexpr int kWgRows = 64;          // rows per complex64 off-diagonal task (32 in complex128)
 constexpr int kCbRows = 128;        // rows per complex128 Schur update task (of 16 columns)
 
-// One supernode of a batched multifrontal factorisation (64 bytes).
-
+// One supernode of a batched multifrontal factorisation (64 bytes: every task reads one).
 struct SnDev {
   int32_t k, m, first, parent;   // pivots, front order, first vector index, parent (-1 root)
-  int32_t ld, pad_;              // panel leading dimension (m, or m rounded up to 4 for complex64)
-  int64_t rowoff;                // into rowlist / cptr slots
+  int32_t ld;                    // panel leading dimension (m, or m rounded up to 4 for complex64)
+  int32_t id;                    // number of the supernode (of a merged chain's first one)
+  int64_t rowoff;                // into rowlist and wpos; into cptr at rowoff + id, m + 1 slots
+  int64_t ubase, wbase;          // into u: its children's updates start here, and its parent's
   int64_t paneloff;              // panel (m x k, column-major, ld m) in the factor store
-  int64_t uoff;                  // update rows (m - k): index into wpos
-  int64_t frontoff;              // front (m x m, column-major) in the frontal workspace
-  int64_t eoff;                  // complex128 solve tree: row exponents of the panel's digits (m of them)
+  union {
+    int64_t frontoff;            // factorisation: front (m x m, column-major) in the frontal workspace
+    int64_t eoff;                // complex128 solve tree: row exponents of the panel's digits (m of them)
+  };
 };
+
+static_assert(sizeof(SnDev) == 64, "two sectors");
 
 // Device view of a batched symbolic factorisation plus its numeric factor.
 struct FactorDev {
@@ -54,8 +58,10 @@ struct FactorDev {
   int16_t* rexp = nullptr;            // complex128: exponent of each solve panel row's digits (sweeps64.cu)
   uint8_t* colnz = nullptr;           // complex128: columns (vector index) of solve panels with entries below the diagonal
   int32_t* rowlist = nullptr;
-  uint32_t* cptr = nullptr;      // per row slot: its children's updates are u[cptr[r] .. cptr[r + 1])
-  uint32_t* wpos = nullptr;      // per update row (uoff + i): where in u it goes
+  // a supernode's row r: its children's updates are u[ubase + cptr[rowoff + id + r] .. [.. + r + 1]); as an
+  // update row (r >= k) it goes to u[wbase + wpos[rowoff + r]].  Offsets within a supernode fit 32 bits, u need not
+  uint32_t* cptr = nullptr;
+  uint32_t* wpos = nullptr;
   int32_t* rel = nullptr;
   int64_t* reloff = nullptr;
   int32_t* gidx = nullptr;       // ntot: global index of each local vector entry

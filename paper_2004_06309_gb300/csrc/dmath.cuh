@@ -186,10 +186,10 @@ template <typename V, int S, int RT> struct UpdateRows {
       const bool ok = e < RT * LR && r >= Sn.k && r < Sn.m;
       c0[q] = ok ? cp[r] : 0u;
       c1[q] = ok ? cp[r + 1] : 0u;
-      to[q] = ok ? wpos[Sn.uoff + (r - Sn.k)] : 0u;
+      to[q] = ok ? wpos[Sn.rowoff + r] : 0u;
       b2[q] = vzero<T>();
     }
-    add_contributions<V, LR, N>(b2, c0, c1, u, threadIdx.x % LR);
+    add_contributions<V, LR, N>(b2, c0, c1, u + Sn.ubase * S, threadIdx.x % LR);
   }
 };
 

@@ -609,14 +609,16 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
   const SnDev S = sn[t.x];
   const int k = S.k, m = S.m, tid = threadIdx.x;
   const int pr = tid % NP, cg = tid / NP;
-  const uint32_t* cp = cptr + S.rowoff;
+  const uint32_t* cp = cptr + S.rowoff + S.id;
+  const float2* ub = u + S.ubase;
   const int r = t.y * ROWS + 2 * pr;                 // rows r, r + 1 (r even, ld % 4 == 0)
   const int rr = t.y * ROWS + tid;                   // update row finished by this thread
   // where this thread's child contributions lie and where its update goes: loaded before the
   // wait for the previous level, so that only the contributions themselves come after it
   const bool upd = tid < ROWS && rr >= k && rr < m;
   const uint32_t g0 = tid < k ? cp[tid] : 0u, g1 = tid < k ? cp[tid + 1] : 0u;
-  const uint32_t h0 = upd ? cp[rr] : 0u, h1 = upd ? cp[rr + 1] : 0u, uw = upd ? wpos[S.uoff + (rr - k)] : 0u;
+  const uint32_t h0 = upd ? cp[rr] : 0u, h1 = upd ? cp[rr + 1] : 0u;
+  float2* uw = u + (upd ? S.wbase + wpos[S.rowoff + rr] : 0);
   float2 a0 = make_float2(0.f, 0.f), a1 = a0, c0 = a0, c1 = a0, b2 = a0;
   if constexpr (CG == 8) {
     constexpr int MQ = kMaxK / CG, PF = 8;              // PF of the MQ columns are prefetched,
@@ -640,10 +642,10 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
     for (int jj = tid; jj < k; jj += 256) {
       const uint32_t c0 = jj == tid ? g0 : cp[jj], c1 = jj == tid ? g1 : cp[jj + 1];
       float2 acc = ldv(tin + S.first + jj);
-      for (uint32_t c = c0; c < c1; c++) acc = cadd(acc, ldv(u + c));
+      for (uint32_t c = c0; c < c1; c++) acc = cadd(acc, ldv(ub + c));
       b1[jj] = acc;
     }
-    for (uint32_t c = h0; c < h1; c++) b2 = cadd(b2, ldv(u + c));
+    for (uint32_t c = h0; c < h1; c++) b2 = cadd(b2, ldv(ub + c));
     if constexpr (NA > 0) cp_async_wait_all();        // each thread reads back only its own copies
     __syncthreads();
     if (r < m) {
@@ -703,10 +705,10 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
     for (int jj = tid; jj < k; jj += 256) {
       const uint32_t c0 = jj == tid ? g0 : cp[jj], c1 = jj == tid ? g1 : cp[jj + 1];
       float2 acc = ldv(tin + S.first + jj);
-      for (uint32_t c = c0; c < c1; c++) acc = cadd(acc, ldv(u + c));
+      for (uint32_t c = c0; c < c1; c++) acc = cadd(acc, ldv(ub + c));
       b1[jj] = acc;
     }
-    for (uint32_t c = h0; c < h1; c++) b2 = cadd(b2, ldv(u + c));
+    for (uint32_t c = h0; c < h1; c++) b2 = cadd(b2, ldv(ub + c));
     if constexpr (NA > 0) cp_async_wait_all();        // each thread reads back only its own copies
     __syncthreads();
     if (r < m) {
@@ -768,7 +770,7 @@ __device__ __forceinline__ void fwd_c64_item(const int2 t, const SnDev* sn, cons
     if (rr < k)
       zout[S.first + rr] = cmul(P[rr + int64_t(rr) * S.ld], cadd(b1[rr], tot));
     else
-      u[uw] = csub(b2, tot);
+      *uw = csub(b2, tot);
   }
 }
 

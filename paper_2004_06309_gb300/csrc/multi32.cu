@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd_multi32(const int2* tasks, const
   const SnDev Sn = sn[tk.x];
   const int k = Sn.k, m = Sn.m, tid = threadIdx.x;
   const int tg = tid % TG, kg = tid / TG, rg = tg % (RT / 4), hg = tg / (RT / 4);
-  const uint32_t* cp = cptr + Sn.rowoff;
+  const uint32_t* cp = cptr + Sn.rowoff + Sn.id;
   const int row0 = tk.y * RT;
   const int jend = min(min(row0 + RT, m) - 1, k);                          // columns any row of the task uses
   auto issue = [&](int c) {                                                // columns c CC .. of the panel into slot c & 1
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd_multi32(const int2* tasks, const
   };
   issue(0);
   issue(1);
-  gather_rows<float2, S>(b1, tin + int64_t(Sn.first) * S, cp, u, k);
+  gather_rows<float2, S>(b1, tin + int64_t(Sn.first) * S, cp, u + Sn.ubase * S, k);
   UpdateRows<float2, S, RT> up;
   up.load(Sn, cp, wpos, u, row0);
   float2 acc[4][4];
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd_multi32(const int2* tasks, const
       const float2 z0 = cmul(d, make_float2(a.x, a.y)), z1 = cmul(d, make_float2(a.z, a.w));
       reinterpret_cast<float4*>(zout)[int64_t(Sn.first + r) * LR + i] = make_float4(z0.x, z0.y, z1.x, z1.y);
     } else {
-      reinterpret_cast<float4*>(u)[int64_t(up.to[n]) * LR + i] = vsub(up.b2[n], s);
+      reinterpret_cast<float4*>(u)[(Sn.wbase + up.to[n]) * LR + i] = vsub(up.b2[n], s);
     }
   }
 }

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
   const SnDev S = sn[tk.x];
   const int k = S.k, m = S.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int g = lane >> 2, t = lane & 3, mt = wid % MT, cg = wid / MT;
-  const uint32_t* cp = cptr + S.rowoff;
+  const uint32_t* cp = cptr + S.rowoff + S.id;
   const int base = tk.y * RT * npass, np = min(npass, (m - base + RT - 1) / RT);
   const uint4* P = reinterpret_cast<const uint4*>(panels + S.paneloff);
   uint4* myring = ring + wid * (kRing * 256) + lane;
@@ -278,14 +278,14 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
     if (mine && r < k) dinv = panels[S.paneloff + r + int64_t(r) * S.ld];
     h0 = upd ? cp[r] : 0u;
     h1 = upd ? cp[r + 1] : 0u;
-    uw = upd ? wpos[S.uoff + (r - k)] : 0u;
+    uw = upd ? wpos[S.rowoff + r] : 0u;
   };
   load_row(0);
   const uint32_t g0 = tid < 2 * k ? cp[tid >> 1] : 0u, g1 = tid < 2 * k ? cp[(tid >> 1) + 1] : 0u;
   const int q1 = tid + 128;
   const uint32_t g2 = q1 < 2 * k ? cp[q1 >> 1] : 0u, g3 = q1 < 2 * k ? cp[(q1 >> 1) + 1] : 0u;
   pdl_wait();
-  const double *tind = reinterpret_cast<const double*>(tin + S.first), *ud = reinterpret_cast<const double*>(u);
+  const double *tind = reinterpret_cast<const double*>(tin + S.first), *ud = reinterpret_cast<const double*>(u + S.ubase);
   int e = 1;
   {
     // the first two rounds (64 columns each) have their row pointers and load together
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(128, 4) k_fwd_dig(const int2* tasks, const SnD
         if (r < k)
           reinterpret_cast<double*>(zout + S.first + r)[pt] = fma(dinv.x, a, pt ? dinv.y * o : -dinv.y * o);
         else
-          reinterpret_cast<double*>(u + uw)[pt] = b2 - s;
+          reinterpret_cast<double*>(u + S.wbase + uw)[pt] = b2 - s;
       }
     }
     load_row(p + 1);
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
   const SnDev Sn = sn[tk.x];
   const int k = Sn.k, m = Sn.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int g = lane >> 2, t = lane & 3, nt = wid % NT, mt = (wid / NT) % MT, kg = wid / (NT * MT);
-  const uint32_t* cp = cptr + Sn.rowoff;
+  const uint32_t* cp = cptr + Sn.rowoff + Sn.id;
   const int row0 = tk.y * RT + mt * 16, ra = row0 + g, rb = ra + 8;
   const int ja = ra < m ? min(ra, k) : 0, jb = rb < m ? min(rb, k) : 0;
   const int jend = min(min(tk.y * RT + RT - 1, m - 1), k);               // columns any row of the task needs
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
     nonfin[tid] = 0;
   }
   if (16 * kg < jend) load(kg);
-  gather_rows<double2, S>(b1, tin + int64_t(Sn.first) * S, cp, u, k);
+  gather_rows<double2, S>(b1, tin + int64_t(Sn.first) * S, cp, u + Sn.ubase * S, k);
   UpdateRows<double2, S, RT> up;
   up.load(Sn, cp, wpos, u, tk.y * RT);
   float cr[8][4], ci[8][4];
@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(256) k_fwd_dig_multi(const int2* tasks, const 
     if (r < k)
       zout[int64_t(Sn.first + r) * S + i] = cmul(panels[Sn.paneloff + r + int64_t(r) * Sn.ld], cadd(b1[r * S + i], s));
     else
-      u[int64_t(up.to[n]) * S + i] = csub(up.b2[n], s);
+      u[(Sn.wbase + up.to[n]) * S + i] = csub(up.b2[n], s);
   }
 }
 
