@@ -1008,7 +1008,9 @@ hz_status factor_one(hz_ctx* c, hz::FactorDev& F, double w, const double maxabs[
 // The subdomain factors on the context's stream and the coarse factor on its side stream at the
 // same time.  The coarse factor is one matrix: above the first few of its tree levels a launch holds
 // a handful of CTAs, whose serial pivot blocks set the time while the subdomains' launches fill
-// the GPU.  The side stream has the higher priority, so that this chain is not queued behind them.
+// the GPU.  The side stream has the context's priority: with the device's highest one the coarse
+// factor also ran ahead of other contexts' solves, and the two together were no faster (349,461 dofs
+// mixed 69.9 ms, 68.5 with equal priority; FP64 365, 362).
 // The subdomain factor's workspace comes first, as without the side stream; the coarse one's is
 // then taken only if it leaves three quarters of the free memory and fits the context's limit,
 // else coarse_follows is set and nothing of the coarse factor has run.
@@ -2676,9 +2678,12 @@ static hz_status populate(hz_ctx* c, hz::HostProblem& P, int order, const hz_opt
   SETUP_TRY(dalloc(c, &c->brk, 1));
   SETUP_TRY(dalloc(c, &c->status, 2));            // the subdomains' factor, the coarse factor
   if (c->levels == 2 && !c->coarse_oras) {
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi) != cudaSuccess ||
+    int prio = 0;
+    if (cudaStreamGetPriority(c->st, &prio) != cudaSuccess) {
+      cudaGetLastError();
+      prio = 0;
+    }
+    if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, prio) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->side_ev, cudaEventDisableTiming) != cudaSuccess)
       SETUP_TRY(fail(c, HZ_ERR_CUDA, "creating the coarse factorisation's stream"));
   }
