@@ -580,6 +580,8 @@ hz_status upload_factor(hz_ctx* c, const hz::SymbolicSet& S, int precision, int6
       }
       TRY(dalloc(c, &F.rexp, std::max<int64_t>(rows, 1)));
       TRY(dalloc(c, &F.colnz, std::max<int64_t>(F.ntot, 1)));
+      TRY(dalloc(c, &F.sig, std::max<int64_t>(F.ntot, 1)));
+      TRY(upload(c, &F.ediag, S.ediag));
     }
     TRY(upload(c, &F.ssn, ssn));
   }
@@ -964,6 +966,7 @@ hz_status factor_launch(FactorRun& r, double w, const double maxabs[3]) {
     cudaStreamSynchronize(r.st);
     t0 = std::chrono::steady_clock::now();
   }
+  if (F.precision == 0) hz::launch_scaling(F, w, r.st);
   for (int g = 0; g < F.ngrp; g++)                 // groups one after the other in one workspace
     for (int l = 0; l < F.nlev; l++) hz::launch_factor_level(F, l, g, w, r.fronts, r.scratch, r.status, tiny, r.st);
   hz::launch_merge_panels(F, r.st);               // merged solve supernodes of the sweeps

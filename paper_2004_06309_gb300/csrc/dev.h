@@ -56,6 +56,10 @@ struct FactorDev {
   int64_t merge_tmp_elems = 0;
   void* merge_tmp = nullptr;
   int16_t* rexp = nullptr;            // complex128: exponent of each solve panel row's digits (sweeps64.cu)
+  // complex128: A is factorised with rows and columns scaled by 2^-sig, sig half the exponent of the
+  // diagonal entry (launch_scaling): per vector index, and the entry of its diagonal
+  int16_t* sig = nullptr;
+  int64_t* ediag = nullptr;
   uint8_t* colnz = nullptr;           // complex128: columns (vector index) of solve panels with entries below the diagonal
   int32_t* rowlist = nullptr;
   // a supernode's row r: its children's updates are u[ubase + cptr[rowoff + id + r] .. [.. + r + 1]); as an
@@ -203,14 +207,17 @@ long long launch_count();
 void add_launches(long long n);   // kernels replayed inside a CUDA graph launch
 void launch_fill_values(int64_t nnz, const double* K, const double2* M, const double2* B, double w,
                         double2* out, cudaStream_t st);
+// complex128: the scaling of A(omega), before its first level.
+void launch_scaling(const FactorDev& F, double w, cudaStream_t st);
 // One assembly-tree level: zero and fill its fronts (A_i(omega) entries), extend-add the
 // children, factor, and copy the panels to the factor store.
 void launch_factor_level(const FactorDev& F, int lev, int grp, double w, void* fronts, void* scratch,
                          DevStatus* status, double tiny, cudaStream_t st);
 
 // Pivot blocks of one level (diag.cu): F11 = L D L^T, T = L^{-1} in place, D^{-1} on the diagonal.
-void launch_diag(int precision, int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, void* fronts,
-                 DevStatus* status, double tiny, cudaStream_t st);
+// sig: complex128, the scaling, taken out of the pivots' magnitudes.
+void launch_diag(int precision, int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, const int16_t* sig,
+                 void* fronts, DevStatus* status, double tiny, cudaStream_t st);
 
 // Complex128 products of one factor level and of the merged solve panels (factor64.cu).
 void launch_wg_dig(int64_t ntask, int maxk, const int2* tasks, const FactorDev& F, double2* fronts, double2* scratch,

@@ -74,7 +74,7 @@ __device__ __forceinline__ void put_operand_pair(uint32_t* dst, int n, uint4 x, 
 }  // namespace
 
 template <typename V>
-__global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, const SnDev* sn, V* fronts,
+__global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, const SnDev* sn, const int16_t* sig, V* fronts,
                                                      DevStatus* status, double tiny) {
   using L = DiagLayout<V>;
   constexpr int P = L::pitch, BLK = 16 * P;
@@ -414,7 +414,8 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
   }
   if (tid < k) {
     const V d = dval[tid];
-    const double mag = sqrt(double(d.x) * double(d.x) + double(d.y) * double(d.y));
+    double mag = sqrt(double(d.x) * double(d.x) + double(d.y) * double(d.y));
+    if constexpr (dbl) mag *= exp2i(2 * sig[S.first + tid]);
     atomicMin(reinterpret_cast<unsigned long long*>(&status->min_pivot),
               static_cast<unsigned long long>(__double_as_longlong(mag)));
     if (!(mag >= tiny)) atomicOr(&status->zero_pivot, 1u);
@@ -425,21 +426,21 @@ __global__ void __launch_bounds__(256, 1) k_diag_blk(const int32_t* lev_sn, cons
 }
 
 template <typename V>
-static void launch_diag_t(int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, V* fronts, DevStatus* status,
-                          double tiny, cudaStream_t st) {
+static void launch_diag_t(int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, const int16_t* sig, V* fronts,
+                          DevStatus* status, double tiny, cudaStream_t st) {
   static const bool attr = [] {
     cudaFuncSetAttribute(k_diag_blk<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     return true;
   }();
   (void)attr;
   add_launches(1);
-  k_diag_blk<V><<<unsigned(nb), 256, diag_bytes<V>((maxk + 15) / 16), st>>>(lev_sn, sn, fronts, status, tiny);
+  k_diag_blk<V><<<unsigned(nb), 256, diag_bytes<V>((maxk + 15) / 16), st>>>(lev_sn, sn, sig, fronts, status, tiny);
 }
 
-void launch_diag(int precision, int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, void* fronts,
-                 DevStatus* status, double tiny, cudaStream_t st) {
-  if (precision == 0) launch_diag_t(nb, maxk, lev_sn, sn, (double2*)fronts, status, tiny, st);
-  else launch_diag_t(nb, maxk, lev_sn, sn, (float2*)fronts, status, tiny, st);
+void launch_diag(int precision, int64_t nb, int maxk, const int32_t* lev_sn, const SnDev* sn, const int16_t* sig,
+                 void* fronts, DevStatus* status, double tiny, cudaStream_t st) {
+  if (precision == 0) launch_diag_t(nb, maxk, lev_sn, sn, sig, (double2*)fronts, status, tiny, st);
+  else launch_diag_t(nb, maxk, lev_sn, sn, sig, (float2*)fronts, status, tiny, st);
 }
 
 }  // namespace hz

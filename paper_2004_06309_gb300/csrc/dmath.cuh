@@ -20,6 +20,9 @@ template <typename V> struct RealOf;
 template <> struct RealOf<float2> { using T = float; };
 template <> struct RealOf<double2> { using T = double; };
 
+// 2^e, |e| <= 1000
+__device__ __forceinline__ double exp2i(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
 template <typename V>
 __device__ __forceinline__ V mk(typename RealOf<V>::T x, typename RealOf<V>::T y) {
   V v;

@@ -71,6 +71,7 @@ struct SymbolicSet {
   std::vector<int64_t> ent_gptr;       // nlev * (groups + 1): entries of each (level, group)
   std::vector<double> ek;
   std::vector<cplx> em, eb;
+  std::vector<int64_t> ediag;          // voff.back(): entry of each vector index's diagonal (-1: none)
   // extend-add: relative positions of each child's contribution rows in its parent
   std::vector<int64_t> sn_reloff;
   std::vector<int32_t> rel;

@@ -67,6 +67,52 @@ __global__ void k_front_fill(int64_t ne, const int64_t* epos, const double* K, c
 }
 
 // ---------------------------------------------------------------------------
+// complex128: symmetric scaling by powers of two.  The factorisation's products hold their operands as
+// digits below the largest entry of a row (digits.cuh), so rows of A of very different size (wave
+// speeds spread over 10^12 within a subdomain) would cost the small ones their digits.  With
+// S A S, S = 2^-sig, the diagonal is within [1/2, 4), and so the rows of L D^(1/2).  A^{-1} v =
+// S (S A S)^{-1} S v: powers of two change no digit of the vectors either.
+// ---------------------------------------------------------------------------
+constexpr int kMaxSig = 200;
+__global__ void k_scaling(int64_t ntot, const int64_t* ediag, const double* K, const double2* M, const double2* B,
+                          double w, int16_t* sig) {
+  for (int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; l < ntot; l += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t e = ediag[l];
+    int s = 0;
+    if (e >= 0) {
+      const double2 v = helmholtz_value(K[e], M[e], B[e], w);
+      const double a = fmax(fabs(v.x), fabs(v.y));
+      if (a > 0.0 && isfinite(a)) s = max(-kMaxSig, min(kMaxSig, ilogb(a) >> 1));
+    }
+    sig[l] = int16_t(s);
+  }
+}
+
+void launch_scaling(const FactorDev& F, double w, cudaStream_t st) {
+  if (F.ntot == 0) return;
+  HZ_COUNT();
+  k_scaling<<<grid_for(F.ntot, 256), 256, 0, st>>>(F.ntot, F.ediag, F.ek, F.em, F.eb, w, F.sig);
+}
+
+// A's entries of a level's fronts (their pivot columns), after k_front_fill; grid as k_front_zero's
+__global__ void __launch_bounds__(256) k_front_scale(const int32_t* lev_sn, const SnDev* sn, const int32_t* rowlist,
+                                                     const int16_t* sig, double2* fronts) {
+  const SnDev S = sn[lev_sn[blockIdx.x]];
+  double2* f = fronts + S.frontoff;
+  const int32_t* rl = rowlist + S.rowoff;
+  for (int j = blockIdx.y * 8 + (threadIdx.x >> 5); j < S.k; j += 8 * gridDim.y) {
+    const int sj = sig[S.first + j];
+    for (int r = j + (threadIdx.x & 31); r < S.m; r += 32) {
+      const double2 v = f[int64_t(j) * S.m + r];
+      if (v.x != 0.0 || v.y != 0.0) {
+        const double c = exp2i(-sj - sig[rl[r]]);
+        f[int64_t(j) * S.m + r] = make_double2(v.x * c, v.y * c);
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // multifrontal factorisation, one assembly-tree level at a time
 // ---------------------------------------------------------------------------
 
@@ -514,6 +560,13 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
     k_front_fill<V><<<grid_for(e1 - e0, 256), 256, 0, st>>>(e1 - e0, F.epos + e0, F.ek + e0, F.em + e0, F.eb + e0,
                                                            w, fronts);
   }
+  if constexpr (sizeof(V) == 16) {
+    if (nb > 0) {
+      HZ_COUNT();
+      k_front_scale<<<dim3(unsigned(nb), split_for(nb, F.h_flev_k[size_t(lev)])), 256, 0, st>>>(lsn, F.sn, F.rowlist,
+                                                                                               F.sig, fronts);
+    }
+  }
   // extend-add, one child slot per launch so that no parent entry is written twice
   for (int q = 0; q < F.max_slot; q++) {
     int64_t b, e;
@@ -525,7 +578,7 @@ static void factor_level_t(const FactorDev& F, int lev, int grp, double w, V* fr
   }
   if (nb == 0) return;
   const int maxk = F.h_flev_k[size_t(lev)];
-  launch_diag(F.precision, nb, maxk, lsn, F.sn, fronts, status, tiny, st);
+  launch_diag(F.precision, nb, maxk, lsn, F.sn, F.sig, fronts, status, tiny, st);
   int64_t wb, we;
   range(F.h_wg_g, lev, wb, we);
   if (we > wb) {
@@ -576,10 +629,23 @@ void launch_factor_level(const FactorDev& F, int lev, int grp, double w, void* f
 // ---------------------------------------------------------------------------
 // batched supernodal solves  (A_i^{-1}: forward with D^{-1}, then backward)
 // ---------------------------------------------------------------------------
+// a vector entry on its way into the factor's scaling and out of it (complex128 factors)
+template <typename V> __device__ __forceinline__ V scaled_in(double2 v, const int16_t* sig, int64_t l) {
+  if constexpr (sizeof(V) == 16) {
+    const double c = exp2i(-sig[l]);
+    return make_double2(v.x * c, v.y * c);
+  } else {
+    return from2<V>(v);
+  }
+}
+template <typename V> __device__ __forceinline__ double scaled_weight(double pw, const int16_t* sig, int32_t l) {
+  if constexpr (sizeof(V) == 16) return pw * exp2i(-sig[l]);
+  else return pw;
+}
 template <typename V>
-__global__ void k_gather(int64_t ntot, const int32_t* gidx, const double2* src, V* dst) {
+__global__ void k_gather(int64_t ntot, const int32_t* gidx, const int16_t* sig, const double2* src, V* dst) {
   for (int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; q < ntot; q += int64_t(gridDim.x) * blockDim.x)
-    dst[q] = from2<V>(src[gidx[q]]);
+    dst[q] = scaled_in<V>(src[gidx[q]], sig, q);
 }
 
 // Backward, split over row chunks so that tall supernodes use many CTAs:
@@ -897,14 +963,15 @@ __global__ void __launch_bounds__(256, MODE == kBwdPrefetch ? 4 : 6)
 }
 
 template <typename V>
-__global__ void k_prolong(int64_t n, const int64_t* pptr, const int32_t* pidx, const double* pw, const V* xl,
-                          const double2* y, double2* z) {
+__global__ void k_prolong(int64_t n, const int64_t* pptr, const int32_t* pidx, const double* pw, const int16_t* sig,
+                          const V* xl, const double2* y, double2* z) {
   for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
     double2 acc = y ? y[g] : make_double2(0.0, 0.0);
     for (int64_t q = pptr[g]; q < pptr[g + 1]; q++) {
       const double2 v = to2(xl[pidx[q]]);
-      acc.x = xfma(pw[q], v.x, acc.x);
-      acc.y = xfma(pw[q], v.y, acc.y);
+      const double c = scaled_weight<V>(pw[q], sig, pidx[q]);
+      acc.x = xfma(c, v.x, acc.x);
+      acc.y = xfma(c, v.y, acc.y);
     }
     z[g] = acc;
   }
@@ -949,10 +1016,10 @@ void launch_gather(const FactorDev& F, const double2* src, cudaStream_t st) {
   if (F.ntot == 0) return;
   if (F.precision == 0) {
     HZ_COUNT();
-    k_gather<double2><<<grid_for(F.ntot, 256), 256, 0, st>>>(F.ntot, F.gidx, src, (double2*)F.t_loc);
+    k_gather<double2><<<grid_for(F.ntot, 256), 256, 0, st>>>(F.ntot, F.gidx, F.sig, src, (double2*)F.t_loc);
   } else {
     HZ_COUNT();
-    k_gather<float2><<<grid_for(F.ntot, 256), 256, 0, st>>>(F.ntot, F.gidx, src, (float2*)F.t_loc);
+    k_gather<float2><<<grid_for(F.ntot, 256), 256, 0, st>>>(F.ntot, F.gidx, F.sig, src, (float2*)F.t_loc);
   }
 }
 
@@ -1086,11 +1153,11 @@ void launch_prolong(const FactorDev& F, const double2* y, double2* z, cudaStream
   if (F.nglob == 0) return;
   if (F.precision == 0) {
     HZ_COUNT();
-    k_prolong<double2><<<grid_for(F.nglob, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw,
+    k_prolong<double2><<<grid_for(F.nglob, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw, F.sig,
                                                                (const double2*)F.x_loc, y, z);
   } else {
     HZ_COUNT();
-    k_prolong<float2><<<grid_for(F.nglob, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw,
+    k_prolong<float2><<<grid_for(F.nglob, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw, F.sig,
                                                               (const float2*)F.x_loc, y, z);
   }
 }
@@ -1101,25 +1168,26 @@ void launch_prolong(const FactorDev& F, const double2* y, double2* z, cudaStream
 // read once and used for all S right-hand sides.
 // ---------------------------------------------------------------------------
 template <typename V, int S>
-__global__ void k_gather_multi(int64_t ntot, const int32_t* gidx, const double2* src, V* dst) {
+__global__ void k_gather_multi(int64_t ntot, const int32_t* gidx, const int16_t* sig, const double2* src, V* dst) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < ntot * S; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t q = e / S;
     const int i = int(e % S);
-    dst[e] = from2<V>(src[int64_t(gidx[q]) * S + i]);
+    dst[e] = scaled_in<V>(src[int64_t(gidx[q]) * S + i], sig, q);
   }
 }
 
 template <typename V, int S>
-__global__ void k_prolong_multi(int64_t n, const int64_t* pptr, const int32_t* pidx, const double* pw, const V* xl,
-                                const double2* y, double2* z) {
+__global__ void k_prolong_multi(int64_t n, const int64_t* pptr, const int32_t* pidx, const double* pw, const int16_t* sig,
+                                const V* xl, const double2* y, double2* z) {
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n * S; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t g = e / S;
     const int i = int(e % S);
     double2 acc = y ? y[e] : make_double2(0.0, 0.0);
     for (int64_t q = pptr[g]; q < pptr[g + 1]; q++) {
       const double2 v = to2(xl[int64_t(pidx[q]) * S + i]);
-      acc.x = xfma(pw[q], v.x, acc.x);
-      acc.y = xfma(pw[q], v.y, acc.y);
+      const double c = scaled_weight<V>(pw[q], sig, pidx[q]);
+      acc.x = xfma(c, v.x, acc.x);
+      acc.y = xfma(c, v.y, acc.y);
     }
     z[e] = acc;
   }
@@ -1129,11 +1197,11 @@ template <typename V, int S>
 static void prec_multi_t(const FactorDev& F, const double2* src, const double2* y, double2* dst, cudaStream_t st) {
   V* t = (V*)F.mt_loc;
   HZ_COUNT();
-  k_gather_multi<V, S><<<grid_for(F.ntot * S, 256), 256, 0, st>>>(F.ntot, F.gidx, src, t);
+  k_gather_multi<V, S><<<grid_for(F.ntot * S, 256), 256, 0, st>>>(F.ntot, F.gidx, F.sig, src, t);
   if constexpr (sizeof(V) == 8) launch_solve_multi32(F, S, st);
   else launch_solve_dig_multi(F, S, st);
   HZ_COUNT();
-  k_prolong_multi<V, S><<<grid_for(F.nglob * S, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw,
+  k_prolong_multi<V, S><<<grid_for(F.nglob * S, 256), 256, 0, st>>>(F.nglob, F.pptr, F.pidx, F.pw, F.sig,
                                                                    (const V*)F.mx_loc, y, dst);
 }
 

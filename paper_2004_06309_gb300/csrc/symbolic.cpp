@@ -25,6 +25,8 @@ struct SymOne {
   // lower-triangle entries: supernode-relative front offset (row + col*m) and source entry
   std::vector<int32_t> e_sn;
   std::vector<int64_t> e_off, e_src;
+  std::vector<int64_t> d_ent;        // diagonal entries (indices into the above), ascending
+  std::vector<int32_t> d_pos;        // ... and their positions
 };
 
 struct NDState {
@@ -163,6 +165,10 @@ void analyse_one(const MatrixInput& in, int leaf, int maxsn, SymOne& S) {
       const int64_t m = S.rowoff[s + 1] - S.rowoff[s];
       const int32_t* b = S.rows.data() + S.rowoff[s];
       const int64_t row = std::lower_bound(b, b + m, pr) - b;
+      if (pr == pc) {
+        S.d_ent.push_back(int64_t(S.e_sn.size()));
+        S.d_pos.push_back(pr);
+      }
       S.e_sn.push_back(s);
       S.e_off.push_back(row + int64_t(pc - S.first[s]) * m);
       S.e_src.push_back(t);
@@ -347,12 +353,15 @@ void symbolic_batch(const std::vector<MatrixInput>& mats, int leaf, int maxsn, S
   }
   {
     std::vector<int64_t> fill(S.ent_ptr.begin(), S.ent_ptr.end() - 1);
+    S.ediag.assign(size_t(ntot), -1);
     for (int i = 0; i < nmat; i++) {
       SymOne& O = one[i];
       const Parts& A = *mats[i].A;
+      size_t nd = 0;
       for (size_t t = 0; t < O.e_sn.size(); t++) {
         const int32_t g = sn_base[i] + O.e_sn[t];
         const int64_t q = fill[S.sn_level[g]]++;
+        if (nd < O.d_ent.size() && O.d_ent[nd] == int64_t(t)) S.ediag[size_t(S.voff[i] + O.d_pos[nd++])] = q;
         S.epos[q] = S.sn_frontoff[g] + O.e_off[t];
         S.ek[q] = A.K[O.e_src[t]];
         S.em[q] = A.M[O.e_src[t]];

@@ -9,7 +9,13 @@ less than a double holds of an entry 2^40 below it.
 - One subdomain is A^{-1}: the residual |A z - v| of every row within 1e-12 of (|A| |z| + |v|) of that row
   for entries spread over 2^40, at random and along an axis.  A sum that is left to the digits, or what it
   is added to, is at least 2^-14 of its bound, and the digits miss 2^-59 (rms) of this bound per
-  column: 2^-45 sqrt(448) = 6e-13 of it for the widest supernode."""
+  column: 2^-45 sqrt(448) = 6e-13 of it for the widest supernode.
+- The same bound for random vectors on matrices whose rows differ: wave speeds 10^12 apart from element to
+  element, and element layers 10^6 thinner than their neighbours, with the library's own A (its product
+  adds 30 entries x 2^-53 per row).  The factorisation scales rows and columns by powers of two for
+  this; unscaled, the rows were off by up to 3e-9 of their terms.  Vectors whose solution decays by more
+  than about 2^40 within a supernode are outside the bound in such media: the panels hold 62 bits below
+  their rows' largest entries.  The smallest pivot stays that of the unscaled matrix."""
 import numpy as np
 import pytest
 
@@ -104,3 +110,45 @@ def test_graded_vectors_row_by_row(hzmod, kw):
         z = G.apply_M(torch.from_numpy(b).cuda()).cpu().numpy()
         assert np.all(np.abs(S.A @ z - b) <= 1e-12 * (abs(S.A) @ np.abs(z) + np.abs(b)))
     G.close()
+
+
+def _contrast():
+    p = synth.unit_cube_problem(n=8, order=2, nsub=1, overlap=0, freq=1.2)
+    p.c = p.c * 10.0 ** np.random.default_rng(1).uniform(-6, 6, len(p.c))
+    return p
+
+
+def _layers():
+    p = synth.unit_cube_problem(n=8, order=2, nsub=1, overlap=0, freq=0.3)
+    z = np.concatenate([[0.0], np.cumsum([1, 1, 1, 1e-6, 1e-6, 1e-6, 1e-6, 1])])
+    a = np.linspace(0.0, 1.0, 9)
+    p.mesh = synth.kuhn_box_mesh(a, a, z / z[-1])
+    return p
+
+
+@pytest.mark.parametrize("make", [_contrast, _layers])
+@pytest.mark.parametrize("kw", [dict(), dict(max_snode=17, leaf_size=8)])
+def test_rows_of_very_different_size(hzmod, make, kw):
+    import torch
+    p = make()
+    S = OracleSolver(p)
+    rng = np.random.default_rng(5)
+    v = rng.standard_normal(S.n) + 1j * rng.standard_normal(S.n)
+    G = hzmod.Solver(p, **kw)
+    G.factor()
+    z = G.apply_M(torch.from_numpy(v).cuda())
+    r = v - G.apply_A(z).cpu().numpy()
+    G.close()
+    assert np.all(np.abs(r) <= 1e-12 * (abs(S.A) @ np.abs(z.cpu().numpy()) + np.abs(v)))
+
+
+def test_smallest_pivot_is_the_unscaled_one(hzmod):
+    """Of a diagonal-dominated matrix (wave speed 10^-3: -w^2 M) in both precisions, to complex64 rounding."""
+    p = synth.unit_cube_problem(n=6, order=1, nsub=3, overlap=1, freq=1.2, c=1e-3 * (1 - 0.01j))
+    out = []
+    for precision in (hzmod.HZ_FP64, hzmod.HZ_MIXED):
+        G = hzmod.Solver(p, precision=precision)
+        G.factor()
+        out.append(G.stats()["min_pivot"])
+        G.close()
+    assert abs(out[0] - out[1]) <= 1e-4 * out[1]
