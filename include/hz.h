@@ -83,7 +83,16 @@ typedef struct {
   int32_t overlap;          /* delta: element layers grown through shared vertices   */
   int32_t levels;           /* 1 (Eq. 4) or 2 (Eq. 3)                                */
   int32_t restart;          /* m of FGMRES(m)                                        */
-  int32_t precision;        /* HZ_FP64, or HZ_MIXED: subdomain factors/solves c64    */
+  int32_t precision;        /* HZ_FP64, or HZ_MIXED: subdomain factors/solves c64.
+                               Complex128 factors (HZ_FP64, and the direct coarse
+                               solve's) multiply fixed-point operands of 62 bits below
+                               the largest entry of a factor row or of a supernode's
+                               right-hand side, with exact sums, on rows and columns
+                               scaled by powers of two; sums more than 2^14 below
+                               their bound are done in FP64.  Normwise the error is
+                               below that of FP64 sums; single entries of A_i^{-1} v
+                               that lie more than about 2^40 below the largest of
+                               their supernode, scaled, can have fewer correct digits */
   int32_t max_iter;         /* total inner-iteration limit per right-hand side       */
   int32_t leaf_size;        /* nested-dissection leaf size (0: default 64)           */
   int32_t max_snode;        /* widest supernode (0: default 128; capped at 112 for
@@ -140,8 +149,9 @@ typedef struct {
                                narrow tasks); 1: wide tasks on every level; 2: narrow
                                tasks on every level.  Wide: 256-row forward tasks and
                                bwd_chunk-row backward chunks (complex64), 64 / bwd_chunk
-                               (complex128); narrow: 64 / 128 (complex64), 16 / 64
-                               (complex128).                                          */
+                               (complex128; with 0, levels of many tasks take up to 256
+                               rows, or four blocks of 32 columns); narrow: 64 / 128
+                               (complex64), 16 / 64 (complex128).                     */
   int32_t bwd_chunk;        /* rows of a wide backward chunk; 0: 512 for complex64 local
                                factors, 256 otherwise; else even, in [32, 512].  A
                                supernode taller than a chunk sums its chunks' partial

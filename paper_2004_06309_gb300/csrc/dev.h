@@ -106,7 +106,7 @@ struct FactorDev {
   int64_t *h_lev_g = nullptr, *h_ent_g = nullptr, *h_wg_g = nullptr, *h_cb_g = nullptr, *h_tc_g = nullptr;
   int64_t* h_ea_g = nullptr;          // ((level * max_slot + slot) * (groups + 1) + group)
   cudaEvent_t* level_events = nullptr;  // optional (diagnostics): 2 * nlev + 1 events around sweep levels
-  int* h_fwd_rt = nullptr;            // nlev: complex128 forward task rows (16 or 64)
+  int* h_fwd_rt = nullptr;            // nlev: forward task rows (complex128: 16, 64, 128 or 256)
   int* h_bwd_rows = nullptr;          // nlev: complex128 backward chunk rows
   // per solve level: widest supernode (rounded up to 16 columns), tallest one, and the rows
   // of the batched forward tasks

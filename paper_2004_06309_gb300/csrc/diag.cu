@@ -12,7 +12,7 @@
 // The unblocked loop (a barrier pair per column and per row of the inverse) took 1.36 ms per
 // level in complex128 (width 112) and 0.61 ms in complex64 (width 128).  A complex128 product is
 // 4 FP64 instructions of 64 clocks per scheduler, whatever its active lanes, so the block
-// products run in exact digits on mma.sync (digits.cuh) and only the 16 x 16 blocks on the FP64
+// products run in digits on mma.sync (digits.cuh) and only the 16 x 16 blocks on the FP64
 // units.  The next pivot's chain (diagonal entry, reciprocal, column) runs in its own warp beside the
 // update, its two parts in different lanes of the same instructions; one after the other a pivot took 2,500
 // clocks.  0.27 ms per level in complex128 and 0.12 ms in complex64 on the same models.

@@ -1,10 +1,19 @@
-// Exact products of complex128 values on the tensor cores.
+// Products of complex128 values on the tensor cores, by splitting the operands into digits whose
+// products and sums are exact (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 2012).
 //
 // A double x of a group whose largest exponent field is E becomes the integer
-// D = x 2^(1084 - E), |D| < 2^62, written as eight balanced base-256 digits in [-128, 127] with
-// 128 added to each (so a byte of the 64-bit word is a digit).  mma.sync m16n8k16 multiplies
-// digits as f16 and adds in f32: a product is at most 2^14, and while at most 2^10 of them meet
-// in one accumulator (8 digit pairs x 128 columns), every sum is below 2^24 and exact.
+// D = x 2^(1084 - E), |D| < 2^62 (its lower bits are cut off), written as eight balanced base-256
+// digits in [-128, 127] with 128 added to each (so a byte of the 64-bit word is a digit).
+// mma.sync m16n8k16 multiplies digits as f16 and adds in f32: a product is at most 2^14, and while at
+// most 2^10 of them meet in one accumulator (8 digit pairs x 128 columns), every sum is below 2^24
+// and exact.
+//
+// Error: D keeps all 53 bits of a value down to 2^-9 of its group's largest, and fewer below; with the
+// digit pairs left out a sum of n products is within about 2^-59 sqrt(n) of the product of the two
+// groups' largest entries.  FP64 sums are within 2^-53 of the sum of the terms' magnitudes.  So the
+// digits are the better ones while the terms reach 2^-6 of that product, as they do for matrices scaled to
+// a diagonal of order one (launch_scaling) and vectors of like entries; the sweeps go back to the FP64
+// units for sums far below it (sweeps64.cu, kGuardBits).
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -97,7 +106,6 @@ __device__ __forceinline__ void step_multi(const uint4* raw, const uint32_t* bd,
   }
 }
 
-// value of the weighted digit sums t[0..7] = result 2^88 2^(exponents)
 // (hi + lo 2^-32) 2^e, rounded once, for |hi|, |lo| < 2^62.  In integer arithmetic: each of the two
 // conversions, the FMA and the scaling holds its scheduler for 64 clocks on the FP64 units.  Same bits;
 // factorisation of 54,925 dofs in FP64 35.9 -> 33.0 ms.

@@ -1,4 +1,4 @@
-// Complex128 products of the factorisation in exact digits on the tensor cores (digits.cuh): the
+// Complex128 products of the factorisation in digits on the tensor cores (digits.cuh): the
 // off-diagonal panels (W = F21 T^T, L21 = W D^{-1}, G = L21 T), the Schur updates
 // F22 -= W L21^T, and the products that merge solve supernodes.  On the FP64 units (2 FMAs per
 // SM and clock) a complex product costs 2 SM-clocks; here 0.14, plus unpacking and the
