@@ -33,7 +33,7 @@ struct hz_ctx {
   // global operator
   int64_t* d_rp = nullptr;
   int32_t* d_ci = nullptr;
-  hz::SpmvRow* d_rows = nullptr;           // rows of the SpMV in its order
+  hz::SpmvRow* d_rows = nullptr;           // rows of the SpMV in its order (null: their own)
   double* d_K = nullptr;
   double2* d_M = nullptr;
   double2* d_B = nullptr;
@@ -51,6 +51,7 @@ struct hz_ctx {
   double cloc_max[3] = {0, 0, 0};
   int32_t* d_Eci = nullptr;
   hz::SpmvRow* d_Erows = nullptr;
+  int64_t* d_Erp = nullptr;
   double* d_EK = nullptr;
   double2 *d_EM = nullptr, *d_EB = nullptr, *d_E = nullptr;
   double2 *VH = nullptr, *ZH = nullptr, *wH = nullptr, *HH = nullptr, *snH = nullptr, *gH = nullptr, *yHs = nullptr;
@@ -1104,7 +1105,7 @@ void coarse_inner(hz_ctx* c, const double2* r, double2* y) {
     hz::launch_gather(c->cloc, vj, st);                                           // R_H,i v
     hz::launch_solve(c->cloc, st);                                                // E_i^{-1}
     hz::launch_prolong(c->cloc, nullptr, zj, st);                                 // sum R^T D x_i
-    hz::launch_spmv(nH, c->d_Erows, c->d_Eci, c->d_E, zj, nullptr, c->wH, st);      // E z_j
+    hz::launch_spmv(nH, c->d_Erows, c->d_Erp, c->d_Eci, c->d_E, zj, nullptr, c->wH, st);      // E z_j
     hz::launch_cgs(nH, j + 1, c->VH, nH, nullptr, c->wH, true, c->partial, c->ticket, c->h1, st);
     hz::launch_cgs(nH, j + 1, c->VH, nH, c->h1, c->wH, true, c->partial, c->ticket, c->h2, st);
     const hz::SlotGivens gv = givens_args(j, mH, c->HH, c->csH, c->snH, c->gH, c->h1, c->h2, c->nrm, c->scalH, 3, c->brkH);
@@ -1141,7 +1142,7 @@ void apply_prec(hz_ctx* c, const double2* v, double2* z) {
     hz::launch_spmv_real(c->nH, c->d_Ztrp, c->d_Ztci, c->d_Ztv, v, c->rH, st);   // r_H = Z^T v
     coarse_solve(c, c->rH, c->yH);                                               // E^{-1}
     hz::launch_spmv_real(c->n, c->d_Zrp, c->d_Zci, c->d_Zv, c->yH, c->y, st);     // y = Z y_H
-    hz::launch_spmv(c->n, c->d_rows, c->d_ci, c->d_A, c->y, v, c->t, st);          // t = v - A y
+    hz::launch_spmv(c->n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->y, v, c->t, st);          // t = v - A y
     hz::launch_gather(c->loc, c->t, st);                                         // R_i t
     hz::launch_solve(c->loc, st);                                                // A_i^{-1}
     hz::launch_prolong(c->loc, c->y, z, st);                                     // y + sum R_i^T D_i x_i
@@ -1172,7 +1173,7 @@ void iteration_kernels(hz_ctx* c, int j) {
   double2* vj = c->V + int64_t(j) * n;
   double2* zj = c->Zs + int64_t(j) * n;
   apply_prec(c, vj, zj);
-  hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, zj, nullptr, c->w, st);
+  hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, zj, nullptr, c->w, st);
   // orthogonalise against [C, v_0..v_j] (C: the recycled space, empty without recycling)
   const int kk = c->ckk, nc = kk + j + 1;
   const double2* base = c->V - int64_t(kk) * n;
@@ -1268,7 +1269,7 @@ hz_status fgmres_one(hz_ctx* c, double tol, hz_rhs_info* info) {
       return HZ_OK;
     }
     hz::launch_update_x(n, k, c->H, m + 1, c->g, c->ysol, c->Zs, n, c->x, st);
-    hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, c->x, c->b, c->w, st);        // r = b - A x
+    hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->x, c->b, c->w, st);        // r = b - A x
     double rn = 0;
     TRY(norm2(c, c->w, rn));
     const double rel = rn / bnorm;
@@ -1515,7 +1516,7 @@ hz_status recycle_rebase(hz_ctx* c) {
   const int kk = c->rdim;
   cudaStream_t st = c->st;
   for (int i = 0; i < kk; i++)
-    hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, c->Ux + int64_t(i) * n, nullptr, c->Ctmp + int64_t(i) * n, st);
+    hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->Ux + int64_t(i) * n, nullptr, c->Ctmp + int64_t(i) * n, st);
   std::vector<double> w0(kk);
   for (int i = 0; i < kk; i++) TRY(norm2(c, c->Ctmp + int64_t(i) * n, w0[i]));
   std::vector<cplx> R;
@@ -1570,7 +1571,7 @@ hz_status gcrodr_one(hz_ctx* c, double tol, hz_rhs_info* info) {
       CU(cudaMemcpyAsync(c->h_pin + 5, &c->nrm[64].x, sizeof(double), cudaMemcpyDeviceToHost, st));
       CU(cudaStreamSynchronize(st));
       if (std::sqrt(c->h_pin[5]) <= 1e-3 * tol * bnorm && !in_span) {
-        hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, c->x, c->b, c->w, st);
+        hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->x, c->b, c->w, st);
         double rn = 0;
         TRY(norm2(c, c->w, rn));
         info->iterations = its;
@@ -1613,7 +1614,7 @@ hz_status gcrodr_one(hz_ctx* c, double tol, hz_rhs_info* info) {
         for (int j = 0; j < k; j++) t[size_t(i)] += Bh[size_t(j) * c->rk + i] * y[size_t(j)];
       combo(c, kk, c->Ux, 0, nullptr, t, 1, c->x, -1.0, true);
     }
-    hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, c->x, c->b, c->w, st);          // r = b - A x
+    hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->x, c->b, c->w, st);          // r = b - A x
     double rn = 0;
     TRY(norm2(c, c->w, rn));
     const double rel = rn / bnorm;
@@ -1799,7 +1800,7 @@ static hz_status slot_end_cycle(hz_ctx* c, int i) {
   double2* xi = slot_col(c, c->Xc, i);
   hz::launch_update_x(n, s.j, c->Hb + int64_t(i) * (m + 1) * m, m + 1, c->gb + int64_t(i) * (m + 1),
                       c->yb + int64_t(i) * m, slot_Z(c, i), n, xi, c->st);
-  hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, xi, slot_col(c, c->Bc, i), slot_col(c, c->Wc, i), c->st);
+  hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, xi, slot_col(c, c->Bc, i), slot_col(c, c->Wc, i), c->st);
   double rn = 0;
   TRY(norm2(c, slot_col(c, c->Wc, i), rn));             // leaves |r|^2 in nrm for a restart
   const double rel = rn / s.bnorm;
@@ -2142,7 +2143,7 @@ hz_status block_batch(hz_ctx* c, int s, double tol, hz_rhs_info* info) {
     // true residuals (into W, the next cycle's residual block)
     bool done = true;
     for (int i = 0; i < s; i++) {
-      hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, c->Xc + int64_t(i) * n, c->Bc + int64_t(i) * n,
+      hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->Xc + int64_t(i) * n, c->Bc + int64_t(i) * n,
                       c->Wc + int64_t(i) * n, st);
       double r;
       TRY(norm2(c, c->Wc + int64_t(i) * n, r));
@@ -2219,9 +2220,9 @@ hz_status tune_spmv(hz_ctx* c) {
   int pick = 8;
   for (int t : {2, 4, 8, 16}) {
     hz::set_spmv_lanes(t);
-    hz::launch_spmv(c->n, c->d_rows, c->d_ci, c->d_A, c->b, nullptr, c->w, c->st);
+    hz::launch_spmv(c->n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->b, nullptr, c->w, c->st);
     CU(cudaEventRecord(e0, c->st));
-    for (int r = 0; r < 3; r++) hz::launch_spmv(c->n, c->d_rows, c->d_ci, c->d_A, c->b, nullptr, c->w, c->st);
+    for (int r = 0; r < 3; r++) hz::launch_spmv(c->n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->b, nullptr, c->w, c->st);
     CU(cudaEventRecord(e1, c->st));
     CU(cudaEventSynchronize(e1));
     float ms = 0;
@@ -2531,10 +2532,27 @@ extern "C" hz_status hz_plan(const hz_mesh_desc* md, const hz_options* op, hz_st
   return HZ_OK;
 }
 
-// Rows sorted by length, longest first, within windows of 4,096 (k_spmv).
+// Rows sorted by length, longest first, within windows of 4,096 (k_spmv), or none for the order they have:
+// where a warp's rows are alike anyway (P1: 1 - 6 % of the steps idle with two lanes per row, P2: 12 - 17 %),
+// and where the matrix is too small to fill the SMs with whole windows.  SpMV in natural order and
+// sorted, best number of lanes: P1, 19,683 rows 6.2 and 7.6 us, P2, 9,801 rows 7.8 and 7.6 us (8 or 4 lanes;
+// 4,913 rows 6.0 and 6.0), 12,321 rows 9.7 and 8.2 us, 54,925 17.9 and 17.2 us, 349,461 94.2 and 86.1 us.
 static std::vector<hz::SpmvRow> spmv_rows(const hz::Csr& A) {
   const int64_t n = int64_t(A.ptr.size()) - 1, W = 4096;
-  std::vector<hz::SpmvRow> o(size_t(std::max<int64_t>(n, 0)));
+  std::vector<hz::SpmvRow> o;
+  if (n <= 3 * W) return o;
+  int64_t steps = 0, longest = 0;
+  for (int64_t b = 0; b + 16 <= n; b += 16) {
+    int64_t most = 0;
+    for (int64_t i = b; i < b + 16; i++) {
+      const int64_t q = (A.ptr[size_t(i) + 1] - A.ptr[size_t(i)] + 1) / 2;
+      steps += q;
+      most = std::max(most, q);
+    }
+    longest += 16 * most;
+  }
+  if (double(steps) > 0.92 * double(longest)) return o;
+  o.resize(size_t(n));
   for (int64_t i = 0; i < n; i++)
     o[size_t(i)] = {A.ptr[size_t(i)], int32_t(A.ptr[size_t(i) + 1] - A.ptr[size_t(i)]), int32_t(i)};
   for (int64_t b = 0; b < n; b += W)
@@ -2614,6 +2632,7 @@ static hz_status populate(hz_ctx* c, hz::HostProblem& P, int order, const hz_opt
                               op->precision == HZ_MIXED ? 512 : 256, 0, op->sweep_tasks, op->bwd_chunk));
       c->cloc.tc_wait = tc_wait;
       SETUP_TRY(upload(c, &c->d_Eci, P.E.pat.col));
+      SETUP_TRY(upload(c, &c->d_Erp, P.E.pat.ptr));
       SETUP_TRY(upload(c, &c->d_Erows, spmv_rows(P.E.pat)));
       SETUP_TRY(upload(c, &c->d_EK, P.E.K));
       SETUP_TRY(upload(c, &c->d_EM, to_d2(P.E.M)));
@@ -2833,7 +2852,7 @@ extern "C" hz_status hz_apply_A(hz_ctx* c, const void* x, void* y) {
   if (c->spmv_lanes) hz::set_spmv_lanes(c->spmv_lanes);
   if (!x || !y) return fail(c, HZ_ERR_ARG, "null vector");
   if (!c->factored) return fail(c, HZ_ERR_STATE, "hz_factor must run first (A depends on the frequency)");
-  hz::launch_spmv(c->n, c->d_rows, c->d_ci, c->d_A, (const double2*)x, nullptr, (double2*)y, c->st);
+  hz::launch_spmv(c->n, c->d_rows, c->d_rp, c->d_ci, c->d_A, (const double2*)x, nullptr, (double2*)y, c->st);
   CU(cudaGetLastError());
   return HZ_OK;
 }
@@ -2928,7 +2947,7 @@ extern "C" hz_status hz_profile(hz_ctx* c, int32_t reps, hz_profile_out* out) {
   const double nt = 16.0;
   auto run = [&](int ph) {
     switch (ph) {
-      case HZ_PH_SPMV: hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, c->b, nullptr, c->w, st); break;
+      case HZ_PH_SPMV: hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, c->b, nullptr, c->w, st); break;
       case HZ_PH_COARSE:
         if (c->levels == 2) {
           hz::launch_spmv_real(c->nH, c->d_Ztrp, c->d_Ztci, c->d_Ztv, c->b, c->rH, st);
@@ -2948,7 +2967,7 @@ extern "C" hz_status hz_profile(hz_ctx* c, int32_t reps, hz_profile_out* out) {
       case HZ_PH_ITERATION: {
         double2* zj = c->Zs + int64_t(jj) * n;
         apply_prec(c, c->V + int64_t(jj) * n, zj);
-        hz::launch_spmv(n, c->d_rows, c->d_ci, c->d_A, zj, nullptr, c->w, st);
+        hz::launch_spmv(n, c->d_rows, c->d_rp, c->d_ci, c->d_A, zj, nullptr, c->w, st);
         hz::launch_cgs(n, jj + 1, c->V, n, nullptr, c->w, true, c->partial, c->ticket, c->h1, st);
         hz::launch_cgs(n, jj + 1, c->V, n, c->h1, c->w, true, c->partial, c->ticket, c->h2, st);
         const hz::SlotGivens gv = givens_args(0, m, c->H, c->cs, c->sn, c->g, c->h1, c->h2, c->nrm, c->scal, 4, c->brk);

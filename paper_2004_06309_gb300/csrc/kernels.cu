@@ -1325,26 +1325,36 @@ void launch_spmv_real_multi(int64_t n, int S, const int64_t* rp, const int32_t* 
 // Bound by FP64 arithmetic (four FMAs per entry: 66 us for the 9.7M entries of the 349,461-dof
 // survey model), a warp taking as long as its longest row: P2 rows hold 10 to 65 entries, and in
 // natural order 15 % of the lanes' steps were idle (counted on the 54,925-dof pattern, two lanes per
-// row).  The rows are walked in an order that sorts them by length within windows of 4,096, which
-// keeps the gathers of x local: 3 % idle.  A row's start, length and number lie together in this order:
-// the number alone, and then the row's pointers, was one more load in the chain (9,261 rows, eight
-// lanes: 6.2 us in natural order, 7.6 so, 6.2 now; 349,461 rows, two lanes: 94.2, 86.2, 86.0).
-template <int TPR>
-__global__ void __launch_bounds__(256) k_spmv(int64_t n, const SpmvRow* rows, const int32_t* ci, const double2* val,
-                                              const double2* x, const double2* sub, double2* y) {
+// row).  SORTED: the rows are walked in an order that sorts them by length within windows of 4,096, which
+// keeps the gathers of x local: 3 % idle.  A row's start, length and number lie together in this
+// order: the number alone, and then the row's pointers, was one more load in the chain.  Where
+// sorting pays: spmv_rows.
+template <int TPR, bool SORTED>
+__global__ void __launch_bounds__(256) k_spmv(int64_t n, const SpmvRow* rows, const int64_t* rp, const int32_t* ci,
+                                              const double2* val, const double2* x, const double2* sub, double2* y) {
   const int lane = threadIdx.x % TPR;
   const int64_t groups = (int64_t(gridDim.x) * blockDim.x) / TPR;
   const int64_t g0 = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) / TPR;
   const int64_t wbase0 = (blockIdx.x * int64_t(blockDim.x) + (threadIdx.x & ~31)) / TPR;
   for (int64_t off = 0; wbase0 + off < n; off += groups) {
-    const bool in = g0 + off < n;
-    SpmvRow r{0, 0, 0};
-    if (in) *reinterpret_cast<int4*>(&r) = __ldg(reinterpret_cast<const int4*>(rows + g0 + off));
+    int64_t row = g0 + off;
+    const bool in = row < n;
     double2 acc = make_double2(0.0, 0.0);
-    const int64_t e = r.start + r.len;
-    for (int64_t q = r.start + lane; q < e; q += TPR) acc = cmad(val[q], x[ci[q]], acc);
+    if (in) {
+      int64_t q, e;
+      if constexpr (SORTED) {
+        const SpmvRow r = rows[row];
+        row = r.row;
+        q = r.start;
+        e = r.start + r.len;
+      } else {
+        e = rp[row + 1];
+        q = rp[row];
+      }
+      for (q += lane; q < e; q += TPR) acc = cmad(val[q], x[ci[q]], acc);
+    }
     for (int o = TPR / 2; o > 0; o >>= 1) acc = cadd(acc, shfl_xor(acc, o, TPR));
-    if (in && lane == 0) y[r.row] = sub ? csub(sub[r.row], acc) : acc;
+    if (in && lane == 0) y[row] = sub ? csub(sub[row], acc) : acc;
   }
 }
 
@@ -1375,16 +1385,22 @@ __global__ void __launch_bounds__(256) k_spmv_real(int64_t n, const int64_t* rp,
 static thread_local int g_spmv_tpr = 8;
 void set_spmv_lanes(int tpr) { g_spmv_tpr = tpr; }
 
-void launch_spmv(int64_t n, const SpmvRow* rows, const int32_t* ci, const double2* val, const double2* x,
-                 const double2* sub, double2* y, cudaStream_t st) {
-  if (n == 0) return;
-  HZ_COUNT();
+template <bool SORTED>
+static void spmv_lanes(int64_t n, const SpmvRow* rows, const int64_t* rp, const int32_t* ci, const double2* val,
+                       const double2* x, const double2* sub, double2* y, cudaStream_t st) {
   const int t = g_spmv_tpr;
   const unsigned g = grid_for(n * t, 256, 152 * 32);
-  if (t == 2) k_spmv<2><<<g, 256, 0, st>>>(n, rows, ci, val, x, sub, y);
-  else if (t == 4) k_spmv<4><<<g, 256, 0, st>>>(n, rows, ci, val, x, sub, y);
-  else if (t == 16) k_spmv<16><<<g, 256, 0, st>>>(n, rows, ci, val, x, sub, y);
-  else k_spmv<8><<<g, 256, 0, st>>>(n, rows, ci, val, x, sub, y);
+  if (t == 2) k_spmv<2, SORTED><<<g, 256, 0, st>>>(n, rows, rp, ci, val, x, sub, y);
+  else if (t == 4) k_spmv<4, SORTED><<<g, 256, 0, st>>>(n, rows, rp, ci, val, x, sub, y);
+  else if (t == 16) k_spmv<16, SORTED><<<g, 256, 0, st>>>(n, rows, rp, ci, val, x, sub, y);
+  else k_spmv<8, SORTED><<<g, 256, 0, st>>>(n, rows, rp, ci, val, x, sub, y);
+}
+void launch_spmv(int64_t n, const SpmvRow* rows, const int64_t* rp, const int32_t* ci, const double2* val,
+                 const double2* x, const double2* sub, double2* y, cudaStream_t st) {
+  if (n == 0) return;
+  HZ_COUNT();
+  if (rows) spmv_lanes<true>(n, rows, rp, ci, val, x, sub, y, st);
+  else spmv_lanes<false>(n, rows, rp, ci, val, x, sub, y, st);
 }
 
 void launch_spmv_real(int64_t n, const int64_t* rp, const int32_t* ci, const double* val, const double2* x,
